@@ -139,7 +139,8 @@ struct PolicyEgarchF32T {
     using Model = EgarchF32<K, I, kDelta>;
     static constexpr int kNs = K + 1;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;   // Table 1
-    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full)
+    static constexpr bool kExpTab = false;
+    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* = nullptr)
     {
         mdl.setup(full, m.gamma, m.eps0_zero);
     }
@@ -174,19 +175,37 @@ struct PolicyEgarchF32 : PolicyEgarchF32T<K, I, false> {};
 template <int K, int I>
 struct PolicyEgarchF32Delta : PolicyEgarchF32T<K, I, true> {};
 
+// FP64: the fixed-point recursion for whole series (PolicyEgarchF64Fx: M phase,
+// stand-alone likelihood), the FP64 recursion observation by observation
+// (PolicyEgarchF64: data-tempering C phase).
+template <int K, int I>
+struct PolicyEgarchF64Fx {
+    using Real = double;
+    using Obs = double;
+    static constexpr int kChunk = kChunkF64;
+    using Model = EgarchFxSafe<K, I>;
+    static constexpr int kNs = K + 1;
+    static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;
+    static constexpr bool kExpTab = true;
+    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* tab)
+    {
+        mdl.setup(full, m.gamma, m.eps0_zero, tab);
+    }
+    __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f64(mdl, pipe, T); }
+    __device__ static void state_out(const Model& mdl, double* st) { mdl.state_out(st); }
+};
+
 template <int K, int I>
 struct PolicyEgarchF64 {
     using Real = double;
     using Obs = double;
-    static constexpr int kChunk = kChunkF64;
     using Model = EgarchF64<K, I>;
     static constexpr int kNs = K + 1;
-    static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;
-    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full)
+    static constexpr bool kExpTab = true;
+    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* tab)
     {
-        mdl.setup(full, m.gamma, m.eps0_zero);
+        mdl.setup(full, m.gamma, m.eps0_zero, tab);
     }
-    __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f64(mdl, pipe, T); }
     __device__ static void state_out(const Model& mdl, double* st) { mdl.state_out(st); }
     __device__ static void load_state(Model& mdl, const double* st) { mdl.load_state(st); }
     __device__ static double logdens(Model& mdl, const Obs* obs, int s, int)
@@ -209,7 +228,8 @@ struct PolicyLinreg {
     using Model = LinregF64;
     static constexpr int kNs = 0;
     static constexpr int kMaxFree = 8;
-    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full)
+    static constexpr bool kExpTab = false;
+    __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t*)
     {
         mdl.setup(full, m.p, m.sigma);
     }
@@ -243,12 +263,25 @@ __device__ __forceinline__ double tempered_target(double lp, double ll, double p
 }
 
 
+// The exp2 table of the FP64 models, staged in shared memory (visible after
+// the caller's next block barrier); other models take one unused entry.
+template <class Pol>
+struct ExpTab {
+    uint64_t t[Pol::kExpTab ? 256 : 1];
+    __device__ __forceinline__ void load()
+    {
+        if constexpr (Pol::kExpTab)
+            for (int i = threadIdx.x; i < 256; i += blockDim.x) t[i] = g_exp2_neg256[i];
+    }
+};
+
 // Shared memory of one mutation tile.
 template <class Pol>
 struct MutateSmem {
     __align__(16) typename Pol::Obs obuf[2 * Pol::kChunk];
     __align__(8) uint64_t bars[2];
     typename Pol::Real Ls[kMaxD * kMaxD];
+    ExpTab<Pol> tab;
     unsigned int acc_s;
 };
 
@@ -271,6 +304,7 @@ __device__ __forceinline__ void mutate_tile(const MutateArgs& a, uint64_t iter, 
     const int d = a.m.d;
     pdl_wait();   // under a dependent launch: nothing the covariance step writes is read before this
     for (int i = threadIdx.x; i < d * d; i += blockDim.x) sm.Ls[i] = (Real)a.L[i];
+    sm.tab.load();
     if (threadIdx.x == 0) sm.acc_s = 0;
 
     const int64_t nelem = (int64_t)a.T * a.W;
@@ -315,7 +349,14 @@ __device__ __forceinline__ void mutate_tile(const MutateArgs& a, uint64_t iter, 
             lp_new = log_prior(a.m, thn);
             full_theta<Real>(a.m, thn, full);
         }
-        Pol::setup(mdl, a.m, full);
+        Pol::setup(mdl, a.m, full, sm.tab.t);
+    }
+    if constexpr (Pol::kExpTab && !kIndep) {
+        // lp* + phi l* below the current target by more than 40 is rejected by
+        // every uniform (log u > -37.5)
+        const double old = tempered_target(a.lp[pp], a.ll[pp], a.phi);
+        if (!(lp_new > -INFINITY)) mdl.reject = INFINITY;
+        else if (a.phi > 0.0 && old > -INFINITY) mdl.reject = (old - 40.0 - lp_new) / a.phi;
     }
     const bool ok = Pol::run(mdl, pipe, a.T, a.W);
     pdl_trigger();   // the covariance step that follows may launch once every block is here
@@ -350,7 +391,8 @@ __device__ __forceinline__ void mutate_tile(const MutateArgs& a, uint64_t iter, 
 }
 
 template <class Pol, bool kIndep = false>
-__global__ void __launch_bounds__(kMutBoundX1) k_mutate(MutateArgs a)
+__global__ void __launch_bounds__(Pol::kExpTab ? kMutMaxThreads : kMutBoundX1, Pol::kExpTab ? 2 : 1)
+k_mutate(MutateArgs a)
 {
     __shared__ MutateSmem<Pol> sm;
     mutate_tile<Pol, kIndep>(a, a.iter, blockIdx.x * blockDim.x, sm);
@@ -446,6 +488,8 @@ __global__ void __launch_bounds__(kMutThreads) k_loglik(LoglikArgs a)
     using Obs = typename Pol::Obs;
     __shared__ __align__(16) Obs obuf[2 * Pol::kChunk];
     __shared__ __align__(8) uint64_t bars[2];
+    __shared__ ExpTab<Pol> tab;
+    tab.load();
 
     const int64_t nelem = (int64_t)a.T * a.W;
     ObsPipe<Obs, Pol::kChunk> pipe{obuf, bars, (const Obs*)a.obs, nelem,
@@ -464,7 +508,7 @@ __global__ void __launch_bounds__(kMutThreads) k_loglik(LoglikArgs a)
     {
         Real full[kMaxD];
         full_theta<Real>(a.m, th, full);
-        Pol::setup(mdl, a.m, full);
+        Pol::setup(mdl, a.m, full, tab.t);
     }
     const bool ok = Pol::run(mdl, pipe, a.T, a.W);
     double ll = ok ? mdl.finish(a.T) : -INFINITY;
@@ -590,13 +634,18 @@ __global__ void __launch_bounds__(kMutThreads) k_cdata(CdataArgs a)
         }
         return;
     }
+    __shared__ ExpTab<Pol> tab;
+    if constexpr (Pol::kExpTab) {
+        tab.load();
+        __syncthreads();
+    }
     double th[kMaxD];
     for (int i = 0; i < a.m.d; ++i) th[i] = a.theta[i * P + pp];
     typename Pol::Model mdl;
     {
         Real full[kMaxD];
         full_theta<Real>(a.m, th, full);
-        Pol::setup(mdl, a.m, full);
+        Pol::setup(mdl, a.m, full, tab.t);
     }
     double st[kMaxState];
     for (int k = 0; k < Pol::kNs; ++k) st[k] = a.state[k * P + pp];

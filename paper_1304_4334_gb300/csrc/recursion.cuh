@@ -17,10 +17,14 @@
 // multiplied together and one lg2 is taken per 32 observations.  Sums of the
 // per-observation terms stay in FP32 for 256 observations and are then added
 // into an FP64 accumulator (the log likelihood itself is FP64).
-// FP64 path (EgarchF64): the four steps as written, in double precision.
+// FP64 path: EgarchFx (egarch_fx.cuh), the recursion in 64-bit fixed point,
+// with EgarchF64, the four steps as written in double precision, for the
+// particles that leave its ranges and for the data-tempering C phase.
 #pragma once
 
 #include "common.cuh"
+#include "egarch_fx.cuh"
+#include "exp2_table.h"
 
 namespace smc {
 
@@ -383,17 +387,21 @@ struct EgarchF32 {
 };
 
 // ------------------------------------------------------------- FP64 recursion
+// The four steps as written with the state in FP64 and any range of values;
+// the exponentials run on the integer pipes (egarch_fx.cuh), and the mixture's
+// logarithm is taken once, of the running product of the sums s_t.
 template <int K, int I>
 struct EgarchF64 {
     double mu, lsy;
     double al[K], be[K], ga[K], v0[K];
     double ainv[I], mui[I], lps[I];        // 1/sigma_i, mu_i, log p_i - log sigma_i
     double v[K], eps, acc;
+    uint64_t pm;                           // product of the s_t: pm 2^(pe - 62)
+    int pe;
+    const uint64_t* tab;                   // exp2 table (shared memory)
 
-    __device__ __forceinline__ void setup(const double* th, int has_gamma, int eps0_zero)
+    __device__ __forceinline__ void setup(const EgarchParams<double, K, I>& q, int eps0_zero, const uint64_t* tab_)
     {
-        EgarchParams<double, K, I> q;
-        egarch_transform<double, K, I>(th, has_gamma, q);
         mu = q.mu_y;
         lsy = q.log_sigma_y;
 #pragma unroll
@@ -403,18 +411,33 @@ struct EgarchF64 {
             ga[k] = q.gamma[k];
             v0[k] = eps0_zero ? -q.beta[k] * kSqrt2OverPi : 0.0;
         }
+        if constexpr (I >= 2) {
 #pragma unroll
-        for (int i = 0; i < I; ++i) {
-            ainv[i] = 1.0 / q.sig[i];
-            mui[i] = q.mu[i];
-            lps[i] = log(q.p[i]) - log(q.sig[i]);
+            for (int i = 0; i < I; ++i) {
+                ainv[i] = 1.0 / q.sig[i];
+                mui[i] = q.mu[i];
+                lps[i] = log(q.p[i]) - log(q.sig[i]);
+            }
         }
         eps = 0.0;
         acc = 0.0;
+        pm = 1ull << 62;
+        pe = 0;
+        tab = tab_;
     }
 
+    __device__ __forceinline__ void setup(const double* th, int has_gamma, int eps0_zero, const uint64_t* tab_)
+    {
+        EgarchParams<double, K, I> q;
+        egarch_transform<double, K, I>(th, has_gamma, q);
+        setup(q, eps0_zero, tab_);
+    }
+
+    // One observation: log p - log s_t, with s_t (I >= 2; units 2^-61) apart.
+    // An infinite or NaN shock makes the largest term x_i, and with it the
+    // result, infinite or NaN.
     template <bool kFirst>
-    __device__ __forceinline__ void step(double y)
+    __device__ __forceinline__ double terms(double y, uint64_t& s)
     {
         if constexpr (kFirst) {
 #pragma unroll
@@ -422,38 +445,56 @@ struct EgarchF64 {
         } else {
             const double ae = fabs(eps) - kSqrt2OverPi;
 #pragma unroll
-            for (int k = 0; k < K; ++k) v[k] = al[k] * v[k] + be[k] * ae + ga[k] * eps;
+            for (int k = 0; k < K; ++k) v[k] = fma(be[k], ae, fma(ga[k], eps, al[k] * v[k]));
         }
-        double vs = 0.0;
+        double vs = v[0];
 #pragma unroll
-        for (int k = 0; k < K; ++k) vs += v[k];
+        for (int k = 1; k < K; ++k) vs += v[k];
         const double lh = lsy + 0.5 * vs;                 // log h_t
-        eps = (y - mu) * exp(-lh);
-        double l;
+        eps = (y - mu) * fx_exp_neg(lh, tab);
         if constexpr (I == 1) {
-            l = -0.5 * eps * eps;
+            return -0.5 * eps * eps - lh;
         } else {
             double x[I];
-            double m = -INFINITY;
 #pragma unroll
             for (int i = 0; i < I; ++i) {
                 const double z = (eps - mui[i]) * ainv[i];
                 x[i] = lps[i] - 0.5 * z * z;
-                m = fmax(m, x[i]);
             }
-            double s = 0.0;
+            double m = x[0];
 #pragma unroll
-            for (int i = 0; i < I; ++i) s += exp(x[i] - m);
-            l = m + log(s);
+            for (int i = 1; i < I; ++i) {   // m ends as the largest, x[1..] as the others
+                const double lo = x[i] > m ? m : x[i];
+                m = x[i] > m ? x[i] : m;
+                x[i] = lo;
+            }
+            s = 1ull << 61;
+#pragma unroll
+            for (int i = 1; i < I; ++i) s += fx_exp_q61(m - x[i], tab);
+            return m - lh;
         }
-        acc += l - lh;
     }
 
-    __device__ __forceinline__ void flush() {}
+    template <bool kFirst>
+    __device__ __forceinline__ void step(double y)
+    {
+        uint64_t s;
+        acc += terms<kFirst>(y, s);
+        if constexpr (I >= 2) fx_product(pm, pe, s);
+    }
+
+    __device__ __forceinline__ void restart()   // of the sums, not the state
+    {
+        acc = 0.0;
+        pm = 1ull << 62;
+        pe = 0;
+    }
 
     __device__ __forceinline__ double finish(int T) const
     {
-        return acc + (double)T * (-0.5 * kLog2Pi);
+        double l = acc + (double)T * (-0.5 * kLog2Pi);
+        if constexpr (I >= 2) l += kLn2 * ((double)pe + log2((double)pm * 0x1p-62));
+        return l;
     }
 
     __device__ __forceinline__ void load_state(const double* st)
@@ -466,11 +507,10 @@ struct EgarchF64 {
     template <bool kFirst>
     __device__ __forceinline__ double logdens(double y)
     {
-        const double before = acc;
-        step<kFirst>(y);
-        const double l = acc - before;
-        acc = before;
-        return l - 0.5 * kLog2Pi;
+        uint64_t s;
+        double l = terms<kFirst>(y, s) - 0.5 * kLog2Pi;
+        if constexpr (I >= 2) l += log((double)s * 0x1p-61);
+        return l;
     }
 
     __device__ __forceinline__ void state_out(double* st) const
@@ -478,6 +518,121 @@ struct EgarchF64 {
 #pragma unroll
         for (int k = 0; k < K; ++k) st[k] = v[k];
         st[K] = eps;
+    }
+};
+
+// EgarchFx with the FP64 recursion behind it: the model of the FP64 M phase
+// and likelihood.  The series runs in blocks of 32 observations; a particle
+// that leaves the fixed-point ranges within a block repeats it in EgarchF64
+// and returns to fixed point at the first block end whose state is in range
+// (a single outlying observation costs one block, not the rest of the
+// series).
+template <int K, int I>
+struct EgarchFxSafe {
+    EgarchFx<K, I> fx;
+    typename EgarchFx<K, I>::Saved saved;  // at the last block end in fixed point
+    EgarchParams<double, K, I> q;
+    EgarchF64<K, I> m;                     // set up when first needed
+    const uint64_t* tab;
+    int eps0_zero;
+    // A log likelihood below this needs no value (-inf is returned for it): a
+    // Metropolis proposal that is rejected whatever the uniform.
+    double reject;
+    int n64;                               // observations taken in FP64
+    double acc64, lmax;                    // their log densities; bound of one (see below)
+    bool fixed, out, ready, dead;          // parameters in range; state out of range; m set up; below reject
+
+    __device__ __forceinline__ void setup(const double* th, int has_gamma, int e0z, const uint64_t* tab_)
+    {
+        egarch_transform<double, K, I>(th, has_gamma, q);
+        tab = tab_;
+        eps0_zero = e0z;
+        reject = -INFINITY;
+        fx.setup(q.mu_y, q.log_sigma_y, q.alpha, q.beta, q.gamma, q.p, q.mu, q.sig, e0z, kLog2e);
+        fixed = fx.bad == 0u;
+        out = !fixed;
+        ready = dead = false;
+        n64 = 0;
+        acc64 = 0.0;
+        fx.save(saved);
+    }
+
+    // Block end after n observations from t0 (0-based; y: their values):
+    // closes the block in whichever recursion holds it.  f is the caller's
+    // copy of fx: it stays in registers, and only a particle out of range
+    // passes through memory.
+    __device__ __forceinline__ void close(EgarchFx<K, I>& f, const double* y, int t0, int n, int T)
+    {
+        if (f.bad == 0u && !out) {
+            f.save(saved);
+        } else if (!dead) {
+            block_f64(y, t0, n, T);
+            f.restore(fx);
+        }
+    }
+
+    // With alpha_k in [0, 1) and |gamma_k| <= beta_k no factor falls below
+    // -beta_k c / (1 - alpha_k) (c = (2/pi)^1/2), so a log density stays below
+    // lmax; once the sum so far and lmax for the rest leave the total below
+    // `reject`, nothing more is computed (a recursion that explodes, as most
+    // that come here do, ends so within a block).
+    __device__ __noinline__ void block_f64(const double* y, int t0, int n, int T)
+    {
+        if (!ready) {
+            ready = true;
+            m.setup(q, eps0_zero, tab);
+            bool bounded = true;
+            double pk = 0.0;
+            lmax = -q.log_sigma_y;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                bounded = bounded && q.alpha[k] >= 0.0 && q.alpha[k] < 1.0 && fabs(q.gamma[k]) <= q.beta[k];
+                lmax += 0.5 * kSqrt2OverPi * q.beta[k] / (1.0 - q.alpha[k]);
+            }
+#pragma unroll
+            for (int i = 0; i < I; ++i) pk += q.p[i] / q.sig[i];
+            lmax += I > 1 ? log(pk) : 0.0;
+            // (rounding included; + 1/2 log 2pi left out)
+            lmax = bounded ? fmax(lmax, 0.0) * (1.0 + 1e-6) + 0.1 : INFINITY;
+        }
+        EgarchF64<K, I> w = m;   // (in registers)
+        if (!out) {
+            fx.restore(saved);
+            double st[K + 1];
+            fx.state_out(st, kLn2);
+            w.load_state(st);
+        }
+        w.restart();
+        int r = 0;
+        if (t0 == 0) {
+            w.template step<true>(y[0]);
+            r = 1;
+        }
+        for (; r < n; ++r) w.template step<false>(y[r]);
+        acc64 += w.finish(n);
+        n64 += n;
+        if (fixed) out = !fx.enter(w.v, w.eps);
+        m = w;
+        if (!out) {
+            fx.save(saved);
+        } else if (reject > -INFINITY) {
+            const double sum = acc64 + (fixed ? fx.finish(t0 + n - n64, kLn2, kLog2Pi) : 0.0);
+            // (a sum that is -inf or NaN gives -inf in the end)
+            dead = !(sum > -INFINITY) || sum + (double)(T - t0 - n) * lmax + fabs(sum) * 1e-6 + 1.0 < reject;
+        }
+    }
+
+    __device__ __forceinline__ double finish(int T) const
+    {
+        if (dead) return -INFINITY;
+        if (n64 == 0) return fx.finish(T, kLn2, kLog2Pi);
+        return acc64 + (fixed ? fx.finish(T - n64, kLn2, kLog2Pi) : 0.0);
+    }
+
+    __device__ __forceinline__ void state_out(double* st) const
+    {
+        if (out) m.state_out(st);
+        else fx.state_out(st, kLn2);
     }
 };
 
@@ -852,9 +1007,10 @@ __device__ __forceinline__ bool run_egarch_f32_x2(EgarchF32<K, I>& ma, EgarchF32
 }
 
 template <int K, int I>
-__device__ __forceinline__ bool run_egarch_f64(EgarchF64<K, I>& mdl, ObsPipe<double, kChunkF64>& pipe,
+__device__ __forceinline__ bool run_egarch_f64(EgarchFxSafe<K, I>& mdl, ObsPipe<double, kChunkF64>& pipe,
                                                int T)
 {
+    EgarchFx<K, I> fx = mdl.fx;
     for (int c = 0; c < pipe.nchunks; ++c) {
         if (!pipe.wait(c)) {
             pipe.drain(c);
@@ -862,14 +1018,26 @@ __device__ __forceinline__ bool run_egarch_f64(EgarchF64<K, I>& mdl, ObsPipe<dou
         }
         const double* yb = pipe.buf + (c & 1) * kChunkF64;
         const int cnt = min(kChunkF64, T - c * kChunkF64);
-        int r = 0;
-        if (c == 0 && cnt > 0) {
-            mdl.template step<true>(yb[0]);
-            r = 1;
+        for (int r0 = 0; r0 < cnt; r0 += 32) {
+            // 32 observations; the mixture part of one runs beside the chain
+            // of the next (they do not depend on each other)
+            const int e = min(cnt, r0 + 32);
+            if (c == 0 && r0 == 0) fx.template chain<true>(yb[0], mdl.tab);
+            else fx.template chain<false>(yb[r0], mdl.tab);
+            for (int r = r0 + 1; r < e; ++r) {
+                const uint64_t E = fx.E;
+                const int32_t neg = fx.neg;
+                fx.template chain<false>(yb[r], mdl.tab);
+                fx.mix(E, neg, mdl.tab);
+                if ((r & 7) == 7) fx.flush();
+            }
+            fx.mix(fx.E, fx.neg, mdl.tab);
+            fx.flush();
+            mdl.close(fx, yb + r0, c * kChunkF64 + r0, e - r0, T);
         }
-        for (; r < cnt; ++r) mdl.template step<false>(yb[r]);
         pipe.release(c);
     }
+    if (!mdl.out) mdl.fx.restore(mdl.saved);
     return true;
 }
 

@@ -1,0 +1,82 @@
+"""FP64 kernels around the edges of the fixed-point recursion: block and chunk
+ends, particles that leave its ranges for a block or for good, and proposals
+whose likelihood is not carried to the end because they are rejected whatever
+it is.  Against the FP64 oracle at the FP64 contract's 1e-9 relative."""
+import numpy as np
+import pytest
+
+import oracle as O
+from tests.gpu_util import dev, egarch_truth, host, particles, soa, torch_cuda
+from paper_1304_4334_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def S():
+    torch_cuda()
+    from paper_1304_4334_gb300 import smc
+    return smc
+
+
+def _series(truth, T):
+    y = I.simulate_egarch(truth, T, seed=71)
+    y[min(T - 1, 30)] += 3.0       # 300 standard deviations: out of range for one block
+    return y
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (2, 2), (3, 4), (4, 3)])
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 511, 512, 513, 1025])
+@pytest.mark.parametrize("outlier", [False, True])
+def test_loglik_block_edges_and_range_exits(S, K, I_, T, outlier):
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = _series(truth, T) if outlier else I.simulate_egarch(truth, T, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    P = 70
+    th = particles(spec.d, truth, K, I_, True, P, 73, prior=O.table1_prior(K, I_, True), frac_prior=0.3)
+    ll_o, st_o = O.loglik(spec, y, th, with_state=True, nthreads=4)
+    ll = torch.empty(P, dtype=torch.float64, device="cuda")
+    st = torch.empty((K + 1, P), dtype=torch.float64, device="cuda")
+    S.loglik(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(th), ll, None, st)
+    ll, st = host(ll), host(st).T
+    sane = ll_o > -1e7
+    cloud = np.arange(P) >= int(P * 0.3)
+    assert cloud[sane].sum() > P // 2
+    np.testing.assert_allclose(ll[sane], ll_o[sane], rtol=1e-9)
+    # (the oracle forms h_t itself, whose overflow makes its value -inf where log
+    # h_t is still finite: those are not compared)
+    assert np.all(ll[np.isfinite(ll_o) & ~sane] < -1e6)
+    np.testing.assert_allclose(st[sane & cloud], st_o[sane & cloud], rtol=1e-9, atol=1e-12)
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (2, 3)])
+@pytest.mark.parametrize("phi", [0.0, 1e-4, 0.02, 1.0])
+def test_mutation_with_out_of_range_proposals(S, K, I_, phi):
+    """Prior draws moved with a wide proposal: many recursions explode.  The
+    decision, theta, l, log prior and state equal the oracle's."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    T, P = 333, 300
+    y = I.simulate_egarch(truth, T, seed=75)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    th = particles(spec.d, truth, K, I_, True, P, 77, prior=O.table1_prior(K, I_, True), frac_prior=0.5)
+    ll, st = O.loglik(spec, y, th, with_state=True, nthreads=4)
+    keep = ll > -1e7
+    th, ll, st = th[keep], ll[keep], st[keep]
+    P = len(th)
+    lp = O.logprior(spec, th)
+    L = np.diag(np.full(spec.d, 0.4))
+    th_o, ll_o, lp_o, st_o, acc_o, n_o = O.mutate_rw(spec, y, th.copy(), ll.copy(), lp.copy(), st.copy(), L, phi, 9, 2, 3)
+    g = [soa(th), dev(ll), dev(lp), soa(st)]
+    n = S.mutate_rw(S.model_egarch(K, I_, True), S.FP64, dev(y), *g, dev(L), phi, 9, 2, 3)
+    th_g, ll_g, lp_g, st_g = host(g[0]).T, host(g[1]), host(g[2]), host(g[3]).T
+    acc_g = np.any(th_g != th, axis=1)
+    acc_o = np.any(th_o != th, axis=1)
+    assert n == n_o and np.array_equal(acc_g, acc_o), (n, n_o)
+    assert 0 < acc_o.sum() < P
+    sane = ll_o > -1e7
+    np.testing.assert_allclose(ll_g[sane], ll_o[sane], rtol=1e-9)
+    np.testing.assert_allclose(th_g, th_o, rtol=1e-12, atol=1e-12)
+    np.testing.assert_allclose(lp_g, lp_o, rtol=1e-12)
+    assert np.all(ll_g[np.isfinite(ll_o) & ~sane] < -1e6)
