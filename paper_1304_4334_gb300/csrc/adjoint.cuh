@@ -33,15 +33,8 @@ namespace smc {
 template <typename Real>
 __device__ __forceinline__ Real nexp(Real x)
 {
-    if constexpr (sizeof(Real) == 4) return ex2_approx(x * (float)kLog2e);
-    else return exp(x);
-}
-
-template <typename Real>
-__device__ __forceinline__ Real nlog(Real x)
-{
-    if constexpr (sizeof(Real) == 4) return lg2_approx(x) * (float)kLn2;
-    else return log(x);
+    static_assert(sizeof(Real) == 4, "the FP64 path is adjoint_f64.cuh");
+    return ex2_approx(x * (float)kLog2e);
 }
 
 template <typename Real>
@@ -148,56 +141,21 @@ struct EgarchNat {
         inv = nexp<Real>(-(lsy + Real(0.5) * vs));
         eps = (y - mu) * inv;
     }
-
-    // One observation: updates (v, eps), returns l_t + (1/2) log 2pi and exp(-s_t).
-    template <bool kFirst>
-    __device__ __forceinline__ Real step(Real y, Real& inv)
-    {
-        if constexpr (kFirst) {
-#pragma unroll
-            for (int k = 0; k < K; ++k) v[k] = v0[k];
-        } else {
-            const Real ae = fabs(eps) - (Real)kSqrt2OverPi;
-#pragma unroll
-            for (int k = 0; k < K; ++k) v[k] = al[k] * v[k] + be[k] * ae + ga[k] * eps;
-        }
-        Real vs = v[0];
-#pragma unroll
-        for (int k = 1; k < K; ++k) vs += v[k];
-        const Real s = lsy + Real(0.5) * vs;
-        inv = nexp<Real>(-s);
-        eps = (y - mu) * inv;
-        if constexpr (I == 1) {
-            return -s - Real(0.5) * eps * eps;
-        } else {
-            Real x[I], m = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < I; ++i) {
-                const Real z = (eps - mi[i]) * a[i];
-                x[i] = lpa[i] - Real(0.5) * z * z;
-                m = fmax(m, x[i]);
-            }
-            Real sum = 0;
-#pragma unroll
-            for (int i = 0; i < I; ++i) sum += nexp<Real>(x[i] - m);
-            return -s + m + nlog<Real>(sum);
-        }
-    }
 };
 
 // Gradient of the natural parameters -> gradient with respect to the full
 // theta vector (Table 1 layout).
 template <typename Real, int K, int I>
-__device__ void natural_to_theta(const EgarchNat<Real, K, I>& m, const double* gn, const Real* th,
-                                 int has_gamma, double* gth)
+__device__ void natural_to_theta(const Real* al, const Real* be, const double* gn, const Real* th, int has_gamma,
+                                 double* gth)
 {
     int j = 0;
     gth[j++] = gn[0] / 1000.0;
     gth[j++] = gn[1];
 #pragma unroll
-    for (int k = 0; k < K; ++k) gth[j++] = gn[2 + k] * (1.0 - (double)m.al[k] * (double)m.al[k]);
+    for (int k = 0; k < K; ++k) gth[j++] = gn[2 + k] * (1.0 - (double)al[k] * (double)al[k]);
 #pragma unroll
-    for (int k = 0; k < K; ++k) gth[j++] = gn[2 + K + k] * (double)m.be[k];
+    for (int k = 0; k < K; ++k) gth[j++] = gn[2 + K + k] * (double)be[k];
     if (has_gamma) {
 #pragma unroll
         for (int k = 0; k < K; ++k) gth[j++] = gn[2 + 2 * K + k];
@@ -217,40 +175,10 @@ __device__ void natural_to_theta(const EgarchNat<Real, K, I>& m, const double* g
     }
 }
 
-// Forward pass from t = 1 to T with checkpoints every kSeg observations:
+// FP32 forward pass through the base-2 recursion of the random-walk kernel
+// (EgarchF32) with natural-unit checkpoints every kSeg observations:
 // ckpt[seg][k][P] holds (v_1..v_K, eps) after observation seg*kSeg (1-based)
 // is processed, for seg = 0.. (the state entering segment seg + 1).
-// Returns l(theta); leaves the end state in m.
-template <typename Real, int K, int I, int kSeg>
-__device__ double adj_forward(EgarchNat<Real, K, I>& m, const Real* __restrict__ y, int T, Real* ckpt,
-                              size_t P, int p, bool write)
-{
-    double acc = 0.0;
-    Real part = 0;
-    const int nseg = (T + kSeg - 1) / kSeg;
-    for (int sg = 0; sg < nseg; ++sg) {
-        const int t0 = sg * kSeg, n = min(kSeg, T - t0);
-        if (write && sg > 0) {
-            Real* c = ckpt + (size_t)(sg - 1) * (K + 1) * P + p;
-#pragma unroll
-            for (int k = 0; k < K; ++k) c[k * P] = m.v[k];
-            c[K * P] = m.eps;
-        }
-        for (int r = 0; r < n; ++r) {
-            Real inv;
-            const Real yy = y[t0 + r];
-            part += (t0 + r == 0) ? m.template step<true>(yy, inv) : m.template step<false>(yy, inv);
-        }
-        if ((sg & 7) == 7 || sg == nseg - 1) {
-            acc += (double)part;
-            part = 0;
-        }
-    }
-    return acc + (double)T * (-0.5 * kLog2Pi);
-}
-
-// FP32 forward pass through the base-2 recursion of the random-walk kernel
-// (EgarchF32), writing the same natural-unit checkpoints as adj_forward.
 template <int K, int I, int kSeg>
 __device__ double adj_forward_fast(const float* th, int has_gamma, int eps0_zero, const float* __restrict__ y,
                                    int T, float* ckpt, size_t P, int p)
@@ -287,7 +215,7 @@ __device__ double adj_forward_fast(const float* th, int has_gamma, int eps0_zero
     return f.finish(T);
 }
 
-// Reverse sweep over all segments; gn (double, kNp) receives d l / d natural
+// FP32 reverse sweep over all segments; gn (double, kNp) receives d l / d natural
 // parameters.  buf is this thread's shared-memory slab laid out
 // [kSeg][K + 2][stride] (v_k, eps, exp(-s)) with element (t, f) at
 // buf[(t * (K + 2) + f) * stride].
@@ -340,8 +268,7 @@ __device__ void adj_reverse(EgarchNat<Real, K, I> m, const Real* __restrict__ y,
                 sum += x[i];
             }
             Real isum;
-            if constexpr (sizeof(Real) == 4) isum = __fdividef(1.0f, sum);   // sum in [1, I]
-            else isum = Real(1) / sum;
+            isum = __fdividef(1.0f, sum);   // sum in [1, I]
             dle = 0;
 #pragma unroll
             for (int i = 0; i < I; ++i) {

@@ -163,6 +163,40 @@ __device__ __noinline__ inline double fx_exp_library(double x) { return exp(x); 
 inline double fx_exp_library(double x) { return std::exp(x); }
 #endif
 
+// M 2^(-63 - n) for M in (2^62, 2^63] as FP64 (normal range).
+SMC_FX double fx_pack(uint64_t M, int n)
+{
+    const uint64_t r = ((M + 512ull) >> 10) + ((uint64_t)(uint32_t)(1021 - n) << 52);
+#if defined(__CUDA_ARCH__)
+    return __longlong_as_double((long long)r);
+#else
+    double d;
+    std::memcpy(&d, &r, 8);
+    return d;
+#endif
+}
+
+// 2^123 / s for s in [2^61, 2^63], within a few units of 2^-59 relative.
+SMC_FX uint64_t fx_rcp(uint64_t s)
+{
+    const uint32_t sh = (uint32_t)(s >> 32);
+#if defined(__CUDA_ARCH__)
+    const float y = __frcp_rn(__uint2float_rn(sh));
+    const uint32_t yb = __float_as_uint(y);
+#else
+    const float y = 1.0f / (float)sh;
+    uint32_t yb;
+    std::memcpy(&yb, &y, 4);
+#endif
+    // y 2^91 = mantissa 2^(exponent - 127 - 23 + 91)
+    uint64_t Y = (uint64_t)((yb & 0x7fffffu) | 0x800000u) << (((yb >> 23) - 59u) & 63u);
+    int64_t e = (int64_t)((1ull << 59) - fx_mulhi(s, Y));                       // relative error 2^-59
+    Y += (uint64_t)(((int64_t)(int32_t)(uint32_t)(Y >> 32) * (int32_t)(e >> 8)) >> 19);
+    e = (int64_t)((1ull << 59) - fx_mulhi(s, Y));
+    Y += (uint64_t)(((int64_t)(int32_t)(uint32_t)(Y >> 32) * (int32_t)e) >> 27);
+    return Y;
+}
+
 // e^-x in FP64 without FP64 instructions for |x| < 128 (within a unit in the
 // last place); the library's exponential beyond.
 SMC_FX double fx_exp_neg(double x, const uint64_t* tab)
@@ -176,16 +210,7 @@ SMC_FX double fx_exp_neg(double x, const uint64_t* tab)
     X = fx_mulhi(X, kFxLog2e);
     const uint64_t sg = (uint64_t)((int64_t)fx_bits(x) >> 63);
     X = (X ^ sg) - sg;
-    const uint64_t M = fx_exp2neg(X, tab);           // e^-x = M 2^(-63 - n)
-    const int n = (int)((int64_t)X >> 55);
-    const uint64_t r = ((M + 512ull) >> 10) + ((uint64_t)(uint32_t)(1021 - n) << 52);
-#if defined(__CUDA_ARCH__)
-    return __longlong_as_double((long long)r);
-#else
-    double d;
-    std::memcpy(&d, &r, 8);
-    return d;
-#endif
+    return fx_pack(fx_exp2neg(X, tab), (int)((int64_t)X >> 55));
 }
 
 // Product of the mixture sums s (units 2^-61, in [1, 4]): pm 2^(pe - 62) with
@@ -231,6 +256,8 @@ struct EgarchFx {
     __int128 s1w;
     int pe;                              // product: pm 2^(pe - 62)
     double c0, m0, a0;                   // component 0: log2(p / sigma), mu, 1 / sigma
+    int ref;                             // its place in the caller's order
+    uint64_t M, X;                       // 1 / h_t = M 2^(-63 - n), n = (X >> 55) - 256
     uint32_t bad;
 
     // Natural parameters (EgarchParams) in; eps0_zero as in EgarchF64.
@@ -284,25 +311,26 @@ struct EgarchFx {
         }
         c0 = m0 = 0.0;
         a0 = 1.0;
+        ref = 0;
         if (I > 1) {
-            // component 0: the one with the largest sigma
-            double ps[I], ms[I], sg[I];
-#pragma unroll
-            for (int i = 0; i < I; ++i) {
-                ps[i] = p[i];
-                ms[i] = mum[i];
-                sg[i] = sig[i];
-            }
+            // component 0: the one with the largest sigma (changes place with ref)
+            double ps[I], ms[I], sg[I], top = sig[0];
 #pragma unroll
             for (int i = 1; i < I; ++i) {
-                const bool sw = sg[i] > sg[0];
-                const double tp = ps[0], tm = ms[0], ts = sg[0];
-                ps[0] = sw ? ps[i] : tp;
-                ms[0] = sw ? ms[i] : tm;
-                sg[0] = sw ? sg[i] : ts;
-                ps[i] = sw ? tp : ps[i];
-                ms[i] = sw ? tm : ms[i];
-                sg[i] = sw ? ts : sg[i];
+                ref = sig[i] > top ? i : ref;
+                top = sig[i] > top ? sig[i] : top;
+            }
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                const bool sw = i > 0 && i == ref;
+                ps[i] = sw ? p[0] : p[i];
+                ms[i] = sw ? mum[0] : mum[i];
+                sg[i] = sw ? sig[0] : sig[i];
+                if (sw) {
+                    ps[0] = p[i];
+                    ms[0] = mum[i];
+                    sg[0] = sig[i];
+                }
             }
             a0 = 1.0 / sg[0];
             m0 = ms[0];
@@ -357,7 +385,7 @@ struct EgarchFx {
         } else {
             update_volatility();
         }
-        uint64_t X = ly;                 // log2 h_t + 256
+        X = ly;                          // log2 h_t + 256
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             X += (uint64_t)V[k];
@@ -365,7 +393,7 @@ struct EgarchFx {
             bad |= ((uint32_t)((uint64_t)V[k] >> 32) + (kVmax << 23)) & ~(uint32_t)((kVmax << 24) - 1);
         }
         sx += X;
-        const uint64_t M = fx_exp2neg(X, tab);
+        M = fx_exp2neg(X, tab);
         // |eps| = |y - mu| 2^-X: the 53-bit significand times M, shifted; the
         // shift passes 63 for a zero return
         const double dy = y - mu;
@@ -383,6 +411,68 @@ struct EgarchFx {
         ll += (uint64_t)(l >> 4) * (l >> 4);
     }
 
+    // d_i = x_i - x_0 (log2 units, 2^-55) for the shock ed (units 2^-53), -128
+    // where it is below that (nothing to the sum).  over: bit 31 set for
+    // d_i >= 2^(9 - lim).
+    SMC_FX int64_t term(int i, double ed, int lim, uint32_t& over) const
+    {
+        const double d = fma(fma(A[i], ed, B[i]), ed, C[i]);
+        const uint64_t db = fx_bits(d);   // |d| = significand 2^(e - 1023 - 63), shifted
+        const int ds = 1086 - ((int)(uint32_t)(db >> 52) & 0x7ff);
+        const int32_t nm = (int32_t)(uint32_t)(db >> 32) >> 31;
+        uint64_t mag = fx_shr((db << 11) | 0x8000000000000000ull, ds);
+        if (ds < 2) mag = 1ull << 62;
+        over = (uint32_t)((ds - lim) & ~nm) & 0x80000000u;
+        const uint64_t nm64 = (uint64_t)(int64_t)nm;
+        return (int64_t)((mag ^ nm64) - nm64);
+    }
+
+    // Posterior weights r_i of the components (order of setup's arguments;
+    // units 2^-59) for the shock eps; false where a d_i is out of range.
+    // 1 / s by two Newton steps on integers from the FP32 reciprocal.
+    SMC_FX bool weights(double eps, uint64_t* r, const uint64_t* tab) const
+    {
+        const double ed = eps * 0x1p53;
+        int64_t D[I], cur = 0;
+        uint32_t over = 0;
+        D[0] = 0;
+#pragma unroll
+        for (int i = 1; i < I; ++i) {
+            uint32_t o;
+            D[i] = term(i - 1, ed, 2, o);
+            over |= o;
+            cur = D[i] > cur ? D[i] : cur;
+        }
+        uint64_t w[I], s = 0;
+        if (I == 2) {   // one of the two is 1
+            const uint64_t Y = (uint64_t)(2 * cur - D[1]);
+            const uint64_t e = fx_shr(fx_exp2neg(Y, tab), (int)(uint32_t)(Y >> 55) + 2);
+            w[0] = cur > 0 ? e : 1ull << 61;
+            w[1] = cur > 0 ? 1ull << 61 : e;
+            s = w[0] + w[1];
+        } else {
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                const uint64_t Y = (uint64_t)(cur - D[i]);
+                w[i] = fx_shr(fx_exp2neg(Y, tab), (int)(uint32_t)(Y >> 55) + 2);
+                s += w[i];
+            }
+        }
+        const uint64_t Y = fx_rcp(s);
+#pragma unroll
+        for (int i = 0; i < I; ++i) r[i] = fx_mulhi(w[i], Y);
+#pragma unroll
+        for (int i = 1; i < I; ++i) {
+            const uint64_t r0 = r[0], ri = r[i];
+            r[0] = i == ref ? ri : r0;
+            r[i] = i == ref ? r0 : ri;
+        }
+        return over == 0u;
+    }
+
+    // 1 / h_t of the last chain().
+    SMC_FX double inv_h() const { return fx_pack(M, (int)(uint32_t)(X >> 55) - 256); }
+
     // The mixture part for the shock (E_, neg_): independent of the next
     // observation's chain.
     SMC_FX void mix(uint64_t E_, int32_t neg_, const uint64_t* tab)
@@ -396,19 +486,9 @@ struct EgarchFx {
         int64_t cur = 0;
 #pragma unroll
         for (int i = 0; i < kM; ++i) {
-            const double d = fma(fma(A[i], ed_, B[i]), ed_, C[i]);
-            // to fixed point: |d| = significand 2^(e - 1023 - 63), shifted;
-            // -128 or less counts as -128 (nothing to the sum), 16 or
-            // more is out of range
-            const uint64_t db = fx_bits(d);
-            const int e = (int)(uint32_t)(db >> 52) & 0x7ff;
-            const int ds = 1086 - e;
-            const int32_t nm = (int32_t)(uint32_t)(db >> 32) >> 31;
-            uint64_t mag = fx_shr((db << 11) | 0x8000000000000000ull, ds);
-            if (ds < 2) mag = 1ull << 62;
-            bad |= (uint32_t)((ds - 5) & ~nm) & 0x80000000u;
-            const uint64_t nm64 = (uint64_t)(int64_t)nm;
-            const int64_t x = (int64_t)((mag ^ nm64) - nm64);
+            uint32_t over;
+            const int64_t x = term(i, ed_, 5, over);   // 16 or more is out of range
+            bad |= over;
             // (cur, D_i) <- (max, min): the terms stay the same set, and cur
             // ends as the largest
             D[i] = x < cur ? x : cur;

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "adjoint.cuh"
+#include "adjoint_f64.cuh"
 #include "kernels.cuh"
 
 namespace smc {
@@ -67,17 +68,20 @@ struct GradEgarch {
         const int nseg = (T + kSeg - 1) / kSeg;
         return (size_t)(nseg > 1 ? nseg - 1 : 1) * (K + 1) * (size_t)P * sizeof(Real);
     }
+    static constexpr bool kExpTab = sizeof(Real) == 8;
+    // tab: the exp2 table in shared memory (FP64)
     __device__ static double eval(const ModelDev& m, const double* th, const void* obs, int T, int,
                                   void* ckpt, size_t P, int p, Real* buf, int stride, double* g,
-                                  double* st)
+                                  double* st, const uint64_t* tab = nullptr)
     {
         Real full[kMaxD];
         full_theta<Real>(m, th, full);
-        EgarchNat<Real, K, I> mdl;
-        mdl.setup(full, m.gamma, m.eps0_zero);
         const Real* y = (const Real*)obs;
         double ll;
+        double gn[EgarchNat<Real, K, I>::kNp], gfull[kMaxD];
         if constexpr (sizeof(Real) == 4) {
+            EgarchNat<Real, K, I> mdl;
+            mdl.setup(full, m.gamma, m.eps0_zero);
             ll = adj_forward_fast<K, I, kSeg>(full, m.gamma, m.eps0_zero, y, T, (Real*)ckpt, P, p);
             // end state: recompute the last segment's tail from its checkpoint
             const int nseg = (T + kSeg - 1) / kSeg;
@@ -92,16 +96,18 @@ struct GradEgarch {
                 if (t == 0) mdl.template step_state<true>(y[0], inv);
                 else mdl.template step_state<false>(y[t], inv);
             }
-        } else {
-            ll = adj_forward<Real, K, I, kSeg>(mdl, y, T, (Real*)ckpt, P, p, true);
-        }
 #pragma unroll
-        for (int k = 0; k < K; ++k) st[k] = (double)mdl.v[k];
-        st[K] = (double)mdl.eps;
-        double gn[EgarchNat<Real, K, I>::kNp];
-        adj_reverse<Real, K, I, kSeg>(mdl, y, T, (const Real*)ckpt, P, p, buf, stride, gn);
-        double gfull[kMaxD];
-        natural_to_theta<Real, K, I>(mdl, gn, full, m.gamma, gfull);
+            for (int k = 0; k < K; ++k) st[k] = (double)mdl.v[k];
+            st[K] = (double)mdl.eps;
+            adj_reverse<Real, K, I, kSeg>(mdl, y, T, (const Real*)ckpt, P, p, buf, stride, gn);
+            natural_to_theta<Real, K, I>(mdl.al, mdl.be, gn, full, m.gamma, gfull);
+        } else {
+            AdjointF64<K, I, kSeg> adj;
+            adj.setup(full, m.gamma, m.eps0_zero, tab);
+            ll = adj.forward(y, T, (double*)ckpt, P, p, st);
+            adj.reverse(y, T, (const double*)ckpt, P, p, buf, stride, gn);
+            natural_to_theta<Real, K, I>(adj.mdl.q.alpha, adj.mdl.q.beta, gn, full, m.gamma, gfull);
+        }
         if (m.has_free)
             for (int k = 0; k < m.d; ++k) g[k] = gfull[m.free_idx[k]];
         else
@@ -115,11 +121,12 @@ struct GradEgarch {
 // dl/db = sum_t (y_t - x_t'b) x_t / sigma^2.
 struct GradLinreg {
     using RealT = double;
+    static constexpr bool kExpTab = false;
     static constexpr int kNs = 0;
     static size_t smem_bytes(int) { return 0; }
     static size_t ckpt_bytes(int, int) { return 8; }
     __device__ static double eval(const ModelDev& m, const double* th, const void* obs, int T, int W,
-                                  void*, size_t, int, double*, int, double* g, double*)
+                                  void*, size_t, int, double*, int, double* g, double*, const uint64_t* = nullptr)
     {
         const double* rec = (const double*)obs;
         const double is2 = 1.0 / (m.sigma * m.sigma);
@@ -151,13 +158,18 @@ __global__ void __launch_bounds__(kMalaThreads) k_loglik_grad(GradArgs a)
 {
     using Real = typename GP::RealT;
     extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ ExpTab<GP> tab;
+    if constexpr (GP::kExpTab) {
+        tab.load();
+        __syncthreads();
+    }
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= a.P) return;
     const size_t P = (size_t)a.P;
     Real* buf = reinterpret_cast<Real*>(sm_raw) + threadIdx.x;
     double th[kMaxD], g[kMaxD], st[kMaxState];
     for (int i = 0; i < a.m.d; ++i) th[i] = a.theta[i * P + p];
-    const double ll = GP::eval(a.m, th, a.obs, a.T, a.W, a.ckpt, P, p, buf, blockDim.x, g, st);
+    const double ll = GP::eval(a.m, th, a.obs, a.T, a.W, a.ckpt, P, p, buf, blockDim.x, g, st, tab.t);
     a.ll[p] = ll;
     for (int i = 0; i < a.m.d; ++i) a.grad[i * P + p] = g[i];
     if (a.state)
@@ -172,7 +184,8 @@ __global__ void __launch_bounds__(kMalaThreads) k_loglik_grad(GradArgs a)
 // memory); buf/stride: this thread's segment slab.  Returns the decision.
 template <class GP>
 __device__ __forceinline__ bool mala_particle(const MalaArgs& a, uint64_t iter, int p,
-                                              const typename GP::RealT* Ls, typename GP::RealT* buf, int stride)
+                                              const typename GP::RealT* Ls, typename GP::RealT* buf, int stride,
+                                              const uint64_t* tab = nullptr)
 {
     using Real = typename GP::RealT;
     const int d = a.m.d;
@@ -202,7 +215,7 @@ __device__ __forceinline__ bool mala_particle(const MalaArgs& a, uint64_t iter, 
     }
     const double lp_new = log_prior(a.m, prop);
     double gl[kMaxD], st[kMaxState];
-    const double ll_new = GP::eval(a.m, prop, a.obs, a.T, a.W, a.ckpt, P, p, buf, stride, gl, st);
+    const double ll_new = GP::eval(a.m, prop, a.obs, a.T, a.W, a.ckpt, P, p, buf, stride, gl, st, tab);
     double log_alpha = -INFINITY;
     if (lp_new > -INFINITY && ll_new > -INFINITY) {
         double g2[kMaxD];
@@ -247,15 +260,17 @@ __global__ void __launch_bounds__(kMalaThreads) k_mutate_mala(MalaArgs a)
     using Real = typename GP::RealT;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     __shared__ Real Ls[kMaxD * kMaxD];
+    __shared__ ExpTab<GP> tab;
     __shared__ unsigned int acc_s;
     const int d = a.m.d;
+    tab.load();
     for (int i = threadIdx.x; i < d * d; i += blockDim.x) Ls[i] = (Real)a.L[i];
     if (threadIdx.x == 0) acc_s = 0;
     __syncthreads();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     bool acc = false;
     if (p < a.P) acc = mala_particle<GP>(a, a.iter, p, Ls, reinterpret_cast<Real*>(sm_raw) + threadIdx.x,
-                                         blockDim.x);
+                                         blockDim.x, tab.t);
     const unsigned int nacc = __popc(__ballot_sync(0xffffffffu, acc));
     if ((threadIdx.x & 31) == 0 && nacc) atomicAdd(&acc_s, nacc);
     __syncthreads();

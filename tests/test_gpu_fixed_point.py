@@ -80,3 +80,31 @@ def test_mutation_with_out_of_range_proposals(S, K, I_, phi):
     np.testing.assert_allclose(th_g, th_o, rtol=1e-12, atol=1e-12)
     np.testing.assert_allclose(lp_g, lp_o, rtol=1e-12)
     assert np.all(ll_g[np.isfinite(ll_o) & ~sane] < -1e6)
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (2, 2), (3, 4)])
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 130])
+def test_gradient_with_range_exits(S, K, I_, T):
+    """Segment edges, a shock out of range, and parameters out of range (a
+    component far narrower than its distance from zero, a large beta), against
+    the oracle's gradient at the FP64 gradient's 1e-7 of the largest entry."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = _series(truth, T)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    P = 48
+    th = particles(spec.d, truth, K, I_, True, P, 79)
+    if I_ > 1:
+        th[:8, spec.d - 1] = -4.0                  # sigma of the last component
+        th[:8, spec.d - I_ - 1] = 3.0              # and its mean
+    th[8:12, 2 + K] = np.log(1.5)                  # beta_1
+    ll_o, g_o = O.loglik_grad(spec, y, th)
+    ll = torch.empty(P, dtype=torch.float64, device="cuda")
+    g = torch.empty((spec.d, P), dtype=torch.float64, device="cuda")
+    S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(th), ll, g)
+    ll, g = host(ll), host(g).T
+    sane = (ll_o > -1e7) & np.isfinite(g_o).all(axis=1)   # (an overflow on the way leaves the oracle's NaN)
+    assert sane[12:].sum() > 30
+    np.testing.assert_allclose(ll[sane], ll_o[sane], rtol=1e-9)
+    err = np.abs(g - g_o)[sane].max(axis=1) / np.abs(g_o[sane]).max(axis=1)
+    assert err.max() <= 1e-7, err.max()
