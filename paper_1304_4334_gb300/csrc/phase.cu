@@ -3,6 +3,7 @@
 #include "covtile.cuh"
 #include "exp2_table.h"
 
+#include <atomic>
 #include <cstdio>
 
 namespace smc {
@@ -21,6 +22,51 @@ int device_sm_count()
     return cached;
 }
 
+// ============================================================ conversions
+// Conversions on the integer pipes.  On this part the FP64 pipe (about two
+// lanes per clock per SM) also executes the conversions that touch 64-bit
+// values (FP32 <-> 64-bit integer, FP64 <-> FP32), so the search keeps them
+// out of its per-particle and per-tile work.
+//
+// floor(f) for finite f >= 0 (f < 2^64): the 24-bit significand shifted.
+__device__ __forceinline__ uint64_t f32_to_u64_floor(float f)
+{
+    const uint32_t u = __float_as_uint(f);
+    if ((u >> 23) == 0u) return 0ull;                 // zero (subnormals are flushed)
+    const int e = (int)(u >> 23) - 150;               // f = m 2^e
+    const uint64_t m = (uint64_t)((u & 0x7fffffu) | 0x800000u);
+    return e >= 0 ? m << e : (e > -24 ? m >> -e : 0ull);
+}
+
+// v to FP32 through its two 32-bit halves (each rounded, then one rounded sum).
+__device__ __forceinline__ float u64_to_f32(uint64_t v)
+{
+    return fmaf(__uint2float_rn((uint32_t)(v >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)v));
+}
+
+// d as hi + lo in FP32 from its bits: hi carries the leading 24 significand
+// bits (truncated), lo the next 29 (rounded to 24).  ok is false outside
+// 2^-126 <= |d| < 2^128 (and for inf or NaN), where the caller converts in FP64.
+// The rare FP64 paths of the conversions below, kept out of line so that the
+// compiler does not evaluate them speculatively beside the integer path.
+__device__ __noinline__ float diff_f64_to_f32(double a, double b) { return __double2float_rn(a - b); }
+__device__ __noinline__ float cvt_f64_to_f32(double d) { return __double2float_rn(d); }
+
+__device__ __forceinline__ float2 split_f64(double d, bool& ok)
+{
+    const uint64_t b = (uint64_t)__double_as_longlong(d);
+    const int e = (int)((b >> 52) & 0x7ffu) - 1023;
+    ok = e >= -126 && e <= 127;
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+    const float hi = __uint_as_float(sign | ((uint32_t)(e + 127) << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
+    float lo = 0.0f;
+    if (e - 52 >= -126) {
+        const float scale = __uint_as_float((uint32_t)(e - 52 + 127) << 23);   // 2^(e - 52)
+        lo = __uint_as_float(sign | __float_as_uint(__uint2float_rn((uint32_t)(b & 0x1fffffffu)) * scale));
+    }
+    return make_float2(hi, lo);
+}
+
 // ============================================================ covariance
 // V_lr of Section 3.3 is the sample variance of the current particles, pooled
 // over all J N.  Sums are taken about a shift (particle 0) so that the final
@@ -31,7 +77,7 @@ int device_sm_count()
 // its ~1e-6 relative accuracy leaves the Metropolis kernel exact.
 constexpr int kCovThreads = 256;
 constexpr int kCovTile = 64;
-constexpr int kCovMaxAcc = (kMaxD + kMaxD * (kMaxD + 1) / 2 + kCovThreads - 1) / kCovThreads;
+constexpr int kCovWarps = kCovThreads / 32;
 
 int cov_grid(int P)
 {
@@ -50,60 +96,179 @@ __device__ __forceinline__ void unpack_pair(int e, int& i, int& k)
     k = e - ii * (ii + 1) / 2;
 }
 
-__device__ void cov_partial_body(const double* __restrict__ theta, int d, int P,
-                                 double* __restrict__ part, int bidx, int G)
+// theta - shift rounded to FP32, without FP64 instructions: the difference of
+// the FP32 high parts is exact as a pair (TwoSum), the low parts' difference
+// joins its error term (the FP64 difference's rounding, but for ties within
+// 2^-23 of an FP32 unit).
+__device__ __forceinline__ float diff_to_f32(double th, double shift, float2 sh, bool sok)
 {
-    __shared__ float tile[kMaxD][kCovTile + 1];
+    bool ok;
+    const float2 t = split_f64(th, ok);
+    if (!(ok && sok)) return diff_f64_to_f32(th, shift);
+    const float s = t.x - sh.x;
+    const float bv = s - t.x;
+    const float e = (t.x - (s - bv)) + (-sh.x - bv);
+    return s + (e + (t.y - sh.y));
+}
+
+// Shared memory of the partial sums: per warp a tile [64][pitch] of shifted
+// values, pitch an odd multiple of 4 (the 16-byte stores of 8 lanes then fall
+// in distinct banks).
+__host__ __device__ __forceinline__ int cov_pitch(int d) { return 4 * (((d + 3) / 4) | 1); }
+size_t cov_smem(int d)
+{
+    const size_t tiles = (size_t)kCovWarps * kCovTile * cov_pitch(d) * sizeof(float);
+    const size_t sums = (size_t)kCovWarps * (d + d * (d + 1) / 2) * sizeof(double);
+    return tiles > sums ? tiles : sums;
+}
+
+// One block's partial sums: a warp per tile.  The warp stages its tile (two
+// particles a lane, four rows a store), and each lane then owns B x B products
+// x_i x_k and, on the diagonal, the B sums x_i (kRounds such blocks above
+// 28 parameters): within a tile one FMA chain per entry in the particles'
+// order, tiles added up as exact pairs (TwoSum) and converted once, so the
+// result does not depend on B.  Bound by the FMAs' issue and the loads of theta
+// (193 MB at d = 23, 1,048,576 particles).  The first form gave one entry to a
+// thread (two 4-byte loads per FMA) and formed and converted theta - shift in
+// FP64: 307 us there, now 94 us (14 parameters, 65,536 particles: the whole call
+// 35 -> 32 us).
+template <int B, int kRounds>
+__device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta, int d, int P,
+                                                double* __restrict__ part, int bidx, int G, float* sm)
+{
+    constexpr int kE = B * B + B;
     __shared__ double shift[kMaxD];
-    __shared__ int pi_[kMaxD * (kMaxD + 1) / 2], pk_[kMaxD * (kMaxD + 1) / 2];
-    const int npair = d * (d + 1) / 2;
-    const int nacc = d + npair;
+    __shared__ float2 shift2[kMaxD];
+    __shared__ bool shift_ok[kMaxD];
+    const int nb = (d + B - 1) / B, nblk = nb * (nb + 1) / 2;
+    const int nacc = d + d * (d + 1) / 2;
     const size_t Ps = (size_t)P;
-    for (int e = threadIdx.x; e < npair; e += blockDim.x) unpack_pair(e, pi_[e], pk_[e]);
-    for (int i = threadIdx.x; i < d; i += blockDim.x) shift[i] = theta[i * Ps];
-    double acc[kCovMaxAcc];
-#pragma unroll
-    for (int r = 0; r < kCovMaxAcc; ++r) acc[r] = 0.0;
-    const int per = (P + G - 1) / G;
-    const int n0 = bidx * per;
-    const int n1 = min(P, n0 + per);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        shift[i] = theta[i * Ps];
+        shift2[i] = split_f64(shift[i], shift_ok[i]);
+    }
     __syncthreads();
-    for (int base = n0; base < n1; base += kCovTile) {
-        const int cnt = min(kCovTile, n1 - base);
-        for (int e = threadIdx.x; e < d * kCovTile; e += blockDim.x) {
-            const int i = e / kCovTile, n = e % kCovTile;
-            tile[i][n] = n < cnt ? (float)(theta[i * Ps + base + n] - shift[i]) : 0.0f;
-        }
-        __syncthreads();
+    const int pitch = cov_pitch(d);
+    float* tile = sm + warp * kCovTile * pitch;
+    int bi[kRounds], bk[kRounds];
+    float hi[kRounds][kE], lo[kRounds][kE];
 #pragma unroll
-        for (int r = 0; r < kCovMaxAcc; ++r) {
-            const int e = threadIdx.x + r * blockDim.x;
-            if (e < d) {
-                float s = 0.0f;
-                for (int n = 0; n < cnt; ++n) s += tile[e][n];
-                acc[r] += (double)s;
-            } else if (e < nacc) {
-                const int i = pi_[e - d], k = pk_[e - d];
-                float s = 0.0f;
-                for (int n = 0; n < cnt; ++n) s = fmaf(tile[i][n], tile[k][n], s);
-                acc[r] += (double)s;
+    for (int q = 0; q < kRounds; ++q) {
+        unpack_pair(min(lane + 32 * q, nblk - 1), bi[q], bk[q]);
+#pragma unroll
+        for (int e = 0; e < kE; ++e) hi[q][e] = lo[q][e] = 0.0f;
+    }
+    const int per = (P + G - 1) / G;
+    const int n0 = bidx * per, n1 = min(P, n0 + per);
+    for (int base = n0 + warp * kCovTile; base < n1; base += kCovWarps * kCovTile) {
+        const int cnt = min(kCovTile, n1 - base);
+        __syncwarp();
+        for (int r = 0; r < d; r += 4) {
+            double t[2][4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    t[h][u] = r + u < d && lane + 32 * h < cnt ? theta[(size_t)(r + u) * Ps + base + lane + 32 * h] : 0.0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    x[u] = r + u < d && lane + 32 * h < cnt
+                               ? diff_to_f32(t[h][u], shift[r + u], shift2[r + u], shift_ok[r + u]) : 0.0f;
+                *reinterpret_cast<float4*>(tile + (lane + 32 * h) * pitch + r) = make_float4(x[0], x[1], x[2], x[3]);
             }
         }
-        __syncthreads();
-    }
+        __syncwarp();
 #pragma unroll
-    for (int r = 0; r < kCovMaxAcc; ++r) {
-        const int e = threadIdx.x + r * blockDim.x;
-        if (e < nacc) part[(size_t)bidx * nacc + e] = acc[r];
+        for (int q = 0; q < kRounds; ++q) {
+            float s[kE];
+#pragma unroll
+            for (int e = 0; e < kE; ++e) s[e] = 0.0f;
+            const float* ti = tile + B * bi[q];
+            const float* tk = tile + B * bk[q];
+#pragma unroll 4
+            for (int n = 0; n < kCovTile; ++n) {   // (zeros past cnt change nothing)
+                float a[B], b[B];
+                if constexpr (B == 4) {
+                    const float4 a4 = *reinterpret_cast<const float4*>(ti + n * pitch);
+                    const float4 b4 = *reinterpret_cast<const float4*>(tk + n * pitch);
+                    a[0] = a4.x, a[1] = a4.y, a[2] = a4.z, a[3] = a4.w;
+                    b[0] = b4.x, b[1] = b4.y, b[2] = b4.z, b[3] = b4.w;
+                } else if constexpr (B == 2) {
+                    const float2 a2 = *reinterpret_cast<const float2*>(ti + n * pitch);
+                    const float2 b2 = *reinterpret_cast<const float2*>(tk + n * pitch);
+                    a[0] = a2.x, a[1] = a2.y;
+                    b[0] = b2.x, b[1] = b2.y;
+                } else {
+                    a[0] = ti[n * pitch];
+                    b[0] = tk[n * pitch];
+                }
+#pragma unroll
+                for (int i = 0; i < B; ++i) {
+#pragma unroll
+                    for (int k = 0; k < B; ++k) s[B * i + k] = fmaf(a[i], b[k], s[B * i + k]);
+                    s[B * B + i] += a[i];
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < kE; ++e) {
+                const float a = hi[q][e] + s[e];
+                const float bv = a - hi[q][e];
+                lo[q][e] += (hi[q][e] - (a - bv)) + (s[e] - bv);
+                hi[q][e] = a;
+            }
+        }
+    }
+    // the warps' sums, added per entry in the warps' order
+    __syncthreads();
+    double* sums = reinterpret_cast<double*>(sm);
+#pragma unroll
+    for (int q = 0; q < kRounds; ++q) {
+        if (lane + 32 * q >= nblk) continue;
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            const int ri = B * bi[q] + i;
+            if (ri >= d) continue;
+            double* w = sums + warp * nacc;
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                const int rk = B * bk[q] + k;
+                if (rk <= ri) w[d + ri * (ri + 1) / 2 + rk] = (double)hi[q][B * i + k] + (double)lo[q][B * i + k];
+            }
+            if (bi[q] == bk[q]) w[ri] = (double)hi[q][B * B + i] + (double)lo[q][B * B + i];
+        }
+    }
+    __syncthreads();
+    const int used = min(kCovWarps, (n1 - n0 + kCovTile - 1) / kCovTile);   // warps that had a tile
+    for (int e = threadIdx.x; e < nacc; e += blockDim.x) {
+        double t = 0.0;
+        for (int w = 0; w < used; ++w) t += sums[w * nacc + e];
+        part[(size_t)bidx * nacc + e] = t;
     }
 }
 
-__global__ void __launch_bounds__(kCovThreads) k_cov_partial(const double* __restrict__ theta, int d,
-                                                            int P, double* __restrict__ part)
+template <int B, int kRounds>
+__global__ void __launch_bounds__(kCovThreads, kRounds == 1 ? 2 : 1) k_cov_partial(const double* __restrict__ theta, int d,
+                                                               int P, double* __restrict__ part)
 {
+    extern __shared__ __align__(16) float cov_sm[];
     pdl_trigger();
     pdl_wait();
-    cov_partial_body(theta, d, P, part, blockIdx.x, gridDim.x);
+    cov_partial_run<B, kRounds>(theta, d, P, part, blockIdx.x, gridDim.x, cov_sm);
+}
+
+// The smallest block that still gives every lane at most one of them: more
+// lanes at work and shorter chains of issue per tile (at d = 4, one tile per
+// block, a 4 x 4 block would sit on a single lane).
+using CovPartialFn = void (*)(const double*, int, int, double*);
+CovPartialFn cov_partial_kernel(int d)
+{
+    if (d <= 7) return k_cov_partial<1, 1>;
+    if (d <= 14) return k_cov_partial<2, 1>;
+    return d <= 28 ? k_cov_partial<4, 1> : k_cov_partial<4, 2>;
 }
 
 __device__ void apply_h_update(Ctl* ctl, int P, double target, int hmin, int hmax)
@@ -406,12 +571,14 @@ __global__ void __launch_bounds__(kCovThreads) k_cov_reduce(const void* __restri
 // A job with tile sums takes them at every iteration (the S phase's gather
 // leaves them for iteration 0, the mutation kernel for the later ones);
 // otherwise block partials of theta, exactly as the single-run path does.
-__global__ void __launch_bounds__(kCovThreads) k_cov_partial_batch(const CovJob* __restrict__ jobs,
+__global__ void __launch_bounds__(kCovThreads, 2) k_cov_partial_batch(const CovJob* __restrict__ jobs,
                                                                   const int* iter)
 {
+    extern __shared__ __align__(16) float cov_sm[];
     const CovJob& j = jobs[blockIdx.y];
     if ((int)blockIdx.x >= j.G || *iter >= j.R || j.tiles) return;
-    cov_partial_body(j.theta, j.d, j.P, j.part, blockIdx.x, j.G);
+    cov_partial_run<4, 1>(j.theta, j.d, j.P, j.part, blockIdx.x, j.G, cov_sm);   // (EGARCH: d <= 26)
+    static_assert(2 + 3 * kMaxK + 3 * kMaxI <= 28);
 }
 
 __global__ void __launch_bounds__(kCovThreads) k_cov_combine_batch(const CovJob* __restrict__ jobs, const int* iter)
@@ -436,9 +603,31 @@ __global__ void __launch_bounds__(kCovThreads) k_cov_final_batch(const CovJob* _
                    j.ctl, 0, j.target, j.hmin, j.hmax, j.mean, j.shift_f, nullptr, j.L);
 }
 
+// Raises the partial-sum kernels' shared-memory limit (74 KB at d = 32) on the
+// current device, once per device.
+static cudaError_t cov_smem_limits()
+{
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    for (const int d : {7, 14, 28, kMaxD}) {
+        e = cudaFuncSetAttribute(cov_partial_kernel(d), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)cov_smem(kMaxD));
+        if (e != cudaSuccess) return e;
+    }
+    e = cudaFuncSetAttribute(k_cov_partial_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cov_smem(kMaxD));
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
 cudaError_t launch_cov_batch(const CovJob* jobs, int n, int Gmax, int dmax, const int* iter, cudaStream_t s)
 {
-    k_cov_partial_batch<<<dim3(Gmax, n), kCovThreads, 0, s>>>(jobs, iter);
+    const cudaError_t ea = cov_smem_limits();
+    if (ea != cudaSuccess) return ea;
+    k_cov_partial_batch<<<dim3(Gmax, n), kCovThreads, cov_smem(dmax), s>>>(jobs, iter);
     count_launch();
     k_cov_combine_batch<<<dim3(dmax + dmax * (dmax + 1) / 2, n), kCovThreads, 0, s>>>(jobs, iter);
     count_launch();
@@ -451,7 +640,9 @@ cudaError_t launch_cov(const double* theta, int d, int P, double* part, int G, u
                        Ctl* ctl, int fixed_h_tenths, double acc_target, int hmin, int hmax, double* mean,
                        double* cov, double* L, cudaStream_t s, float* mean_f)
 {
-    cudaError_t e = pdl_launch(k_cov_partial, dim3(G), dim3(kCovThreads), 0, s, theta, d, P, part);
+    cudaError_t e = cov_smem_limits();
+    if (e != cudaSuccess) return e;
+    e = pdl_launch(cov_partial_kernel(d), dim3(G), dim3(kCovThreads), cov_smem(d), s, theta, d, P, part);
     count_launch();
     if (e != cudaSuccess) return e;
     const int nacc = d + d * (d + 1) / 2;
@@ -651,50 +842,6 @@ __device__ __forceinline__ long long warp_max_key(long long k)
         k = v > k ? v : k;
     }
     return k;
-}
-
-// Conversions on the integer pipes.  On this part the FP64 pipe (about two
-// lanes per clock per SM) also executes the conversions that touch 64-bit
-// values (FP32 <-> 64-bit integer, FP64 <-> FP32), so the search keeps them
-// out of its per-particle and per-tile work.
-//
-// floor(f) for finite f >= 0 (f < 2^64): the 24-bit significand shifted.
-__device__ __forceinline__ uint64_t f32_to_u64_floor(float f)
-{
-    const uint32_t u = __float_as_uint(f);
-    if ((u >> 23) == 0u) return 0ull;                 // zero (subnormals are flushed)
-    const int e = (int)(u >> 23) - 150;               // f = m 2^e
-    const uint64_t m = (uint64_t)((u & 0x7fffffu) | 0x800000u);
-    return e >= 0 ? m << e : (e > -24 ? m >> -e : 0ull);
-}
-
-// v to FP32 through its two 32-bit halves (each rounded, then one rounded sum).
-__device__ __forceinline__ float u64_to_f32(uint64_t v)
-{
-    return fmaf(__uint2float_rn((uint32_t)(v >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)v));
-}
-
-// d as hi + lo in FP32 from its bits: hi carries the leading 24 significand
-// bits (truncated), lo the next 29 (rounded to 24).  ok is false outside
-// 2^-126 <= |d| < 2^128 (and for inf or NaN), where the caller converts in FP64.
-// The rare FP64 paths of the conversions below, kept out of line so that the
-// compiler does not evaluate them speculatively beside the integer path.
-__device__ __noinline__ float diff_f64_to_f32(double a, double b) { return __double2float_rn(a - b); }
-__device__ __noinline__ float cvt_f64_to_f32(double d) { return __double2float_rn(d); }
-
-__device__ __forceinline__ float2 split_f64(double d, bool& ok)
-{
-    const uint64_t b = (uint64_t)__double_as_longlong(d);
-    const int e = (int)((b >> 52) & 0x7ffu) - 1023;
-    ok = e >= -126 && e <= 127;
-    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-    const float hi = __uint_as_float(sign | ((uint32_t)(e + 127) << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
-    float lo = 0.0f;
-    if (e - 52 >= -126) {
-        const float scale = __uint_as_float((uint32_t)(e - 52 + 127) << 23);   // 2^(e - 52)
-        lo = __uint_as_float(sign | __float_as_uint(__uint2float_rn((uint32_t)(b & 0x1fffffffu)) * scale));
-    }
-    return make_float2(hi, lo);
 }
 
 // Particles split into one contiguous range of 32-particle tiles per block.

@@ -559,3 +559,22 @@ def test_prior_draws_match_the_oracle(S):
         np.testing.assert_allclose(th, th_o, rtol=1e-12, atol=1e-13)
         mean, sd, lo = O.table1_prior(K, I_)
         assert np.all(th >= lo)
+
+
+@pytest.mark.parametrize("d,P", [(1, 2), (7, 63), (8, 64), (14, 65), (15, 1000), (28, 20000), (29, 129), (32, 40000)])
+def test_covariance_block_shapes_match_numpy(S, d, P):
+    """Each blocking of the covariance's partial sums (d up to 7, 14, 28, 32),
+    full and ragged tiles: FP32 products within 64-particle tiles leave V
+    within 64 x 2^-24 of its largest entry; the factor reproduces (h^2) V."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(100 * d + P)
+    th = rng.normal(size=(P, d)) * 0.5 + np.linspace(-2.0, 2.0, d)
+    mean, cov, L = (torch.empty(s, dtype=torch.float64, device="cuda") for s in ((d,), (d, d), (d, d)))
+    S.cov_chol(soa(th), 5, mean, cov, L)
+    want = np.cov(th.T).reshape(d, d)
+    tol = 64 * 2.0 ** -24 * np.abs(want).max()
+    assert np.abs(host(cov) - want).max() <= tol
+    np.testing.assert_allclose(host(mean), th.mean(axis=0), atol=64 * 2.0 ** -24)
+    if P > 4 * d:
+        Lh = host(L)
+        assert np.abs(Lh @ Lh.T - 0.25 * want).max() <= 2 * tol
