@@ -67,6 +67,25 @@ static int balanced_threads(int P, int ppt)
     return kMutMaxThreads;
 }
 
+// Blocks of up to 224 threads, sized to the SM count, while more than four warps
+// per SM are there and at most three such blocks per SM hold them (the SMs are
+// then evenly loaded: K=2, I=2, 65,536 x 2,000 in FP32 0.125 ms against
+// 0.128 ms in 128-thread blocks, in FP64 2.18 against 2.24 ms; 98,304: 0.178
+// against 0.182 ms), 128 beyond (131,072: 0.206 against 0.213 ms).  Two
+// particles per thread only at I = 1, where there is no mixture to pair over
+// observations, and from 40 warps per SM (K=1, 262,144 x 2,000: 0.170 against
+// 0.187 ms; 196,608: equal; K=3, I=4, 524,288: 1.41 ms against 1.29 ms with one
+// particle per thread).
+void mutate_default_shape(const ModelDev& m, int precision, bool random_walk, int P, int* ppt, int* threads)
+{
+    const int warps = (P + 31) / 32, sms = device_sm_count();
+    *ppt = 1;
+    *threads = kMutThreads;
+    if (m.kind == SMC_LINREG) return;
+    if (warps > 4 * sms && warps <= 3 * sms * (kMutMaxThreads / 32)) *threads = balanced_threads(P, 1);
+    else if (m.I == 1 && precision == SMC_FP32 && random_walk && warps >= 40 * sms) *ppt = 2;
+}
+
 cudaError_t launch_mutate_x2(const MutateArgs& a, int threads, cudaStream_t s)
 {
     if (a.qmean || !valid_mut_threads(threads)) return cudaErrorInvalidValue;   // random walk only
@@ -776,6 +795,8 @@ smc_status smc_init(const smc_model* m, const smc_config* c, const double* y, co
     ctx->ns = m->model == SMC_EGARCH ? m->K + 1 : 0;
     ctx->W = m->model == SMC_LINREG ? smc_linreg_width(m->p) : 1;
     ctx->stream = (cudaStream_t)stream;
+    if (c->mutation != SMC_MALA)
+        mutate_default_shape(ctx->mdev, c->precision, c->mutation == SMC_RW, ctx->P, &ctx->ppt, &ctx->mut_threads);
     const int P = ctx->P, d = ctx->d, J = c->J;
     const size_t Ps = (size_t)P;
 

@@ -3,10 +3,28 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "phase.cuh"
+
+#include <type_traits>
 
 namespace smc {
 
 inline int mutate_grid(int P, int threads = kMutThreads) { return (P + threads - 1) / threads; }
+
+// The kernel variant for P particles (one per thread): the policy's Wide form,
+// where it has one, while the particles leave the SMs room for it.
+template <class Pol, class = void>
+struct MutateKernel {
+    static void (*pick(int))(MutateArgs) { return k_mutate<Pol>; }
+};
+template <class Pol>
+struct MutateKernel<Pol, std::enable_if_t<!std::is_same_v<typename Pol::Wide, Pol> && (Pol::kMinBlocks > 1) &&
+                                          (Pol::kNi > 2)>> {
+    static void (*pick(int P))(MutateArgs)
+    {
+        return P <= kWideWarpsPerSm * 32 * device_sm_count() ? k_mutate<typename Pol::Wide> : k_mutate<Pol>;
+    }
+};
 
 // One particle per thread; threads = a multiple of 32 up to kMutMaxThreads (the caller checks).
 template <template <int, int> class Pol, int K>
@@ -25,10 +43,10 @@ cudaError_t launch_mutate_k(const MutateArgs& a, int threads, cudaStream_t s)
     }
     void (*k)(MutateArgs) = nullptr;
     switch (a.m.I) {
-    case 1: k = k_mutate<Pol<K, 1>>; break;
-    case 2: k = k_mutate<Pol<K, 2>>; break;
-    case 3: k = k_mutate<Pol<K, 3>>; break;
-    case 4: k = k_mutate<Pol<K, 4>>; break;
+    case 1: k = MutateKernel<Pol<K, 1>>::pick(a.P); break;
+    case 2: k = MutateKernel<Pol<K, 2>>::pick(a.P); break;
+    case 3: k = MutateKernel<Pol<K, 3>>::pick(a.P); break;
+    case 4: k = MutateKernel<Pol<K, 4>>::pick(a.P); break;
     default: return cudaErrorInvalidValue;
     }
     if (a.dependent) return pdl_launch(k, g, threads, 0, s, a);

@@ -68,14 +68,14 @@ constexpr int kMutThreads = 128;
 // Largest mutation block (threads, a multiple of 32): any multiple of 32 up to
 // this is a valid launch shape, so that P particles can be spread as evenly
 // as the warp granularity allows over the SMs.  The launch bounds also steer
-// the register allocation, and with it the speed (measured on the FP32
-// EGARCH(2,2) kernels, 65,536 particles in 224-thread blocks): one particle
-// per thread is fastest compiled for 256-thread blocks (48 registers,
-// 0.282 ms per launch against 0.292 ms with 56 registers under a 224 or
-// 128 bound, 0.288 ms at a 64-register cap), two per thread for 224 (111
-// registers, 0.297 ms; 80 registers under a 256 bound: 0.307 ms).
+// the register allocation, and with it the speed: one particle per thread
+// under a 224 bound (72 registers at K=3, I=4, 56 at K=2, I=2) takes
+// 2.53 / 0.274 ms (1,048,576 x 2,000 / 65,536 x 5,000 particles x
+// observations) against 2.57 / 0.277 ms under a 256 bound (64, 48 registers),
+// but I = 1 is 2% faster under 256; two per thread needs 224 (111 registers at
+// K=2, I=2, 0.297 ms; 80 under a 256 bound, 0.307 ms; 96 registers at K=3,
+// I=4, five warps a scheduler: 2.71 ms against 2.68 ms with 128).
 constexpr int kMutMaxThreads = 224;
-constexpr int kMutBoundX1 = 256;
 
 // Probability integral transform draw (Section 4.1): the standardized shock
 // of Y_s ~ p(Y_s | y_1:s-1, theta), location + scale * e, so that
@@ -139,6 +139,7 @@ struct PolicyEgarchF32T {
     using Model = EgarchF32<K, I, kDelta>;
     static constexpr int kNs = K + 1;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;   // Table 1
+    static constexpr int kBound = I == 1 ? 256 : kMutMaxThreads, kMinBlocks = 0;
     static constexpr bool kExpTab = false;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* = nullptr)
     {
@@ -178,14 +179,21 @@ struct PolicyEgarchF32Delta : PolicyEgarchF32T<K, I, true> {};
 // FP64: the fixed-point recursion for whole series (PolicyEgarchF64Fx: M phase,
 // stand-alone likelihood), the FP64 recursion observation by observation
 // (PolicyEgarchF64: data-tempering C phase).
-template <int K, int I>
-struct PolicyEgarchF64Fx {
+// kWide: no register cap.  Two blocks of 224 per SM (128 registers) are faster
+// where the particles fill them (K=3, I=4, 65,536 x 2,000: 4.0 ms against
+// 5.0 ms with 187 registers; K=I=1: 0.96 against 1.01 ms), except at I = 2
+// (2.21 against 2.18 ms); with at most 10 warps per SM the kernel is bound by
+// each warp's own latency and the spills cost (K=3, I=4, 10,007 particles:
+// 2.10 ms against 1.88 ms).
+template <int K, int I, bool kWide = (I == 2)>
+struct PolicyEgarchF64FxT {
     using Real = double;
     using Obs = double;
     static constexpr int kChunk = kChunkF64;
     using Model = EgarchFxSafe<K, I>;
-    static constexpr int kNs = K + 1;
+    static constexpr int kNs = K + 1, kNi = I;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;
+    static constexpr int kBound = kMutMaxThreads, kMinBlocks = kWide ? 0 : 2;   // (0: no minimum)
     static constexpr bool kExpTab = true;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* tab)
     {
@@ -194,6 +202,12 @@ struct PolicyEgarchF64Fx {
     __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f64(mdl, pipe, T); }
     __device__ static void state_out(const Model& mdl, double* st) { mdl.state_out(st); }
 };
+
+template <int K, int I>
+struct PolicyEgarchF64Fx : PolicyEgarchF64FxT<K, I> {
+    using Wide = PolicyEgarchF64FxT<K, I, true>;
+};
+constexpr int kWideWarpsPerSm = 10;
 
 template <int K, int I>
 struct PolicyEgarchF64 {
@@ -228,6 +242,7 @@ struct PolicyLinreg {
     using Model = LinregF64;
     static constexpr int kNs = 0;
     static constexpr int kMaxFree = 8;
+    static constexpr int kBound = 256, kMinBlocks = 0;
     static constexpr bool kExpTab = false;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t*)
     {
@@ -391,8 +406,7 @@ __device__ __forceinline__ void mutate_tile(const MutateArgs& a, uint64_t iter, 
 }
 
 template <class Pol, bool kIndep = false>
-__global__ void __launch_bounds__(Pol::kExpTab ? kMutMaxThreads : kMutBoundX1, Pol::kExpTab ? 2 : 1)
-k_mutate(MutateArgs a)
+__global__ void __launch_bounds__(Pol::kBound, Pol::kMinBlocks) k_mutate(MutateArgs a)
 {
     __shared__ MutateSmem<Pol> sm;
     mutate_tile<Pol, kIndep>(a, a.iter, blockIdx.x * blockDim.x, sm);
@@ -819,6 +833,10 @@ __global__ void __launch_bounds__(kMutThreads) k_cdata(CdataArgs a)
 cudaError_t launch_indep_logq(const double* theta, int d, int P, const double* L, const double* qmean,
                               double* lq, cudaStream_t s);
 cudaError_t launch_mutate(const MutateArgs& a, int precision, int threads, cudaStream_t s);
+cudaError_t launch_mutate_x2(const MutateArgs& a, int threads, cudaStream_t s);
+// Launch shape of a mutation without an autotuned one: particles per thread
+// (2 only for the FP32 EGARCH random walk) and threads per block.
+void mutate_default_shape(const ModelDev& m, int precision, bool random_walk, int P, int* ppt, int* threads);
 cudaError_t launch_loglik(const LoglikArgs& a, int precision, cudaStream_t s);
 cudaError_t launch_cdata(const CdataArgs& a, int precision, cudaStream_t s);
 

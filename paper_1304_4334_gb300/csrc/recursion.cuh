@@ -169,6 +169,21 @@ __device__ __forceinline__ void egarch_transform(const Real* th, int has_gamma,
     }
 }
 
+// Blackwell's paired FP32 instructions (each lane rounds as the scalar one).
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 f2_sub(float2 a, float2 b)
+{
+    unsigned long long x, y, r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    float2 o;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
+    return o;
+}
+
 // ------------------------------------------------------------- FP32 recursion
 // The first factor carries log2 sigma_Y - log2 s: u = lsy2p + v'_1, so that
 // log2 h - log2 s = u + v'_2 + ... + v'_K; its update is
@@ -304,6 +319,77 @@ struct EgarchF32 {
     {
         chain<kFirst>(y);
         mix(es);
+    }
+
+    // The mixture's constants for a pair of observations.
+    struct MixPair {
+        float2 a[I], b[I], nc[I];          // 1/sigma_i; -mu_i s / sigma_i; -log2(p_i / sigma_i)
+    };
+    __device__ __forceinline__ MixPair mix_pair() const
+    {
+        MixPair c2;
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            c2.a[i] = make_float2(a[i], a[i]);
+            c2.b[i] = make_float2(b[i], b[i]);
+            c2.nc[i] = make_float2(-c[i], -c[i]);
+        }
+        return c2;
+    }
+
+    // mix(x.x); mix(x.y) with the two observations' terms in paired FP32
+    // instructions: the shocks of consecutive observations wait for each other
+    // only in the chain.  The terms are carried negated (y_i = -x_i exactly),
+    // and the sums keep their order, so the results are bitwise the scalar
+    // ones.  The kernel is bound by the issue of its instructions and by
+    // FP32-pipe conflicts; this takes 5 (I = 2) to 11 (I = 4) instructions off
+    // two observations: K=3, I=4, 524,288 particles x 2,000: 1.41 -> 1.29 ms
+    // (two particles per thread: 1.41), K=2, I=2, 65,536 x 5,000: 0.278 ->
+    // 0.274 ms, K=2, I=3, 524,288 x 2,000: 1.04 -> 0.96 ms.
+    __device__ __forceinline__ void mix2(float2 x, const MixPair& q)
+    {
+        if constexpr (I == 1) {
+            mix(x.x);
+            mix(x.y);
+        } else if constexpr (I == 2) {
+            const float2 z0 = f2_fma(q.a[0], x, q.b[0]), z1 = f2_fma(q.a[1], x, q.b[1]);
+            const float2 y0 = f2_fma(z0, z0, q.nc[0]), y1 = f2_fma(z1, z1, q.nc[1]);
+            const float2 dd = f2_sub(y1, y0);
+            sm += fmaxf(-y0.x, -y1.x);
+            sm += fmaxf(-y0.y, -y1.y);
+            prod = fmaf(prod, ex2_approx(-fabsf(dd.x)), prod);
+            prod = fmaf(prod, ex2_approx(-fabsf(dd.y)), prod);
+        } else {
+            float2 yv[I];
+#pragma unroll
+            for (int i = 0; i < I; ++i) {
+                const float2 z = f2_fma(q.a[i], x, q.b[i]);
+                yv[i] = f2_fma(z, z, q.nc[i]);
+            }
+            float2 m = make_float2(-yv[0].x, -yv[0].y);
+#pragma unroll
+            for (int i = 1; i < I; ++i) m = make_float2(fmaxf(m.x, -yv[i].x), fmaxf(m.y, -yv[i].y));
+            float2 t = f2_add(yv[0], m);
+            float2 ssum = make_float2(ex2_approx(-t.x), ex2_approx(-t.y));
+#pragma unroll
+            for (int i = 1; i < I; ++i) {
+                t = f2_add(yv[i], m);
+                ssum = f2_add(ssum, make_float2(ex2_approx(-t.x), ex2_approx(-t.y)));
+            }
+            sm += m.x;
+            sm += m.y;
+            prod *= ssum.x;
+            prod *= ssum.y;
+        }
+    }
+
+    template <bool kFirst>
+    __device__ __forceinline__ void step2(float y0, float y1, const MixPair& q)
+    {
+        chain<kFirst>(y0);
+        const float e0 = es;
+        chain<false>(y1);
+        mix2(make_float2(e0, es), q);
     }
 
     // Continue from a saved state (natural units) and evaluate one observation's
@@ -733,6 +819,7 @@ template <int K, int I, bool kDelta>
 __device__ __forceinline__ bool run_egarch_f32(EgarchF32<K, I, kDelta>& mdl, ObsPipe<float, kChunkF32>& pipe,
                                                int T)
 {
+    const typename EgarchF32<K, I, kDelta>::MixPair mp = mdl.mix_pair();
     for (int c = 0; c < pipe.nchunks; ++c) {
         if (!pipe.wait(c)) {
             pipe.drain(c);
@@ -745,26 +832,20 @@ __device__ __forceinline__ bool run_egarch_f32(EgarchF32<K, I, kDelta>& mdl, Obs
             const float4* y4 = reinterpret_cast<const float4*>(yb + 32 * u);
             if (c == 0 && u == 0) {
                 float4 q = y4[0];
-                mdl.template step<true>(q.x);
-                mdl.template step<false>(q.y);
-                mdl.template step<false>(q.z);
-                mdl.template step<false>(q.w);
+                mdl.template step2<true>(q.x, q.y, mp);
+                mdl.template step2<false>(q.z, q.w, mp);
 #pragma unroll
                 for (int j = 1; j < 8; ++j) {
                     q = y4[j];
-                    mdl.template step<false>(q.x);
-                    mdl.template step<false>(q.y);
-                    mdl.template step<false>(q.z);
-                    mdl.template step<false>(q.w);
+                    mdl.template step2<false>(q.x, q.y, mp);
+                    mdl.template step2<false>(q.z, q.w, mp);
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float4 q = y4[j];
-                    mdl.template step<false>(q.x);
-                    mdl.template step<false>(q.y);
-                    mdl.template step<false>(q.z);
-                    mdl.template step<false>(q.w);
+                    mdl.template step2<false>(q.x, q.y, mp);
+                    mdl.template step2<false>(q.z, q.w, mp);
                 }
             }
             mdl.flush();
@@ -785,7 +866,7 @@ __device__ __forceinline__ bool run_egarch_f32(EgarchF32<K, I, kDelta>& mdl, Obs
 }
 
 // ------------------------------------------- two particles in packed FP32x2
-// Blackwell's paired FP32 instructions (fma/add/mul/sub .f32x2) run the same
+// Paired FP32 instructions (fma/add/mul/sub .f32x2) run the same
 // operation on two particles' recursions in one issue slot.  The pair is
 // packed from two set-up EgarchF32 models and unpacked back into them, and
 // every lane performs exactly the scalar recursion's operations in its order
@@ -793,20 +874,6 @@ __device__ __forceinline__ bool run_egarch_f32(EgarchF32<K, I, kDelta>& mdl, Obs
 // EgarchF32 runs.  The mixture terms are carried negated where that saves a
 // negation: y_i = z_i^2 - c_i = -x_i exactly, max_i x_i = max_i(-y_i),
 // x_0 - x_1 = y_1 - y_0.
-__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 f2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 f2_sub(float2 a, float2 b)
-{
-    unsigned long long x, y, r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
-    asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
-    float2 o;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
-    return o;
-}
-
 template <int K, int I>
 struct EgarchF32Pair {
     float2 nmu;                            // -mu_Y

@@ -139,7 +139,9 @@ static smc_status mutate_impl(const smc_model* m, int precision, const void* obs
     a.acc_count = cnt;
     a.pending = nullptr;
     a.err = nullptr;
-    cudaError_t e = launch_mutate(a, precision, kMutThreads, s);
+    int ppt, threads;
+    mutate_default_shape(a.m, precision, qmean == nullptr, P, &ppt, &threads);
+    cudaError_t e = ppt == 2 ? launch_mutate_x2(a, threads, s) : launch_mutate(a, precision, threads, s);
     unsigned long long h = 0;
     if (e == cudaSuccess && accepted) {
         e = cudaMemcpyAsync(&h, cnt, sizeof h, cudaMemcpyDeviceToHost, s);
