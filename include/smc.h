@@ -392,8 +392,11 @@ void smc_batch_free(smc_batch* b);
 /* ---------------------------------------------------------------------------
  * Stateless entry points on caller-owned device memory (for tests, autograd
  * and custom drivers).  All enqueue on `stream`; temporaries they need are
- * allocated stream-ordered (cudaMallocAsync) and released before return.
+ * allocated stream-ordered from the library's memory pool of the current device
+ * and released to it before return.  The pool keeps up to 512 MiB for the next
+ * call; smc_release_workspace gives the unused part back to the device.
  * ------------------------------------------------------------------------- */
+smc_status smc_release_workspace(void);
 
 /* Log likelihood log p(y_1:T | theta) of Section 5.1 (four evaluation steps)
  * for P particles.  obs: device observations, float[T] for EGARCH with

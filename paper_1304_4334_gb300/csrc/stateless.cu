@@ -1,6 +1,7 @@
 // Stateless entry points of the C ABI: each phase kernel on caller-owned device
 // memory, for tests, the autograd binding and custom drivers.  Temporaries are
-// allocated stream-ordered on the caller's stream and freed before returning.
+// allocated stream-ordered on the caller's stream, one block per call, from the
+// library's memory pool, and freed before returning.
 #include "../../include/smc.h"
 #include "kernels.cuh"
 #include "mala.cuh"
@@ -8,6 +9,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <mutex>
 
 namespace smc {
 void count_launch();
@@ -60,6 +62,82 @@ bool model_ok(const smc_model* m, int precision)
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
+// The pool of the stateless calls' temporaries, one per device, made at the
+// first call.  It keeps up to kPoolKeep bytes across synchronisations: the
+// device's default pool gives everything back at each one, and every call here
+// that returns a number synchronises, so a call after a device-wide wait paid
+// 200 us for mapping its memory again (random walk, K=2, I=2, 65,536 x 5,000:
+// first call after a wait 545 -> 341 us; power search, S phase and covariance
+// at 1,024 particles: 475 -> 250 us; calls in a row cost the same).  What is kept serves every stream and thread (the pool orders
+// reuse between streams itself); smc_release_workspace() gives it back.
+constexpr uint64_t kPoolKeep = 512ull << 20;
+constexpr int kMaxPools = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxPools] = {};
+
+cudaError_t pool_of_device(cudaMemPool_t* out)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxPools) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof props);
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        e = cudaMemPoolCreate(&pool, &props);
+        if (e != cudaSuccess) return e;
+        uint64_t keep = kPoolKeep;
+        e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(pool);
+            return e;
+        }
+        g_pool[dev] = pool;
+    }
+    *out = g_pool[dev];
+    return cudaSuccess;
+}
+
+// One call's temporaries: a single stream-ordered block cut into 256-byte
+// aligned parts, freed (stream-ordered) when it goes out of scope.  add() every
+// part, then get(), then take() them in the same order.
+class Scratch {
+public:
+    explicit Scratch(cudaStream_t s) : s_(s) {}
+    ~Scratch()
+    {
+        if (base_) cudaFreeAsync(base_, s_);
+    }
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    void add(size_t bytes) { size_ += round(bytes); }
+    cudaError_t get()
+    {
+        cudaMemPool_t pool = nullptr;
+        const cudaError_t e = pool_of_device(&pool);
+        if (e != cudaSuccess) return e;
+        return cudaMallocFromPoolAsync((void**)&base_, size_ ? size_ : 256, pool, s_);
+    }
+    template <typename T>
+    T* take(size_t bytes)
+    {
+        char* p = base_ + used_;
+        used_ += round(bytes);
+        return reinterpret_cast<T*>(p);
+    }
+
+private:
+    static size_t round(size_t b) { return (b + 255) & ~(size_t)255; }
+    cudaStream_t s_;
+    char* base_ = nullptr;
+    size_t size_ = 0, used_ = 0;
+};
+
 smc_status from_cuda(cudaError_t e) { return e == cudaSuccess ? SMC_OK : SMC_ECUDA; }
 
 }  // namespace
@@ -71,6 +149,15 @@ smc_status from_cuda(cudaError_t e) { return e == cudaSuccess ? SMC_OK : SMC_ECU
     } while (0)
 
 extern "C" {
+
+smc_status smc_release_workspace(void)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SMC_ECUDA;
+    if (dev < 0 || dev >= kMaxPools) return SMC_OK;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    return g_pool[dev] ? from_cuda(cudaMemPoolTrimTo(g_pool[dev], 0)) : SMC_OK;
+}
 
 smc_status smc_loglik(const smc_model* m, int precision, const void* obs, int T, const double* theta,
                       int P, double* ll, double* lp, double* state, void* stream)
@@ -103,16 +190,17 @@ static smc_status mutate_impl(const smc_model* m, int precision, const void* obs
         return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int d = m->n_free > 0 ? m->n_free : m->d_full;
-    double* thp = nullptr;
-    unsigned long long* cnt = nullptr;
-    CK(cudaMallocAsync((void**)&thp, (size_t)P * d * sizeof(double), s));
-    CK(cudaMallocAsync((void**)&cnt, sizeof(unsigned long long), s));
+    const size_t n_thp = (size_t)P * d * sizeof(double), n_lq = qmean ? (size_t)P * sizeof(double) : 0;
+    Scratch w(s);
+    w.add(n_thp);
+    w.add(sizeof(unsigned long long));
+    w.add(n_lq);
+    CK(w.get());
+    double* thp = w.take<double>(n_thp);
+    unsigned long long* cnt = w.take<unsigned long long>(sizeof(unsigned long long));
+    double* lq = qmean ? w.take<double>(n_lq) : nullptr;
     CK(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
-    double* lq = nullptr;
-    if (qmean) {
-        CK(cudaMallocAsync((void**)&lq, (size_t)P * sizeof(double), s));
-        CK(launch_indep_logq(theta, d, P, L, qmean, lq, s));
-    }
+    if (qmean) CK(launch_indep_logq(theta, d, P, L, qmean, lq, s));
     MutateArgs a;
     a.m = ModelDev{};
     model_dev(*m, a.m);
@@ -148,9 +236,6 @@ static smc_status mutate_impl(const smc_model* m, int precision, const void* obs
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         *accepted = h;
     }
-    cudaFreeAsync(thp, s);
-    cudaFreeAsync(cnt, s);
-    if (lq) cudaFreeAsync(lq, s);
     return from_cuda(e);
 }
 
@@ -191,11 +276,12 @@ smc_status smc_loglik_grad(const smc_model* m, int precision, const void* obs, i
     a.ll = ll;
     a.grad = grad;
     a.state = m->model == SMC_EGARCH ? state : nullptr;
-    a.ckpt = nullptr;
-    CK(cudaMallocAsync(&a.ckpt, mala_ckpt_bytes(a.m, precision, T, P), s));
-    const cudaError_t e = launch_loglik_grad(a, precision, s);
-    cudaFreeAsync(a.ckpt, s);
-    return from_cuda(e);
+    const size_t n_ckpt = mala_ckpt_bytes(a.m, precision, T, P);
+    Scratch w(s);
+    w.add(n_ckpt);
+    CK(w.get());
+    a.ckpt = w.take<void>(n_ckpt);
+    return from_cuda(launch_loglik_grad(a, precision, s));
 }
 
 smc_status smc_mutate_mala(const smc_model* m, int precision, const void* obs, int T, double* theta,
@@ -207,7 +293,6 @@ smc_status smc_mutate_mala(const smc_model* m, int precision, const void* obs, i
         !aligned16(obs) || !(phi >= 0.0))
         return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned long long* cnt = nullptr;
     MalaArgs a;
     a.m = ModelDev{};
     model_dev(*m, a.m);
@@ -219,7 +304,6 @@ smc_status smc_mutate_mala(const smc_model* m, int precision, const void* obs, i
     a.lp = lp;
     a.state = m->model == SMC_EGARCH ? state : nullptr;
     a.grad = grad;
-    a.ckpt = nullptr;
     a.P = P;
     a.ns = m->model == SMC_EGARCH ? m->K + 1 : 0;
     a.L = L;
@@ -229,8 +313,13 @@ smc_status smc_mutate_mala(const smc_model* m, int precision, const void* obs, i
     a.iter = iter;
     a.pending = nullptr;
     a.err = nullptr;
-    CK(cudaMallocAsync(&a.ckpt, mala_ckpt_bytes(a.m, precision, T, P), s));
-    CK(cudaMallocAsync((void**)&cnt, sizeof(unsigned long long), s));
+    const size_t n_ckpt = mala_ckpt_bytes(a.m, precision, T, P);
+    Scratch w(s);
+    w.add(n_ckpt);
+    w.add(sizeof(unsigned long long));
+    CK(w.get());
+    a.ckpt = w.take<void>(n_ckpt);
+    unsigned long long* cnt = w.take<unsigned long long>(sizeof(unsigned long long));
     CK(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), s));
     a.acc_count = cnt;
     cudaError_t e = launch_mala(a, precision, s);
@@ -240,8 +329,6 @@ smc_status smc_mutate_mala(const smc_model* m, int precision, const void* obs, i
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         *accepted = h;
     }
-    cudaFreeAsync(a.ckpt, s);
-    cudaFreeAsync(cnt, s);
     return from_cuda(e);
 }
 
@@ -251,14 +338,14 @@ smc_status smc_cov_chol(const double* theta, int d, int P, int h_tenths, double*
     if (!theta || d < 1 || d > SMC_MAX_D || P < 2 || h_tenths < 0) return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     const int G = cov_grid(P);
-    double* part = nullptr;
     const size_t n = (size_t)(G + 1) * (d + d * (d + 1) / 2);
-    CK(cudaMallocAsync((void**)&part, (n + 1) * sizeof(double), s));
+    Scratch w(s);
+    w.add((n + 1) * sizeof(double));
+    CK(w.get());
+    double* part = w.take<double>((n + 1) * sizeof(double));
     unsigned int* counter = reinterpret_cast<unsigned int*>(part + n);
     CK(cudaMemsetAsync(counter, 0, sizeof(unsigned int), s));
-    cudaError_t e = launch_cov(theta, d, P, part, G, counter, nullptr, h_tenths, 0.0, 1, 10, mean, cov, L, s);
-    cudaFreeAsync(part, s);
-    return from_cuda(e);
+    return from_cuda(launch_cov(theta, d, P, part, G, counter, nullptr, h_tenths, 0.0, 1, 10, mean, cov, L, s));
 }
 
 smc_status smc_power_search(const double* ll, int P, double phi, double d1, int passes, double* dphi,
@@ -267,19 +354,20 @@ smc_status smc_power_search(const double* ll, int P, double phi, double d1, int 
     if (!ll || P < 1 || !(phi >= 0.0 && phi < 1.0) || !(d1 > 0.0 && d1 < 1.0) || passes < 1)
         return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    double* part = nullptr;
-    Ctl* ctl = nullptr;
-    double* gstat = nullptr;
-    double* lw = nullptr;
-    double* a = nullptr;
-    int32_t* idx = nullptr;
-    CK(cudaMallocAsync((void**)&part, search_part_len(P) * sizeof(double), s));
+    const size_t n_part = search_part_len(P) * sizeof(double), n_idx = (size_t)P * sizeof(int32_t);
+    Scratch w(s);
+    w.add(n_part);
+    w.add(sizeof(Ctl));
+    for (int i = 0; i < 3; ++i) w.add(3 * sizeof(double));   // gstat, lw, a
+    w.add(n_idx);
+    CK(w.get());
+    double* part = w.take<double>(n_part);
+    Ctl* ctl = w.take<Ctl>(sizeof(Ctl));
+    double* gstat = w.take<double>(3 * sizeof(double));
+    double* lw = w.take<double>(3 * sizeof(double));
+    double* a = w.take<double>(3 * sizeof(double));
+    int32_t* idx = w.take<int32_t>(n_idx);
     CK(cudaMemsetAsync(part, 0, search_bar_bytes(), s));
-    CK(cudaMallocAsync((void**)&ctl, sizeof(Ctl), s));
-    CK(cudaMallocAsync((void**)&gstat, 3 * sizeof(double), s));
-    CK(cudaMallocAsync((void**)&lw, sizeof(double), s));
-    CK(cudaMallocAsync((void**)&a, sizeof(double), s));
-    CK(cudaMallocAsync((void**)&idx, (size_t)P * sizeof(int32_t), s));
     Ctl init;
     std::memset(&init, 0, sizeof init);
     init.phi = phi;
@@ -311,12 +399,6 @@ smc_status smc_power_search(const double* ll, int P, double phi, double d1, int 
         if (dphi) *dphi = h.dphi;
         if (rss) *rss = P <= SMC_MAX_N ? h.rss : NAN;
     }
-    cudaFreeAsync(part, s);
-    cudaFreeAsync(ctl, s);
-    cudaFreeAsync(gstat, s);
-    cudaFreeAsync(lw, s);
-    cudaFreeAsync(a, s);
-    cudaFreeAsync(idx, s);
     return from_cuda(e);
 }
 
@@ -325,8 +407,10 @@ smc_status smc_resample(const double* w, int J, int N, int resampler, uint64_t s
 {
     if (!w || !idx || J < 1 || N < 1 || N > SMC_MAX_N) return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    int* err = nullptr;
-    CK(cudaMallocAsync((void**)&err, sizeof(int), s));
+    Scratch w_(s);
+    w_.add(sizeof(int));
+    CK(w_.get());
+    int* err = w_.take<int>(sizeof(int));
     CK(cudaMemsetAsync(err, 0, sizeof(int), s));
     SelectArgs sa;
     std::memset(&sa, 0, sizeof sa);
@@ -343,7 +427,6 @@ smc_status smc_resample(const double* w, int J, int N, int resampler, uint64_t s
     int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(err, s);
     if (e != cudaSuccess) return SMC_ECUDA;
     if (h & kErrDegenerate) return SMC_EDEGENERATE;
     return h ? SMC_ECUDA : SMC_OK;
@@ -354,12 +437,14 @@ smc_status smc_resample_logw(const double* logw, int J, int N, int resampler, ui
 {
     if (!logw || !idx || J < 1 || N < 1 || N > SMC_MAX_N || resampler < 0 || resampler > 3) return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    int* err = nullptr;
-    double* buf = nullptr;   // a [J], lw [J], gstat [3 J]
-    CK(cudaMallocAsync((void**)&err, sizeof(int), s));
-    CK(cudaMallocAsync((void**)&buf, (size_t)5 * J * sizeof(double), s));
-    CK(cudaMemsetAsync(err, 0, sizeof(int), s));
-    CK(cudaMemsetAsync(buf, 0, (size_t)J * sizeof(double), s));
+    // a [J] and the error word (cleared together), lw [J], gstat [3 J]
+    const size_t n_buf = (size_t)(5 * J + 1) * sizeof(double);
+    Scratch w(s);
+    w.add(n_buf);
+    CK(w.get());
+    double* buf = w.take<double>(n_buf);
+    int* err = reinterpret_cast<int*>(buf + J);
+    CK(cudaMemsetAsync(buf, 0, (size_t)(J + 1) * sizeof(double), s));
     SelectArgs sa;
     std::memset(&sa, 0, sizeof sa);
     sa.mode = 1;
@@ -370,18 +455,16 @@ smc_status smc_resample_logw(const double* logw, int J, int N, int resampler, ui
     sa.seed = seed;
     sa.cycle = cycle;
     sa.a = buf;
-    sa.lw = buf + J;
-    sa.gstat = buf + 2 * J;
+    sa.lw = buf + J + 1;
+    sa.gstat = buf + 2 * J + 1;
     sa.idx = idx;
     sa.err = err;
     cudaError_t e = launch_select(sa, s);
     int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && lwbar)
-        e = cudaMemcpyAsync(lwbar, buf + J, (size_t)J * sizeof(double), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(lwbar, buf + J + 1, (size_t)J * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(err, s);
-    cudaFreeAsync(buf, s);
     if (e != cudaSuccess) return SMC_ECUDA;
     if (h & kErrDegenerate) return SMC_EDEGENERATE;
     return h ? SMC_ECUDA : SMC_OK;
@@ -391,15 +474,16 @@ smc_status smc_group_moments(const double* g, int nf, int J, int N, double* out,
 {
     if (!g || !out || nf < 1 || J < 2 || N < 1) return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    double* part = nullptr;
-    double* dout = nullptr;
-    CK(cudaMallocAsync((void**)&part, (size_t)nf * J * 2 * sizeof(double), s));
-    CK(cudaMallocAsync((void**)&dout, (size_t)nf * 4 * sizeof(double), s));
+    const size_t n_part = (size_t)nf * J * 2 * sizeof(double), n_out = (size_t)nf * 4 * sizeof(double);
+    Scratch w(s);
+    w.add(n_part);
+    w.add(n_out);
+    CK(w.get());
+    double* part = w.take<double>(n_part);
+    double* dout = w.take<double>(n_out);
     cudaError_t e = launch_moments(g, nf, J, N, part, dout, nullptr, 0, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, (size_t)nf * 4 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(part, s);
-    cudaFreeAsync(dout, s);
     return from_cuda(e);
 }
 
@@ -407,13 +491,14 @@ smc_status smc_ml_from_groups(const double* a, int J, double* log_ml, double* ns
 {
     if (!a || J < 2) return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    double* dout = nullptr;
-    CK(cudaMallocAsync((void**)&dout, 3 * sizeof(double), s));
+    Scratch w(s);
+    w.add(3 * sizeof(double));
+    CK(w.get());
+    double* dout = w.take<double>(3 * sizeof(double));
     cudaError_t e = launch_ml(a, J, nullptr, dout, s);
     double h[3] = {0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, dout, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFreeAsync(dout, s);
     if (log_ml) *log_ml = h[0];
     if (nse) *nse = h[1];
     return from_cuda(e);

@@ -134,6 +134,7 @@ def _declare(L):
     L.smc_last_error.restype = C.c_char_p
     L.smc_status_str.argtypes = [C.c_int]
     L.smc_status_str.restype = C.c_char_p
+    L.smc_release_workspace.argtypes = []
     L.smc_loglik.argtypes = [P(smc_model), C.c_int, vp, C.c_int, vp, C.c_int, vp, vp, vp, vp]
     L.smc_linreg_width.argtypes = [C.c_int]
     L.smc_linreg_width.restype = C.c_int
@@ -531,6 +532,12 @@ def draw_prior(model, seed, P, stream=None):
 # ------------------------------------------------ stateless (torch device buffers)
 def _ptr(t):
     return C.c_void_p(t.data_ptr()) if t is not None else None
+
+
+def release_workspace():
+    """Give back the memory that the stateless calls keep for the next one
+    (smc_release_workspace; at most 512 MiB per device)."""
+    _check(lib().smc_release_workspace())
 
 
 def linreg_width(p):
