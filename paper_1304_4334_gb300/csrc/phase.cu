@@ -725,9 +725,15 @@ constexpr int kSearchWarps = kSearchThreads / 32;
 constexpr int kCand = 32;
 constexpr float kFixScale = 68719476736.0f;       // 2^36
 
+// Up to kSoloTiles tiles one block runs the search alone, with block barriers
+// in the place of grid barriers and global totals (about 4 us a pass): 32 ->
+// 12 us at 1,024 particles; at 4,096 both take the same.
+constexpr int kSoloTiles = 64;
+
 int search_grid(int P)
 {
     const int tiles = (P + 31) / 32;
+    if (tiles <= kSoloTiles) return 1;
     const int by = (tiles + kSearchWarps - 1) / kSearchWarps;
     const int cap = device_sm_count();
     return by < 1 ? 1 : (by < cap ? by : cap);
@@ -895,21 +901,24 @@ __global__ void __launch_bounds__(kSearchThreads, 1) k_power_search(const double
     km = warp_max_key(km);
     if (lane == 0) skey[warp] = km;
     __syncthreads();
-    if (warp == 0) {
-        long long k = lane < kSearchWarps ? skey[lane] : kNegInfKey;
-        k = warp_max_key(k);
-        if (lane == 0) sc.bkey[blockIdx.x] = k;
+    const bool solo = G == 1;
+    if (!solo) {
+        if (warp == 0) {
+            long long k = lane < kSearchWarps ? skey[lane] : kNegInfKey;
+            k = warp_max_key(k);
+            if (lane == 0) sc.bkey[blockIdx.x] = k;
+        }
+        if (!grid_barrier(sc.bar, G, gen)) {
+            if (threadIdx.x == 0) raise_error(&ctl->err, kErrTimeout);
+            return;
+        }
+        // every block reads the G block maxima, one per thread (G <= SMs)
+        long long kb = (int)threadIdx.x < G ? __ldcg(sc.bkey + threadIdx.x) : kNegInfKey;
+        kb = warp_max_key(kb);
+        if (lane == 0) skey[warp] = kb;
+        __syncthreads();
     }
-    if (!grid_barrier(sc.bar, G, gen)) {
-        if (threadIdx.x == 0) raise_error(&ctl->err, kErrTimeout);
-        return;
-    }
-    // every block reads the G block maxima, one per thread (G <= SMs)
-    long long kg = (int)threadIdx.x < G ? __ldcg(sc.bkey + threadIdx.x) : kNegInfKey;
-    kg = warp_max_key(kg);
-    if (lane == 0) skey[warp] = kg;
-    __syncthreads();
-    kg = warp_max_key(lane < kSearchWarps ? skey[lane] : kNegInfKey);
+    const long long kg = warp_max_key(lane < kSearchWarps ? skey[lane] : kNegInfKey);
     const double llmax = key_value(kg);
 
     // ---- shifted FP32 log likelihoods x_n = l_n - max l (-inf past P) ----
@@ -949,6 +958,8 @@ __global__ void __launch_bounds__(kSearchThreads, 1) k_power_search(const double
             const double cv = candidate(lo, hi, lane);
             scand[lane] = cv;
             sdc[lane] = fmaxf((float)(cv * kLog2e), 1e-30f);
+        } else if (solo && threadIdx.x - 32 < 2 * kCand) {
+            sacc[threadIdx.x - 32] = 0ull;   // (read before the barrier that ended the last pass)
         }
         __syncthreads();
         const float dc = sdc[lane];
@@ -988,20 +999,28 @@ __global__ void __launch_bounds__(kSearchThreads, 1) k_power_search(const double
         atomicAdd(&sacc[lane], q1);
         atomicAdd(&sacc[kCand + lane], q2);
         __syncthreads();
-        if (threadIdx.x < 2 * kCand) {
-            atomicAdd(&sc.acc[slot * 2 * kCand + threadIdx.x], sacc[threadIdx.x]);
-            sacc[threadIdx.x] = 0ull;
-        } else if (blockIdx.x == 0 && threadIdx.x < 4 * kCand) {
-            // the slot of the next pass was last read before the previous barrier
-            sc.acc[((p + 1) % 3) * 2 * kCand + threadIdx.x - 2 * kCand] = 0ull;
-        }
-        if (!grid_barrier(sc.bar, G, gen)) {
-            if (threadIdx.x == 0) raise_error(&ctl->err, kErrTimeout);
-            return;
+        unsigned long long t1, t2;   // the totals of candidate `lane`
+        if (solo) {
+            t1 = sacc[lane];
+            t2 = sacc[kCand + lane];
+        } else {
+            if (threadIdx.x < 2 * kCand) {
+                atomicAdd(&sc.acc[slot * 2 * kCand + threadIdx.x], sacc[threadIdx.x]);
+                sacc[threadIdx.x] = 0ull;
+            } else if (blockIdx.x == 0 && threadIdx.x < 4 * kCand) {
+                // the slot of the next pass was last read before the previous barrier
+                sc.acc[((p + 1) % 3) * 2 * kCand + threadIdx.x - 2 * kCand] = 0ull;
+            }
+            if (!grid_barrier(sc.bar, G, gen)) {
+                if (threadIdx.x == 0) raise_error(&ctl->err, kErrTimeout);
+                return;
+            }
+            t1 = __ldcg(sc.acc + slot * 2 * kCand + lane);
+            t2 = __ldcg(sc.acc + slot * 2 * kCand + kCand + lane);
         }
         // every warp takes the same decision from the same totals
-        const float q1s = u64_to_f32(__ldcg(sc.acc + slot * 2 * kCand + lane)) * 2.3283064365386963e-10f;
-        const float q2s = u64_to_f32(__ldcg(sc.acc + slot * 2 * kCand + kCand + lane)) * 2.3283064365386963e-10f;
+        const float q1s = u64_to_f32(t1) * 2.3283064365386963e-10f;
+        const float q2s = u64_to_f32(t2) * 2.3283064365386963e-10f;
         const unsigned below = __ballot_sync(0xffffffffu, q1s * q1s < cmp * q2s);
         if (below == 0u) {
             // RSS stays >= D1 up to hi: in the first pass this takes the whole
@@ -1259,7 +1278,8 @@ __global__ void __launch_bounds__(kSelThreads) k_select(SelectArgs a)
     const size_t base = (size_t)j * N;
     const int tid = threadIdx.x;
     if (tid == 0) bad = 0;
-    if (a.mode != 2 && tid < 256) tab[tid] = g_exp2_neg256[tid];
+    if (a.mode != 2)
+        for (int i = tid; i < 256; i += blockDim.x) tab[i] = g_exp2_neg256[i];
 
     // ---- weights ----
     // Maxima as order-preserving integer keys and the two weight sums as
@@ -1317,6 +1337,7 @@ __global__ void __launch_bounds__(kSelThreads) k_select(SelectArgs a)
             a.gstat[3 * j + 1] = s1;
             a.gstat[3 * j + 2] = s2;
         }
+        if (a.stats_only) return;
         wmax = lmax == -INFINITY ? 0.0 : 1.0;
     }
     if (!(wmax > 0.0) || !isfinite(wmax)) {
@@ -1430,6 +1451,12 @@ __global__ void __launch_bounds__(kSelThreads) k_select(SelectArgs a)
     if (tid == 0 && bad) raise_error(a.err, kErrBounds);
 }
 
+// A block's time is its scans and barriers: fewer warps shorten both while a
+// thread has few particles to walk.  Whole smc_resample_logw calls with 256,
+// 512 and 1,024 threads: 47.8 / 51.1 / 50.9 us at 4 x 512, 59.2 / 62.6 / 60.7
+// at 4 x 2,048, 73.0 / 68.9 / 72.3 at 16 x 4,096, 110 / 91 / 86.5 at 128 x 8,192.
+static int select_threads(int N) { return N <= 2048 ? 256 : (N <= 4096 ? 512 : kSelThreads); }
+
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t s)
 {
     const size_t sm = select_smem(a.N);
@@ -1439,7 +1466,7 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t s)
                              (int)select_smem(kMaxN));
         attr = true;
     }
-    k_select<<<a.J, kSelThreads, sm, s>>>(a);
+    k_select<<<a.J, select_threads(a.N), sm, s>>>(a);
     count_launch();
     return cudaGetLastError();
 }

@@ -99,6 +99,7 @@ struct SelectArgs {
     int32_t* idx;     // [J*N]
     Ctl* ctl;
     int* err;
+    int stats_only;   // modes 0, 1: gstat, lw and a only (no resampling, idx untouched)
 };
 size_t select_smem(int N);
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t s);

@@ -354,25 +354,23 @@ smc_status smc_power_search(const double* ll, int P, double phi, double d1, int 
     if (!ll || P < 1 || !(phi >= 0.0 && phi < 1.0) || !(d1 > 0.0 && d1 < 1.0) || passes < 1)
         return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t n_part = search_part_len(P) * sizeof(double), n_idx = (size_t)P * sizeof(int32_t);
+    const size_t n_part = search_part_len(P) * sizeof(double);
+    struct Out {
+        Ctl ctl;
+        double gstat[3], lw, a;
+    };
     Scratch w(s);
     w.add(n_part);
-    w.add(sizeof(Ctl));
-    for (int i = 0; i < 3; ++i) w.add(3 * sizeof(double));   // gstat, lw, a
-    w.add(n_idx);
+    w.add(sizeof(Out));
     CK(w.get());
     double* part = w.take<double>(n_part);
-    Ctl* ctl = w.take<Ctl>(sizeof(Ctl));
-    double* gstat = w.take<double>(3 * sizeof(double));
-    double* lw = w.take<double>(3 * sizeof(double));
-    double* a = w.take<double>(3 * sizeof(double));
-    int32_t* idx = w.take<int32_t>(n_idx);
+    Out* out = w.take<Out>(sizeof(Out));
     CK(cudaMemsetAsync(part, 0, search_bar_bytes(), s));
-    Ctl init;
-    std::memset(&init, 0, sizeof init);
-    init.phi = phi;
-    cudaError_t e = cudaMemcpyAsync(ctl, &init, sizeof init, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_power_search(ll, P, d1, passes, part, ctl, s);
+    Out h;
+    std::memset(&h, 0, sizeof h);
+    h.ctl.phi = phi;
+    cudaError_t e = cudaMemcpyAsync(out, &h, sizeof h, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = launch_power_search(ll, P, d1, passes, part, &out->ctl, s);
     // FP64 RSS at the chosen power: the weights pass of the S phase over one
     // group holding all particles gives (max, sum w, sum w^2).
     if (e == cudaSuccess && P <= SMC_MAX_N) {
@@ -382,22 +380,18 @@ smc_status smc_power_search(const double* ll, int P, double phi, double d1, int 
         sa.ll = ll;
         sa.J = 1;
         sa.N = P;
-        sa.scheme = 0;
-        sa.a = a;
-        sa.lw = lw;
-        sa.gstat = gstat;
-        sa.idx = idx;
-        sa.ctl = ctl;
-        CK(cudaMemsetAsync(a, 0, sizeof(double), s));
+        sa.a = &out->a;
+        sa.lw = &out->lw;
+        sa.gstat = out->gstat;
+        sa.ctl = &out->ctl;
+        sa.stats_only = 1;
         e = launch_select(sa, s);
-        if (e == cudaSuccess) e = launch_cycle_close(gstat, lw, 1, P, 0, ctl, s);
     }
-    Ctl h;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, out, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) {
-        if (dphi) *dphi = h.dphi;
-        if (rss) *rss = P <= SMC_MAX_N ? h.rss : NAN;
+        if (dphi) *dphi = h.ctl.dphi;
+        if (rss) *rss = P <= SMC_MAX_N ? h.gstat[1] * h.gstat[1] / ((double)P * h.gstat[2]) : NAN;
     }
     return from_cuda(e);
 }

@@ -578,3 +578,20 @@ def test_covariance_block_shapes_match_numpy(S, d, P):
     if P > 4 * d:
         Lh = host(L)
         assert np.abs(Lh @ Lh.T - 0.25 * want).max() <= 2 * tol
+
+
+@pytest.mark.parametrize("P", [1, 31, 33, 511, 2047, 2048, 2049, 8192])
+def test_power_search_one_block_and_grid(S, P):
+    """Sizes on both sides of the single-block search, with dead particles:
+    the increment within the k-ary resolution of the RSS = D1 point (as the
+    oracle's bisection gives it, 1e-4), the FP64 RSS at it to 1e-11."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(P)
+    ll = 1000.0 - 40.0 * rng.chisquare(5, size=P)
+    if P > 4:
+        ll[rng.integers(0, P, P // 5)] = -np.inf
+    dphi, rss = S.power_search(dev(ll), 0.25)
+    d_o, _ = O.power_search(ll, 0.25, 0.5)
+    assert abs(dphi - d_o) <= 1e-4 * d_o + 1e-12, (dphi, d_o)
+    w = np.exp(dphi * (ll - ll.max()))
+    np.testing.assert_allclose(rss, w.sum() ** 2 / (P * (w ** 2).sum()), rtol=1e-11)
