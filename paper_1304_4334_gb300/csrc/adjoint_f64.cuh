@@ -51,19 +51,8 @@ struct AdjointF64 {
                 else fx.state_out(st, kLn2);
 #pragma unroll
                 for (int k = 0; k <= K; ++k) c[k * P] = st[k];
-                fx.template chain<false>(y[t0], mdl.tab);
-            } else {
-                fx.template chain<true>(y[0], mdl.tab);
             }
-            for (int r = 1; r < n; ++r) {
-                const uint64_t E = fx.E;
-                const int32_t neg = fx.neg;
-                fx.template chain<false>(y[t0 + r], mdl.tab);
-                fx.mix(E, neg, mdl.tab);
-                if ((r & 7) == 7) fx.flush();
-            }
-            fx.mix(fx.E, fx.neg, mdl.tab);
-            fx.flush();
+            fx.block(y + t0, n, t0 == 0, mdl.tab);
             mdl.close(fx, y + t0, t0, n, T);
         }
         if (!mdl.out) mdl.fx.restore(mdl.saved);
@@ -201,12 +190,18 @@ struct AdjointF64 {
             }
             bool ok = fixed && (sg == 0 || fx.enter(vprev, eprev));
             fx.bad = 0;
-            for (int r = 0; r < n; ++r) {
-                if (t0 + r == 0) fx.template chain<true>(y[0], mdl.tab);
-                else fx.template chain<false>(y[t0 + r], mdl.tab);
+            auto keep = [&](int r) {
                 double s[K + 1];
                 fx.state_out(s, kLn2);
                 put(buf + (size_t)r * W * stride, stride, s, s[K], fx.inv_h());
+            };
+            if (t0 == 0) fx.template chain<true>(y[0], mdl.tab);
+            else fx.template chain<false>(y[t0], mdl.tab);
+            keep(0);
+#pragma unroll 2
+            for (int r = 1; r < n; ++r) {
+                fx.template chain<false>(y[t0 + r], mdl.tab);
+                keep(r);
             }
             ok = ok && fx.bad == 0u;
             if (!ok) segment_f64(y, t0, n, vprev, eprev, buf, stride);

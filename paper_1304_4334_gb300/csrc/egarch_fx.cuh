@@ -108,22 +108,25 @@ SMC_FX uint64_t fx_mulhi(uint64_t a, uint64_t b)
 }
 
 // 2^-x for x = n + X 2^-55 (the low 55 bits of X used): M 2^-63, M in (2^62, 2^63];
-// tab[j] = round(2^(63 - j/256)).  With r = rho 2^-8 the fraction below the
+// tab[j] = round(2^(63 - j/256)), M = tab[j] 2^-r.  With r = rho 2^-8 the fraction below the
 // table's, 2^-r = 1 - rho (k1 - rho (k2 - rho (k3 - rho (k4 - rho k5)))),
 // k_i = ln2^i / i! 2^-8i; k5, k4 in units of 2^-64, k3 of 2^-60, k2 and k1 of
 // 2^-72: each level carries the bits that reach the result, and one shift
 // at the end puts the sum into the table's units.
-SMC_FX uint64_t fx_exp2neg(uint64_t X, const uint64_t* tab)
+SMC_FX uint64_t fx_exp2neg_q(uint64_t X)   // 1 - 2^-r in units of 2^-72
 {
-    const uint64_t T = tab[(uint32_t)(X >> 47) & 255u];
     const uint64_t R = X << 17;
     const uint32_t rho = (uint32_t)(R >> 32);
     const uint32_t t4 = kFxC4 - fx_mulhi32(rho, kFxC5);
     const uint32_t t3 = kFxC3 - (fx_mulhi32(rho, t4) >> 4);
     const uint64_t t2 = kFxC2 - (((uint64_t)rho * t3) >> 20);
     const uint64_t t1 = kFxC1 - fx_mulhi(R, t2);
-    const uint64_t q = fx_mulhi(R, t1);
-    return T - (fx_mulhi(T, q) >> 8);
+    return fx_mulhi(R, t1);
+}
+SMC_FX uint64_t fx_exp2neg(uint64_t X, const uint64_t* tab)
+{
+    const uint64_t T = tab[(uint32_t)(X >> 47) & 255u];
+    return T - (fx_mulhi(T, fx_exp2neg_q(X)) >> 8);
 }
 
 SMC_FX int64_t fx_round(double x)   // nearest integer (|x| < 2^62)
@@ -197,20 +200,31 @@ SMC_FX uint64_t fx_rcp(uint64_t s)
     return Y;
 }
 
-// e^-x in FP64 without FP64 instructions for |x| < 128 (within a unit in the
-// last place); the library's exponential beyond.
+// e^-x in FP64 without FP64 instructions for |x| < 700: within a unit in the
+// last place for |x| < 128, within 2^-51 beyond, where x itself, a rounded
+// FP64 sum, is known to 2^-46 at best; the library's exponential where the
+// result leaves the normal range, and its limits past that.
 SMC_FX double fx_exp_neg(double x, const uint64_t* tab)
 {
-    uint64_t X;
-    if (!fx_fixed56(x, X)) {
-        // beyond the exponent range the result is 0 or inf (a NaN stays one)
-        if (std::fabs(x) >= 1024.0) return x > 0.0 ? 0.0 : INFINITY;
-        return fx_exp_library(-x);
-    }
-    X = fx_mulhi(X, kFxLog2e);
     const uint64_t sg = (uint64_t)((int64_t)fx_bits(x) >> 63);
-    X = (X ^ sg) - sg;
-    return fx_pack(fx_exp2neg(X, tab), (int)((int64_t)X >> 55));
+    uint64_t X;
+    int n;
+    if (fx_fixed56(x, X)) {
+        X = fx_mulhi(X, kFxLog2e);
+        X = (X ^ sg) - sg;
+        n = (int)((int64_t)X >> 55);
+    } else if (std::fabs(x) < 700.0) {
+        const uint64_t b = fx_bits(x);                // units of 2^-53, then 2^-52
+        X = fx_mulhi(((b << 11) | 0x8000000000000000ull) >> (1033 - ((int)(b >> 52) & 0x7ff)), kFxLog2e);
+        X = (X ^ sg) - sg;
+        n = (int)((int64_t)X >> 52);
+        X <<= 3;
+    } else if (std::fabs(x) < 1024.0) {
+        return fx_exp_library(-x);
+    } else {
+        return x > 0.0 ? 0.0 : (x < 0.0 ? INFINITY : x);   // (a NaN stays one)
+    }
+    return fx_pack(fx_exp2neg(X, tab), n);            // e^-x = M 2^(-63 - n)
 }
 
 // Product of the mixture sums s (units 2^-61, in [1, 4]): pm 2^(pe - 62) with
@@ -371,7 +385,8 @@ struct EgarchFx {
             const int64_t S = (int64_t)cl * eh + ((int64_t)ch * el + (int64_t)nf[k]);
             const int32_t vh = (int32_t)(V[k] >> 30), vl = (int32_t)((uint32_t)V[k] & 0x3fffffffu);
             const int64_t Q = (int64_t)al[k] * vh + ((int64_t)ah[k] * vl + (int64_t)na[k]);
-            V[k] = ((int64_t)ah[k] * vh + ((int64_t)ch * eh + (S >> 29))) + (Q >> 30) + (nb[k] - V[k]);
+            const int64_t off = ((int64_t)ah[k] * vh + (Q >> 30)) + (nb[k] - V[k]);   // (before the shock is known)
+            V[k] = ((int64_t)ch * eh + off) + (S >> 29);
         }
     }
 
@@ -393,13 +408,15 @@ struct EgarchFx {
             bad |= ((uint32_t)((uint64_t)V[k] >> 32) + (kVmax << 23)) & ~(uint32_t)((kVmax << 24) - 1);
         }
         sx += X;
-        M = fx_exp2neg(X, tab);
+        const uint64_t T = tab[(uint32_t)(X >> 47) & 255u], q = fx_exp2neg_q(X);
+        M = T - (fx_mulhi(T, q) >> 8);   // (only where inv_h() is used)
         // |eps| = |y - mu| 2^-X: the 53-bit significand times M, shifted; the
         // shift passes 63 for a zero return
         const double dy = y - mu;
         const uint64_t b = fx_bits(dy);
         const int ed = (int)(uint32_t)(b >> 52) & 0x7ff;
-        const uint64_t prod = fx_mulhi((b << 11) | 0x8000000000000000ull, M);
+        const uint64_t p0 = fx_mulhi((b << 11) | 0x8000000000000000ull, T);   // beside the polynomial
+        const uint64_t prod = p0 - (fx_mulhi(p0, q) >> 8);
         const int sh = (1032 - 256) + (int)(uint32_t)(X >> 55) - ed;
         bad |= (uint32_t)(sh - 3 - cs) & 0x80000000u;   // |eps| 2^cs < 128
         E = fx_shr(prod, sh);
@@ -504,7 +521,38 @@ struct EgarchFx {
         fx_product(pm, pe, s);
     }
 
-    // At least every 8 observations (E < 2^60: hl and |s1| stay below 2^63).
+    // One step of block(): the chain of an observation and the mixture part of
+    // the one before, which do not depend on each other.
+    SMC_FX void step(double y, const uint64_t* tab)
+    {
+        const uint64_t E0 = E;
+        const int32_t neg0 = neg;
+        chain<false>(y, tab);
+        mix(E0, neg0, tab);
+    }
+
+    // n observations (first: they open the series), sums flushed.  Eight steps
+    // between flushes without a test in between, unrolled by two: the pieces
+    // of two steps interleave (K=3, I=4, one warp per scheduler: MEASURED_BLK
+    // cycles an observation; by three or four it is slower again).
+    SMC_FX void block(const double* y, int n, bool first, const uint64_t* tab)
+    {
+        if (first) chain<true>(y[0], tab);
+        else chain<false>(y[0], tab);
+        int r = 1;
+        for (; r + 8 <= n; r += 8) {
+#pragma unroll 2
+            for (int u = 0; u < 8; ++u) step(y[r + u], tab);
+            flush();
+        }
+#pragma unroll 2
+        for (; r < n; ++r) step(y[r], tab);
+        mix(E, neg, tab);
+        flush();
+    }
+
+    // At least every 8 observations (9 of chain(): E < 2^60, so hl stays below
+    // 2^64 and |s1| below 2^63).
     SMC_FX void flush()
     {
         s2 += ((unsigned __int128)hh << 42) + ((unsigned __int128)hl << 12) + (ll >> 12);

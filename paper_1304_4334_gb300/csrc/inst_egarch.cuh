@@ -18,8 +18,7 @@ struct MutateKernel {
     static void (*pick(int))(MutateArgs) { return k_mutate<Pol>; }
 };
 template <class Pol>
-struct MutateKernel<Pol, std::enable_if_t<!std::is_same_v<typename Pol::Wide, Pol> && (Pol::kMinBlocks > 1) &&
-                                          (Pol::kNi > 2)>> {
+struct MutateKernel<Pol, std::enable_if_t<!std::is_same_v<typename Pol::Wide, Pol> && (Pol::kNi > 1)>> {
     static void (*pick(int P))(MutateArgs)
     {
         return P <= kWideWarpsPerSm * 32 * device_sm_count() ? k_mutate<typename Pol::Wide> : k_mutate<Pol>;

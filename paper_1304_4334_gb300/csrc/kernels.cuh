@@ -180,12 +180,12 @@ struct PolicyEgarchF32Delta : PolicyEgarchF32T<K, I, true> {};
 // stand-alone likelihood), the FP64 recursion observation by observation
 // (PolicyEgarchF64: data-tempering C phase).
 // kWide: no register cap.  Two blocks of 224 per SM (128 registers) are faster
-// where the particles fill them (K=3, I=4, 65,536 x 2,000: 4.0 ms against
-// 5.0 ms with 187 registers; K=I=1: 0.96 against 1.01 ms), except at I = 2
-// (2.21 against 2.18 ms); with at most 10 warps per SM the kernel is bound by
-// each warp's own latency and the spills cost (K=3, I=4, 10,007 particles:
-// 2.10 ms against 1.88 ms).
-template <int K, int I, bool kWide = (I == 2)>
+// where the particles fill them (65,536 x 2,000: K=3, I=4 4.0 ms against 4.3 ms
+// with 255 registers, K=2, I=3 2.83 against 3.53 ms; K=2, I=2, x 5,000: 5.14
+// against 6.06 ms); with at most 10 warps per SM the kernel is bound by each
+// warp's own latency and the spills cost (K=3, I=4: 10,007 particles 1.98 ms
+// against 1.53 ms, 30,000 2.49 against 2.13 ms).
+template <int K, int I, bool kWide = false>
 struct PolicyEgarchF64FxT {
     using Real = double;
     using Obs = double;

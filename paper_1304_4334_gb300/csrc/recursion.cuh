@@ -1086,20 +1086,8 @@ __device__ __forceinline__ bool run_egarch_f64(EgarchFxSafe<K, I>& mdl, ObsPipe<
         const double* yb = pipe.buf + (c & 1) * kChunkF64;
         const int cnt = min(kChunkF64, T - c * kChunkF64);
         for (int r0 = 0; r0 < cnt; r0 += 32) {
-            // 32 observations; the mixture part of one runs beside the chain
-            // of the next (they do not depend on each other)
             const int e = min(cnt, r0 + 32);
-            if (c == 0 && r0 == 0) fx.template chain<true>(yb[0], mdl.tab);
-            else fx.template chain<false>(yb[r0], mdl.tab);
-            for (int r = r0 + 1; r < e; ++r) {
-                const uint64_t E = fx.E;
-                const int32_t neg = fx.neg;
-                fx.template chain<false>(yb[r], mdl.tab);
-                fx.mix(E, neg, mdl.tab);
-                if ((r & 7) == 7) fx.flush();
-            }
-            fx.mix(fx.E, fx.neg, mdl.tab);
-            fx.flush();
+            fx.block(yb + r0, e - r0, c == 0 && r0 == 0, mdl.tab);
             mdl.close(fx, yb + r0, c * kChunkF64 + r0, e - r0, T);
         }
         pipe.release(c);
