@@ -14,15 +14,15 @@ inline int mutate_grid(int P, int threads = kMutThreads) { return (P + threads -
 // The kernel variant for P particles (one per thread): the policy's Wide form,
 // where it has one, while the particles leave the SMs room for it.
 template <class Pol, class = void>
-struct MutateKernel {
-    static void (*pick(int))(MutateArgs) { return k_mutate<Pol>; }
+struct KernelPick {
+    static void (*mutate(int))(MutateArgs) { return k_mutate<Pol>; }
+    static void (*loglik(int))(LoglikArgs) { return k_loglik<Pol>; }
 };
 template <class Pol>
-struct MutateKernel<Pol, std::enable_if_t<!std::is_same_v<typename Pol::Wide, Pol> && (Pol::kNi > 1)>> {
-    static void (*pick(int P))(MutateArgs)
-    {
-        return P <= kWideWarpsPerSm * 32 * device_sm_count() ? k_mutate<typename Pol::Wide> : k_mutate<Pol>;
-    }
+struct KernelPick<Pol, std::enable_if_t<!std::is_same_v<typename Pol::Wide, Pol> && (Pol::kNi > 1)>> {
+    static bool wide(int P) { return P <= kWideWarpsPerSm * 32 * device_sm_count(); }
+    static void (*mutate(int P))(MutateArgs) { return wide(P) ? k_mutate<typename Pol::Wide> : k_mutate<Pol>; }
+    static void (*loglik(int P))(LoglikArgs) { return wide(P) ? k_loglik<typename Pol::Wide> : k_loglik<Pol>; }
 };
 
 // One particle per thread; threads = a multiple of 32 up to kMutMaxThreads (the caller checks).
@@ -42,10 +42,10 @@ cudaError_t launch_mutate_k(const MutateArgs& a, int threads, cudaStream_t s)
     }
     void (*k)(MutateArgs) = nullptr;
     switch (a.m.I) {
-    case 1: k = MutateKernel<Pol<K, 1>>::pick(a.P); break;
-    case 2: k = MutateKernel<Pol<K, 2>>::pick(a.P); break;
-    case 3: k = MutateKernel<Pol<K, 3>>::pick(a.P); break;
-    case 4: k = MutateKernel<Pol<K, 4>>::pick(a.P); break;
+    case 1: k = KernelPick<Pol<K, 1>>::mutate(a.P); break;
+    case 2: k = KernelPick<Pol<K, 2>>::mutate(a.P); break;
+    case 3: k = KernelPick<Pol<K, 3>>::mutate(a.P); break;
+    case 4: k = KernelPick<Pol<K, 4>>::mutate(a.P); break;
     default: return cudaErrorInvalidValue;
     }
     if (a.dependent) return pdl_launch(k, g, threads, 0, s, a);
@@ -74,14 +74,15 @@ cudaError_t launch_mutate_x2_k(const MutateArgs& a, int threads, cudaStream_t s)
 template <template <int, int> class Pol, int K>
 cudaError_t launch_loglik_k(const LoglikArgs& a, cudaStream_t s)
 {
-    const int g = mutate_grid(a.P);
+    void (*k)(LoglikArgs) = nullptr;
     switch (a.m.I) {
-    case 1: k_loglik<Pol<K, 1>><<<g, kMutThreads, 0, s>>>(a); break;
-    case 2: k_loglik<Pol<K, 2>><<<g, kMutThreads, 0, s>>>(a); break;
-    case 3: k_loglik<Pol<K, 3>><<<g, kMutThreads, 0, s>>>(a); break;
-    case 4: k_loglik<Pol<K, 4>><<<g, kMutThreads, 0, s>>>(a); break;
+    case 1: k = KernelPick<Pol<K, 1>>::loglik(a.P); break;
+    case 2: k = KernelPick<Pol<K, 2>>::loglik(a.P); break;
+    case 3: k = KernelPick<Pol<K, 3>>::loglik(a.P); break;
+    case 4: k = KernelPick<Pol<K, 4>>::loglik(a.P); break;
     default: return cudaErrorInvalidValue;
     }
+    k<<<mutate_grid(a.P), kMutThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -139,7 +139,7 @@ struct PolicyEgarchF32T {
     using Model = EgarchF32<K, I, kDelta>;
     static constexpr int kNs = K + 1;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;   // Table 1
-    static constexpr int kBound = I == 1 ? 256 : kMutMaxThreads, kMinBlocks = 0;
+    static constexpr int kBound = I == 1 ? 256 : kMutMaxThreads, kMinBlocks = 0, kLoglikBlocks = 0;
     static constexpr bool kExpTab = false;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* = nullptr)
     {
@@ -194,6 +194,7 @@ struct PolicyEgarchF64FxT {
     static constexpr int kNs = K + 1, kNi = I;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;
     static constexpr int kBound = kMutMaxThreads, kMinBlocks = kWide ? 0 : 2;   // (0: no minimum)
+    static constexpr int kLoglikBlocks = kWide ? 1 : 4;
     static constexpr bool kExpTab = true;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* tab)
     {
@@ -242,7 +243,7 @@ struct PolicyLinreg {
     using Model = LinregF64;
     static constexpr int kNs = 0;
     static constexpr int kMaxFree = 8;
-    static constexpr int kBound = 256, kMinBlocks = 0;
+    static constexpr int kBound = 256, kMinBlocks = 0, kLoglikBlocks = 0;
     static constexpr bool kExpTab = false;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t*)
     {
@@ -496,7 +497,7 @@ __global__ void __launch_bounds__(kMutMaxThreads) k_mutate_x2(MutateArgs a)
 }
 
 template <class Pol>
-__global__ void __launch_bounds__(kMutThreads) k_loglik(LoglikArgs a)
+__global__ void __launch_bounds__(kMutThreads, Pol::kLoglikBlocks) k_loglik(LoglikArgs a)
 {
     using Real = typename Pol::Real;
     using Obs = typename Pol::Obs;
