@@ -21,6 +21,65 @@
 
 namespace smc {
 
+// Gradient with respect to the full theta vector (Table 1 layout) from the
+// natural parameters' (mu, log sigma, alpha, beta, gamma, log p_i, mu_i, a_i):
+// the transforms and the mixture's normalisation taken backwards,
+//   p_i = P_i / S,  m = sum p_i M_i,  V = sum p_i ((M_i - m)^2 + s_i^2),  c = V^-1/2,
+//   mu_i = c (M_i - m),  1 / a_i = c s_i
+// (about 15 FP64 instructions per component; forward-mode duals along each of
+// the 3 I directions made the K=2, I=2 gradient of 4,096 particles 36 us
+// longer, as long as some 60 observations).
+template <int K, int I>
+__device__ __forceinline__ void natural_to_theta_f64(const EgarchParams<double, K, I>& q, const double* gn,
+                                                     const double* th, int has_gamma, double* gth)
+{
+    int j = 0;
+    gth[j++] = gn[0] / 1000.0;
+    gth[j++] = gn[1];
+#pragma unroll
+    for (int k = 0; k < K; ++k) gth[j++] = gn[2 + k] * (1.0 - q.alpha[k] * q.alpha[k]);
+#pragma unroll
+    for (int k = 0; k < K; ++k) gth[j++] = gn[2 + K + k] * q.beta[k];
+    if (has_gamma) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) gth[j++] = gn[2 + 2 * K + k];
+    }
+    if constexpr (I >= 2) {
+        const double* glp = gn + 2 + 3 * K;
+        const double* gmu = glp + I;
+        const double* ga = gmu + I;
+        double P[I], s[I], pb[I], m2b[I], S = 0.0;
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            P[i] = 2.0 / (1.0 + exp(-2.0 * th[j + i]));
+            s[i] = exp(th[j + 2 * I + i]);
+            S += P[i];
+        }
+        const double c = q.sig[0] / s[0], ic = 1.0 / c, c2 = c * c;
+        double cb = 0.0;
+#pragma unroll
+        for (int i = 0; i < I; ++i) cb += gmu[i] * q.mu[i] - ga[i] / q.sig[i];   // c dL/dc
+        const double Vb = -0.5 * c2 * cb;                                            // dL/dV
+        double mb = 0.0, pp = 0.0;
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            const double m2 = q.mu[i] * ic;
+            m2b[i] = c * gmu[i] + 2.0 * Vb * q.p[i] * m2;
+            mb -= m2b[i];
+            pb[i] = glp[i] / q.p[i] + Vb * (m2 * m2 + s[i] * s[i]);
+            gth[j + 2 * I + i] = -ga[i] / q.sig[i] + 2.0 * Vb * q.p[i] * s[i] * s[i];
+        }
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            gth[j + I + i] = m2b[i] + mb * q.p[i];
+            pb[i] += mb * th[j + I + i];
+            pp += pb[i] * q.p[i];
+        }
+#pragma unroll
+        for (int i = 0; i < I; ++i) gth[j + i] = (pb[i] - pp) / S * (P[i] * (2.0 - P[i]));
+    }
+}
+
 template <int K, int I, int kSeg>
 struct AdjointF64 {
     EgarchFxSafe<K, I> mdl;

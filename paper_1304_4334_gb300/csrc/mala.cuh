@@ -106,7 +106,7 @@ struct GradEgarch {
             adj.setup(full, m.gamma, m.eps0_zero, tab);
             ll = adj.forward(y, T, (double*)ckpt, P, p, st);
             adj.reverse(y, T, (const double*)ckpt, P, p, buf, stride, gn);
-            natural_to_theta<Real, K, I>(adj.mdl.q.alpha, adj.mdl.q.beta, gn, full, m.gamma, gfull);
+            natural_to_theta_f64<K, I>(adj.mdl.q, gn, full, m.gamma, gfull);
         }
         if (m.has_free)
             for (int k = 0; k < m.d; ++k) g[k] = gfull[m.free_idx[k]];
