@@ -21,6 +21,21 @@
 
 namespace smc {
 
+struct GradArgs {
+    ModelDev m;
+    const void* obs;
+    int T, W;
+    const double* theta;   // [d][P]
+    int P;
+    double* ll;            // [P]
+    double* grad;          // [d][P] d log p(y|theta) / d theta (free parameters)
+    double* state;         // [K+1][P] (nullable)
+    void* ckpt;            // segment checkpoints (gradient policy's layout)
+    int by_size;           // the kernel may be chosen by P: the last bits of l and of the gradient
+                           // differ between them, so a run, whose particles do not depend on how
+                           // they are divided over launches, leaves it 0
+};
+
 // Gradient with respect to the full theta vector (Table 1 layout) from the
 // natural parameters' (mu, log sigma, alpha, beta, gamma, log p_i, mu_i, a_i):
 // the transforms and the mixture's normalisation taken backwards,
@@ -78,6 +93,31 @@ __device__ __forceinline__ void natural_to_theta_f64(const EgarchParams<double, 
 #pragma unroll
         for (int i = 0; i < I; ++i) gth[j + i] = (pb[i] - pp) / S * (P[i] * (2.0 - P[i]));
     }
+}
+
+// r_i (2^-59) with the terms x_i formed in FP64 (any parameters and shock);
+// returns log sum_i exp(x_i).
+template <int K, int I>
+__device__ __noinline__ double weights_f64(const EgarchParams<double, K, I>& q, double eps, const uint64_t* tab,
+                                           uint64_t* r)
+{
+    double x[I], mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+        const double z = (eps - q.mu[i]) / q.sig[i];
+        x[i] = log(q.p[i]) - log(q.sig[i]) - 0.5 * z * z;
+        mx = fmax(mx, x[i]);
+    }
+    uint64_t s = 0;
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+        r[i] = fx_exp_q61(mx - x[i], tab);
+        s += r[i];
+    }
+    const uint64_t Y = fx_rcp(s);
+#pragma unroll
+    for (int i = 0; i < I; ++i) r[i] = fx_mulhi(r[i], Y);
+    return isnan(eps) ? eps : mx + log((double)s * 0x1p-61);
 }
 
 template <int K, int I, int kSeg>
@@ -148,27 +188,6 @@ struct AdjointF64 {
         b[(K + 1) * stride] = inv;
     }
 
-    // r_i (2^-59) with the terms x_i formed in FP64 (any parameters and shock).
-    __device__ __noinline__ void weights_f64(double eps, uint64_t* r) const
-    {
-        double x[I], mx = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < I; ++i) {
-            const double z = (eps - mdl.q.mu[i]) / mdl.q.sig[i];
-            x[i] = log(mdl.q.p[i]) - log(mdl.q.sig[i]) - 0.5 * z * z;
-            mx = fmax(mx, x[i]);
-        }
-        uint64_t s = 0;
-#pragma unroll
-        for (int i = 0; i < I; ++i) {
-            r[i] = fx_exp_q61(mx - x[i], mdl.tab);
-            s += r[i];
-        }
-        const uint64_t Y = fx_rcp(s);
-#pragma unroll
-        for (int i = 0; i < I; ++i) r[i] = fx_mulhi(r[i], Y);
-    }
-
     // Reverse sweep; gn (EgarchNat<double, K, I>::kNp) receives d l / d natural
     // parameters.  buf: this thread's slab, [kSeg][v_1..v_K, eps, 1/h][stride].
     __device__ __forceinline__ void reverse(const double* __restrict__ y, int T, const double* ckpt, size_t P, int p,
@@ -203,7 +222,7 @@ struct AdjointF64 {
             double eb = -eps;
             if constexpr (I >= 2) {
                 uint64_t r[I];
-                if (!(fixed && fx.weights(eps, r, mdl.tab))) weights_f64(eps, r);
+                if (!(fixed && fx.weights(eps * 0x1p53, r, mdl.tab))) weights_f64(mdl.q, eps, mdl.tab, r);
                 eb = 0.0;
 #pragma unroll
                 for (int i = 0; i < I; ++i) {
@@ -306,6 +325,366 @@ struct AdjointF64 {
                 gn[NS + 2 * I + i] = q.sig[i] * r0 - a * (r2 - mu * (2.0 * r1 - mu * r0));
             }
         }
+    }
+};
+
+// ------------------------------------------- two warps per 32 particles
+// The same computation split over two warps for particles too few to fill the
+// SMs' schedulers (I >= 2): the first carries the volatility chain and the
+// adjoint carry, the second everything about the mixture, a segment behind.
+// A warp's own latency (about 4,000 cycles per observation in AdjointF64 at
+// K=2, I=2) is what bounds such a launch; the two halves run side by side.
+// Forward: warp 0 leaves each segment's shocks, warp 1 takes their mixture
+// densities.  Backward, at step j: warp 0 recomputes segment n-1-j and runs the
+// carry over segment n+1-j, warp 1 forms dl/deps and the component sums of
+// segment n-j.  Shocks are kept in units of 2^-53 and V_k in 2^-55, and the
+// sums scaled once at the end.
+// Measured at T=600, up to one block (of 32 particles) per SM, one warp ->
+// two: K=1,I=2 1,298 -> 703 us, K=2,I=2 1,441 -> 823 us, K=3,I=4 2,604 ->
+// 1,347 us, K=4,I=4 2,884 -> 1,364 us; with all the blocks an SM's shared
+// memory holds 1,358 -> 822, 1,495 -> 976, 2,723 -> 1,645 us.  Beyond that a
+// second wave would take what the split gains (k_loglik_grad then).
+template <int K, int I>
+struct GradSplit {
+    static constexpr int kSeg = 16, W = K + 2;
+    static constexpr double kVu = 0x1p55 * 0.5 / kLn2;   // V_k units of v_k
+    struct Smem {
+        double slab[3][kSeg][W][32];       // V_1..V_K, eps, 1/h
+        double x[2][kSeg][32];             // forward: shocks; backward: dl/deps 2^-53
+        double comb[3 * I + 2][32];        // warp 1's results
+        uint64_t tab[256];
+    };
+
+    // Both warps, each from its own place in the code.
+    __device__ __forceinline__ static void meet() { asm volatile("barrier.sync 1, 64;" ::: "memory"); }
+
+    // A segment of warp 0 in FP64: shocks out (and V, 1/h for the recomputation),
+    // log h summed; w carries the state.
+    __device__ __noinline__ static double segment_f64(EgarchF64<K, I>& w, double lsy, const double* __restrict__ y,
+                                                      int t0, int n, double* es, int es_stride, double* v, double* inv)
+    {
+        double sum = 0.0;
+        for (int r = 0; r < n; ++r) {
+            uint64_t s;
+            if (t0 + r == 0) w.template terms<true>(y[0], s);
+            else w.template terms<false>(y[t0 + r], s);
+            double vs = w.v[0];
+#pragma unroll
+            for (int k = 1; k < K; ++k) vs += w.v[k];
+            sum += lsy + 0.5 * vs;
+            es[(size_t)r * es_stride] = w.eps * 0x1p53;
+            if (v) {
+#pragma unroll
+                for (int k = 0; k < K; ++k) v[(size_t)r * es_stride + 32 * k] = w.v[k] * kVu;
+                inv[(size_t)r * es_stride] = fx_exp_neg(lsy + 0.5 * vs, w.tab);
+            }
+        }
+        return sum;
+    }
+
+    __device__ static void run(const GradArgs& a, Smem& sm)
+    {
+        const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+        for (int i = threadIdx.x; i < 256; i += blockDim.x) sm.tab[i] = g_exp2_neg256[i];
+        const int p = blockIdx.x * 32 + lane;
+        const bool active = p < a.P;
+        const int pp = active ? p : a.P - 1;
+        const size_t P = (size_t)a.P;
+        const int T = a.T, nseg = (T + kSeg - 1) / kSeg;
+        const double* __restrict__ y = (const double*)a.obs;
+        double* ckpt = (double*)a.ckpt;
+        double th[kMaxD], full[kMaxD];
+        for (int i = 0; i < a.m.d; ++i) th[i] = a.theta[i * P + pp];
+        full_theta<double>(a.m, th, full);
+        EgarchParams<double, K, I> q;
+        egarch_transform<double, K, I>(full, a.m.gamma, q);
+        EgarchFx<K, I> fx;
+        fx.setup(q.mu_y, q.log_sigma_y, q.alpha, q.beta, q.gamma, q.p, q.mu, q.sig, a.m.eps0_zero, kLog2e);
+        const bool fixed = fx.bad == 0u;
+        __syncthreads();
+        if (role == 0) chain_warp(a, sm, fx, q, fixed, lane, p, pp, active, full, y, ckpt, P, T, nseg);
+        else mixture_warp(sm, fx, q, fixed, lane, T, nseg);
+    }
+
+    __device__ __forceinline__ static void chain_warp(const GradArgs& a, Smem& sm, EgarchFx<K, I> fx,
+                                                      const EgarchParams<double, K, I>& q, bool fixed, int lane,
+                                                      int p, int pp, bool active, const double* full,
+                                                      const double* __restrict__ y, double* ckpt, size_t P, int T,
+                                                      int nseg)
+    {
+        EgarchF64<K, I> w;
+        w.setup(q, a.m.eps0_zero, sm.tab);
+        bool out = !fixed;
+        double st[K + 1], lh64 = 0.0;      // state at the segment's start; log h summed in FP64
+        int n64 = 0;
+        unsigned __int128 sx = 0;
+#pragma unroll
+        for (int k = 0; k <= K; ++k) st[k] = 0.0;
+        for (int sg = 0; sg <= nseg; ++sg) {
+            if (sg < nseg) {
+                const int t0 = sg * kSeg, n = min(kSeg, T - t0);
+                if (sg > 0) {
+                    double* c = ckpt + (size_t)(sg - 1) * (K + 1) * P + pp;
+                    if (active)
+#pragma unroll
+                        for (int k = 0; k <= K; ++k) c[k * P] = st[k];
+                }
+                double* es = &sm.x[sg & 1][0][lane];
+                fx.bad = 0;
+                fx.sx = 0;
+                if (t0 == 0) fx.template chain<true>(y[0], sm.tab);
+                else fx.template chain<false>(y[t0], sm.tab);
+                es[0] = (double)fx.shock();
+#pragma unroll 2
+                for (int r = 1; r < n; ++r) {
+                    fx.template chain<false>(y[t0 + r], sm.tab);
+                    es[r * 32] = (double)fx.shock();
+                }
+                if (fx.bad == 0u && !out) {
+                    sx += fx.sx;
+                    fx.state_out(st, kLn2);
+                } else {
+                    if (!out) w.load_state(st);
+                    lh64 += segment_f64(w, q.log_sigma_y, y, t0, n, es, 32, nullptr, nullptr);
+                    n64 += n;
+                    out = !(fixed && fx.enter(w.v, w.eps));
+                    w.state_out(st);
+                }
+            }
+            meet();
+        }
+        const double logh = lh64 + kLn2 * EgarchFx<K, I>::to_double((__int128)sx - ((__int128)(T - n64) << 63)) * 0x1p-55;
+        if (active && a.state)
+#pragma unroll
+            for (int k = 0; k <= K; ++k) a.state[k * P + p] = st[k];
+
+        constexpr int NS = 2 + 3 * K;
+        double gn[NS + 3 * I], gs[NS], vb[K], al[K], bp[K], bm[K], ga[K];
+#pragma unroll
+        for (int i = 0; i < NS; ++i) gn[i] = gs[i] = 0.0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            vb[k] = 0.0;                   // 2 dL/dv_k,t+1
+            al[k] = q.alpha[k];
+            ga[k] = q.gamma[k] * 0x1p-54;
+            bp[k] = (q.beta[k] + q.gamma[k]) * 0x1p-54;
+            bm[k] = (q.gamma[k] - q.beta[k]) * 0x1p-54;
+        }
+        auto carry = [&](double dle, double es, double inv, const double* vp, double ep, bool has_prev) {
+            double eb = dle;               // dL/deps 2^-53
+#pragma unroll
+            for (int k = 0; k < K; ++k) eb = fma(vb[k], es > 0.0 ? bp[k] : (es < 0.0 ? bm[k] : ga[k]), eb);
+            const double sb = fma(-eb, es, -1.0);
+            gs[0] = fma(-eb, inv, gs[0]);
+            gs[1] += sb;
+            const double ae = fabs(ep) - kSqrt2OverPi * 0x1p53;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                vb[k] = fma(al[k], vb[k], sb);
+                if (has_prev) {
+                    gs[2 + k] = fma(vb[k], vp[k], gs[2 + k]);
+                    gs[2 + K + k] = fma(vb[k], ae, gs[2 + K + k]);
+                    gs[2 + 2 * K + k] = fma(vb[k], ep, gs[2 + 2 * K + k]);
+                } else if (a.m.eps0_zero) {
+                    gs[2 + K + k] = fma(vb[k], -kSqrt2OverPi * 0x1p53, gs[2 + K + k]);
+                }
+            }
+        };
+        auto entering = [&](int sg, double* v, double& e) {   // the state entering segment sg
+            if (sg > 0) {
+                const double* c = ckpt + (size_t)(sg - 1) * (K + 1) * P + pp;
+#pragma unroll
+                for (int k = 0; k < K; ++k) v[k] = c[k * P];
+                e = c[K * P];
+            } else {
+#pragma unroll
+                for (int k = 0; k < K; ++k) v[k] = 0.0;
+                e = 0.0;
+            }
+        };
+        for (int j = 0; j < nseg + 2; ++j) {
+            if (j < nseg) {                // recompute segment nseg - 1 - j
+                const int sg = nseg - 1 - j, t0 = sg * kSeg, n = min(kSeg, T - t0);
+                double v0[K], e0;
+                entering(sg, v0, e0);
+                bool ok = fixed && (sg == 0 || fx.enter(v0, e0));
+                fx.bad = 0;
+                double(*b)[W][32] = sm.slab[j % 3];
+                auto put = [&](int r) {
+#pragma unroll
+                    for (int k = 0; k < K; ++k) b[r][k][lane] = (double)fx.V[k];
+                    b[r][K][lane] = (double)fx.shock();
+                    b[r][K + 1][lane] = fx.inv_h();
+                };
+                if (t0 == 0) fx.template chain<true>(y[0], sm.tab);
+                else fx.template chain<false>(y[t0], sm.tab);
+                put(0);
+#pragma unroll 2
+                for (int r = 1; r < n; ++r) {
+                    fx.template chain<false>(y[t0 + r], sm.tab);
+                    put(r);
+                }
+                ok = ok && fx.bad == 0u;
+                if (!ok) {
+#pragma unroll
+                    for (int k = 0; k < K; ++k) w.v[k] = v0[k];
+                    w.eps = e0;
+                    segment_f64(w, q.log_sigma_y, y, t0, n, &b[0][K][lane], W * 32, &b[0][0][lane], &b[0][K + 1][lane]);
+                }
+            }
+            if (j >= 2) {                  // carry over segment nseg + 1 - j
+                const int sg = nseg + 1 - j, t0 = sg * kSeg, n = min(kSeg, T - t0);
+                const double(*b)[W][32] = sm.slab[(j - 2) % 3];
+                const double* dl = &sm.x[j & 1][0][lane];
+#pragma unroll 2
+                for (int r = n - 1; r >= 1; --r) {
+                    double vp[K];
+#pragma unroll
+                    for (int k = 0; k < K; ++k) vp[k] = b[r - 1][k][lane];
+                    carry(dl[r * 32], b[r][K][lane], b[r][K + 1][lane], vp, b[r - 1][K][lane], true);
+                }
+                double v0[K], e0;
+                entering(sg, v0, e0);
+#pragma unroll
+                for (int k = 0; k < K; ++k) v0[k] *= kVu;
+                carry(dl[0], b[0][K][lane], b[0][K + 1][lane], v0, e0 * 0x1p53, t0 > 0);
+                if ((sg & 7) == 0) {
+#pragma unroll
+                    for (int i = 0; i < NS; ++i) {
+                        gn[i] += gs[i];
+                        gs[i] = 0.0;
+                    }
+                }
+            }
+            meet();
+        }
+        gn[0] *= 0x1p53;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            gn[2 + k] *= 0.5 / kVu;
+            gn[2 + K + k] *= 0x1p-54;
+            gn[2 + 2 * K + k] *= 0x1p-54;
+        }
+        meet();                            // warp 1's results
+#pragma unroll
+        for (int i = 0; i < 3 * I; ++i) gn[NS + i] = sm.comb[i][lane];
+        double ll = sm.comb[3 * I][lane] - logh - 0.5 * kLog2Pi * (double)T;
+        if (!(ll > -INFINITY)) ll = -INFINITY;
+        double gfull[kMaxD];
+        natural_to_theta_f64<K, I>(q, gn, full, a.m.gamma, gfull);
+        if (!active) return;
+        a.ll[p] = ll;
+        for (int k = 0; k < a.m.d; ++k) a.grad[k * P + p] = gfull[a.m.has_free ? a.m.free_idx[k] : k];
+    }
+
+    __device__ __forceinline__ static void mixture_warp(Smem& sm, EgarchFx<K, I> fx,
+                                                        const EgarchParams<double, K, I>& q, bool fixed, int lane,
+                                                        int T, int nseg)
+    {
+        // forward: sum_t log mixture density
+        double e1 = 0.0, e2 = 0.0, lm64 = 0.0;   // sums of eps, eps^2 (2^-53, 2^-106); densities in FP64
+        int n64 = 0;
+        unsigned __int128 scw = 0;
+        meet();                            // (segment 0 is warp 0's alone)
+        for (int sg = 0; sg < nseg; ++sg) {
+            const int n = min(kSeg, T - sg * kSeg);
+            const double* es = &sm.x[sg & 1][0][lane];
+            double u1 = 0.0, u2 = 0.0;
+            for (int h = 0; h < n; h += 8) {
+                fx.sc = 0;
+#pragma unroll 2
+                for (int r = h; r < min(n, h + 8); ++r) {
+                    const double e = es[r * 32];
+                    const uint64_t pm = fx.pm, sc = fx.sc;
+                    const int pe = fx.pe;
+                    uint32_t over;
+                    fx.mix_terms(e, sm.tab, over);
+                    if (over != 0u || !fixed) {
+                        uint64_t r8[I];
+                        fx.pm = pm;
+                        fx.pe = pe;
+                        fx.sc = sc;
+                        lm64 += weights_f64(q, e * 0x1p-53, sm.tab, r8);
+                        ++n64;
+                    } else {
+                        u1 += e;
+                        u2 = fma(e, e, u2);
+                    }
+                }
+                scw += fx.sc;
+            }
+            e1 += u1;
+            e2 += u2;
+            meet();
+        }
+        double lm = lm64;
+        if (fixed) {
+            const double nf = (double)(T - n64);
+            lm += kLn2 * (EgarchFx<K, I>::to_double((__int128)scw) * 0x1p-55 + (double)fx.pe + log2((double)fx.pm * 0x1p-62)) -
+                  0.5 * (fx.a0 * fx.a0) * (e2 * 0x1p-106 - 2.0 * fx.m0 * (e1 * 0x1p-53) + nf * (fx.m0 * fx.m0)) +
+                  nf * (kLn2 * fx.c0);
+        }
+        // backward: dl/deps and the component sums
+        double a2[I], m2[I], s1[I], s2[I], g[3 * I];
+        uint64_t s0[I];
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            const double ai = 1.0 / q.sig[i];
+            a2[i] = ai * ai * 0x1p-165;    // (r_i 2^59, eps 2^53, dl/deps 2^-53)
+            m2[i] = q.mu[i] * (ai * ai) * 0x1p-112;
+            s1[i] = s2[i] = 0.0;
+            s0[i] = 0;
+            g[i] = g[I + i] = g[2 * I + i] = 0.0;
+        }
+        meet();                            // (step 0 is warp 0's alone)
+        for (int j = 1; j < nseg + 2; ++j) {
+            if (j <= nseg) {
+                const int sg = nseg - j, n = min(kSeg, T - sg * kSeg);
+                const double(*b)[W][32] = sm.slab[(j - 1) % 3];
+                double* dl = &sm.x[(j - 1) & 1][0][lane];
+#pragma unroll 2
+                for (int r = n - 1; r >= 0; --r) {
+                    const double es = b[r][K][lane];
+                    uint64_t ri[I];
+                    if (!(fixed && fx.weights(es, ri, sm.tab))) weights_f64(q, es * 0x1p-53, sm.tab, ri);
+                    double d = 0.0;
+#pragma unroll
+                    for (int i = 0; i < I; ++i) {
+                        const double rd = (double)(int64_t)ri[i];
+                        const double re = rd * es;
+                        d = fma(-re, a2[i], fma(rd, m2[i], d));
+                        s0[i] += ri[i];
+                        s1[i] += re;
+                        s2[i] = fma(re, es, s2[i]);
+                    }
+                    dl[r * 32] = d;
+                }
+#pragma unroll
+                for (int i = 0; i < I; ++i) {
+                    g[i] += (double)s0[i] * 0x1p-59;   // (16 r_i of at most 2^59)
+                    s0[i] = 0;
+                }
+                if ((sg & 7) == 0) {
+#pragma unroll
+                    for (int i = 0; i < I; ++i) {
+                        g[I + i] += s1[i];
+                        g[2 * I + i] += s2[i];
+                        s1[i] = s2[i] = 0.0;
+                    }
+                }
+            }
+            meet();
+        }
+#pragma unroll
+        for (int i = 0; i < I; ++i) {
+            const double r0 = g[i], r1 = g[I + i] * 0x1p-112, r2 = g[2 * I + i] * 0x1p-112 * 0x1p-53;
+            const double ai = 1.0 / q.sig[i], mu = q.mu[i];
+            sm.comb[i][lane] = r0;
+            sm.comb[I + i][lane] = ai * ai * (r1 - mu * r0);
+            sm.comb[2 * I + i][lane] = q.sig[i] * r0 - ai * (r2 - mu * (2.0 * r1 - mu * r0));
+        }
+        sm.comb[3 * I][lane] = lm;
+        meet();                            // warp 0 takes them
     }
 };
 

@@ -589,6 +589,7 @@ static smc_status refresh_gradient(smc_ctx* ctx, int T)
     g.grad = ctx->grad[ctx->cur];
     g.state = ctx->ns ? ctx->state[ctx->cur] : nullptr;
     g.ckpt = ctx->ckpt;
+    g.by_size = 0;
     CU(launch_loglik_grad(g, ctx->cfg.precision, ctx->stream));
     return SMC_OK;
 }

@@ -445,11 +445,10 @@ struct EgarchFx {
     }
 
     // Posterior weights r_i of the components (order of setup's arguments;
-    // units 2^-59) for the shock eps; false where a d_i is out of range.
+    // units 2^-59) for the shock ed (units 2^-53); false where a d_i is out of range.
     // 1 / s by two Newton steps on integers from the FP32 reciprocal.
-    SMC_FX bool weights(double eps, uint64_t* r, const uint64_t* tab) const
+    SMC_FX bool weights(double ed, uint64_t* r, const uint64_t* tab) const
     {
-        const double ed = eps * 0x1p53;
         int64_t D[I], cur = 0;
         uint32_t over = 0;
         D[0] = 0;
@@ -490,6 +489,13 @@ struct EgarchFx {
     // 1 / h_t of the last chain().
     SMC_FX double inv_h() const { return fx_pack(M, (int)(uint32_t)(X >> 55) - 256); }
 
+    // eps_t of the last chain() (units 2^-53).
+    SMC_FX int64_t shock() const
+    {
+        const uint64_t sg = (uint64_t)(int64_t)neg;
+        return (int64_t)((E ^ sg) - sg);
+    }
+
     // The mixture part for the shock (E_, neg_): independent of the next
     // observation's chain.
     SMC_FX void mix(uint64_t E_, int32_t neg_, const uint64_t* tab)
@@ -498,14 +504,23 @@ struct EgarchFx {
         const uint64_t sg = (uint64_t)(int64_t)neg_;
         const int64_t es = (int64_t)((E_ ^ sg) - sg);
         s1 += es;
-        const double ed_ = (double)es;
+        uint32_t over;
+        mix_terms((double)es, tab, over);
+        bad |= over;
+    }
+
+    // m_t and s_t of the shock ed_ (units 2^-53) into their sums; over: bit 31
+    // set (and the sums spoiled) where a d_i is out of range.
+    SMC_FX void mix_terms(double ed_, const uint64_t* tab, uint32_t& over)
+    {
+        over = 0;
         int64_t D[kM];
         int64_t cur = 0;
 #pragma unroll
         for (int i = 0; i < kM; ++i) {
-            uint32_t over;
-            const int64_t x = term(i, ed_, 5, over);   // 16 or more is out of range
-            bad |= over;
+            uint32_t o;
+            const int64_t x = term(i, ed_, 5, o);   // 16 or more is out of range
+            over |= o;
             // (cur, D_i) <- (max, min): the terms stay the same set, and cur
             // ends as the largest
             D[i] = x < cur ? x : cur;

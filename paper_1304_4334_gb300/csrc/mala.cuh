@@ -5,6 +5,7 @@
 #include "adjoint.cuh"
 #include "adjoint_f64.cuh"
 #include "kernels.cuh"
+#include "phase.cuh"
 
 namespace smc {
 
@@ -13,18 +14,6 @@ constexpr int kMalaThreads = 128;
 // for one segment's recomputed states (mala_seg x (K + 2) values), so narrower blocks
 // pack more resident blocks per SM and leave a smaller last wave.
 constexpr int kMalaLaunch = 64;
-
-struct GradArgs {
-    ModelDev m;
-    const void* obs;
-    int T, W;
-    const double* theta;   // [d][P]
-    int P;
-    double* ll;            // [P]
-    double* grad;          // [d][P] d log p(y|theta) / d theta (free parameters)
-    double* state;         // [K+1][P] (nullable)
-    void* ckpt;            // segment checkpoints (gradient policy's layout)
-};
 
 // One MALA iteration: theta* = theta + (1/2) L L' g + L z with g the gradient
 // of the tempered log target lp + phi l at theta (from the stored likelihood
@@ -69,6 +58,7 @@ struct GradEgarch {
         return (size_t)(nseg > 1 ? nseg - 1 : 1) * (K + 1) * (size_t)P * sizeof(Real);
     }
     static constexpr bool kExpTab = sizeof(Real) == 8;
+    static constexpr int kNi = I;
     // tab: the exp2 table in shared memory (FP64)
     __device__ static double eval(const ModelDev& m, const double* th, const void* obs, int T, int,
                                   void* ckpt, size_t P, int p, Real* buf, int stride, double* g,
@@ -122,6 +112,7 @@ struct GradEgarch {
 struct GradLinreg {
     using RealT = double;
     static constexpr bool kExpTab = false;
+    static constexpr int kNi = 1;
     static constexpr int kNs = 0;
     static size_t smem_bytes(int) { return 0; }
     static size_t ckpt_bytes(int, int) { return 8; }
@@ -278,9 +269,38 @@ __global__ void __launch_bounds__(kMalaThreads) k_mutate_mala(MalaArgs a)
     if (blockIdx.x == 0 && threadIdx.x == 0 && a.pending) *a.pending = 1;
 }
 
+template <int K, int I>
+__global__ void __launch_bounds__(64, 1) k_loglik_grad_split(GradArgs a)
+{
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    GradSplit<K, I>::run(a, *reinterpret_cast<typename GradSplit<K, I>::Smem*>(sm_raw));
+}
+
+// Two warps per 32 particles while all of them are resident at once (224 KB of
+// shared memory per SM, 1 KB of it the system's per block): GradSplit's figures
+// are 1.4-2.1x there, and a second wave of blocks costs as much as the first.
+template <int K, int I>
+cudaError_t launch_grad_split(const GradArgs& a, cudaStream_t s, bool* taken)
+{
+    constexpr size_t sm = sizeof(typename GradSplit<K, I>::Smem);
+    constexpr int per_sm = (int)(224 * 1024 / (sm + 1024));
+    *taken = (a.P + 31) / 32 <= per_sm * device_sm_count();
+    if (!*taken) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(k_loglik_grad_split<K, I>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sm);
+    if (e != cudaSuccess) return e;
+    k_loglik_grad_split<K, I><<<(a.P + 31) / 32, 64, sm, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <class GP>
 cudaError_t launch_grad_t(const GradArgs& a, cudaStream_t s)
 {
+    if constexpr (GP::kExpTab && GP::kNi > 1) {
+        bool taken = false;
+        const cudaError_t e = a.by_size ? launch_grad_split<GP::kNs - 1, GP::kNi>(a, s, &taken) : cudaSuccess;
+        if (taken) return e;
+    }
     const size_t sm = GP::smem_bytes(kMalaLaunch);
     static bool attr = false;
     if (!attr && sm > 0) {   // static + dynamic shared memory may pass the 48 KB default

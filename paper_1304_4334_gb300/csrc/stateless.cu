@@ -281,6 +281,7 @@ smc_status smc_loglik_grad(const smc_model* m, int precision, const void* obs, i
     w.add(n_ckpt);
     CK(w.get());
     a.ckpt = w.take<void>(n_ckpt);
+    a.by_size = 1;
     return from_cuda(launch_loglik_grad(a, precision, s));
 }
 

@@ -108,3 +108,34 @@ def test_gradient_with_range_exits(S, K, I_, T):
     np.testing.assert_allclose(ll[sane], ll_o[sane], rtol=1e-9)
     err = np.abs(g - g_o)[sane].max(axis=1) / np.abs(g_o[sane]).max(axis=1)
     assert err.max() <= 1e-7, err.max()
+
+
+@pytest.mark.parametrize("K,I_", [(1, 2), (2, 3), (4, 4)])
+@pytest.mark.parametrize("T", [1, 16, 17, 33, 530])
+def test_gradient_kernels_of_few_and_many_particles(S, K, I_, T):
+    """The same particles in a call small enough for two warps per 32 of them and
+    in one that is not, a ragged last warp, range exits and a shock out of range
+    included: two orders of the same FP64 sums, so far within 1e-9 (of the
+    largest entry of the gradient, whose entries cancel)."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = _series(truth, T)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    P, n = 77, 200 * torch.cuda.get_device_properties(0).multi_processor_count
+    th = particles(spec.d, truth, K, I_, True, P, 81, prior=O.table1_prior(K, I_, True), frac_prior=0.2)
+    th[:8, spec.d - 1] = -4.0                      # a component far narrower
+    th[:8, spec.d - I_ - 1] = 3.0                  # than its distance from zero
+    out = []
+    for tt in (th, np.resize(th, (n, spec.d))):
+        ll = torch.empty(len(tt), dtype=torch.float64, device="cuda")
+        g = torch.empty((spec.d, len(tt)), dtype=torch.float64, device="cuda")
+        st = torch.empty((K + 1, len(tt)), dtype=torch.float64, device="cuda")
+        S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(tt), ll, g, st)
+        out.append([host(ll)[:P], host(g).T[:P], host(st).T[:P]])
+    (l1, g1, s1), (l2, g2, s2) = out
+    assert np.array_equal(l1 > -1e7, l2 > -1e7)
+    sane = (l2 > -1e7) & np.isfinite(g2).all(axis=1)
+    assert sane.sum() > P // 2
+    np.testing.assert_allclose(l1[sane], l2[sane], rtol=1e-9)
+    assert (np.abs(g1 - g2)[sane].max(axis=1) <= 1e-9 * np.abs(g2[sane]).max(axis=1)).all()
+    np.testing.assert_allclose(s1[sane], s2[sane], rtol=1e-9, atol=1e-12)
