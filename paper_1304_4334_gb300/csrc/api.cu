@@ -957,6 +957,7 @@ static smc_status start_run(smc_ctx* ctx, const double* theta0, int theta0_on_de
         la.P = P;
         la.ns = ctx->ns;
         la.err = &ctx->ctl->err;
+        la.by_size = 0;
         CU(launch_loglik(la, c->precision, ctx->stream));
         if (c->mutation == SMC_MALA) {
             smc_status st = refresh_gradient(ctx, T);

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "loglik_split.cuh"
 #include "phase.cuh"
 
 #include <type_traits>
@@ -74,6 +75,16 @@ cudaError_t launch_mutate_x2_k(const MutateArgs& a, int threads, cudaStream_t s)
 template <template <int, int> class Pol, int K>
 cudaError_t launch_loglik_k(const LoglikArgs& a, cudaStream_t s)
 {
+    if constexpr (Pol<K, 2>::kExpTab) {   // FP64: the fixed-point recursion
+        bool taken = false;
+        cudaError_t e = cudaSuccess;
+        switch (a.m.I) {
+        case 2: e = launch_loglik_split<K, 2>(a, s, &taken); break;
+        case 3: e = launch_loglik_split<K, 3>(a, s, &taken); break;
+        case 4: e = launch_loglik_split<K, 4>(a, s, &taken); break;
+        }
+        if (taken) return e;
+    }
     void (*k)(LoglikArgs) = nullptr;
     switch (a.m.I) {
     case 1: k = KernelPick<Pol<K, 1>>::loglik(a.P); break;

@@ -62,6 +62,7 @@ struct LoglikArgs {
     double* state;          // [ns][P] (nullable)
     int P, ns;
     int* err;
+    int by_size;            // the kernel may be chosen by P (the last bits of ll differ between them)
 };
 
 constexpr int kMutThreads = 128;

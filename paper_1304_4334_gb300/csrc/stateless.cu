@@ -177,6 +177,7 @@ smc_status smc_loglik(const smc_model* m, int precision, const void* obs, int T,
     a.P = P;
     a.ns = m->model == SMC_EGARCH ? m->K + 1 : 0;
     a.err = nullptr;
+    a.by_size = 1;
     return from_cuda(launch_loglik(a, precision, (cudaStream_t)stream));
 }
 

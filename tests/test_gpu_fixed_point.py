@@ -139,3 +139,32 @@ def test_gradient_kernels_of_few_and_many_particles(S, K, I_, T):
     np.testing.assert_allclose(l1[sane], l2[sane], rtol=1e-9)
     assert (np.abs(g1 - g2)[sane].max(axis=1) <= 1e-9 * np.abs(g2[sane]).max(axis=1)).all()
     np.testing.assert_allclose(s1[sane], s2[sane], rtol=1e-9, atol=1e-12)
+
+
+@pytest.mark.parametrize("K,I_", [(1, 2), (2, 3), (4, 4)])
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 65, 530])
+def test_likelihood_kernels_of_few_and_many_particles(S, K, I_, T):
+    """As above for the log likelihood: two or three warps per 32 particles in
+    the small call, one in the large, the same integer sums but for the order of
+    the mixture sums' product and the FP64 parts of range exits."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = _series(truth, T)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    P, n = 77, 200 * torch.cuda.get_device_properties(0).multi_processor_count
+    th = particles(spec.d, truth, K, I_, True, P, 83, prior=O.table1_prior(K, I_, True), frac_prior=0.2)
+    th[:8, spec.d - 1] = -4.0                      # a component far narrower
+    th[:8, spec.d - I_ - 1] = 3.0                  # than its distance from zero
+    out = []
+    for tt in (th, np.resize(th, (n, spec.d))):
+        ll = torch.empty(len(tt), dtype=torch.float64, device="cuda")
+        lp = torch.empty(len(tt), dtype=torch.float64, device="cuda")
+        st = torch.empty((K + 1, len(tt)), dtype=torch.float64, device="cuda")
+        S.loglik(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(tt), ll, lp, st)
+        out.append([host(ll)[:P], host(lp)[:P], host(st).T[:P]])
+    (l1, p1, s1), (l2, p2, s2) = out
+    assert np.array_equal(l1 > -1e7, l2 > -1e7) and np.array_equal(p1, p2)
+    sane = l2 > -1e7
+    assert sane.sum() > P // 2
+    np.testing.assert_allclose(l1[sane], l2[sane], rtol=1e-9)
+    np.testing.assert_allclose(s1[sane], s2[sane], rtol=1e-9, atol=1e-12)
