@@ -25,11 +25,12 @@
 // (EgarchF64), which takes any value.
 //
 // Measured, random-walk iteration at K = 2, I = 2, 65,536 particles x 5,000
-// observations: 76.1 ms with the recursion in FP64, 5.5 ms (about 330
-// instructions per particle and observation, 55% of the FP64 pipe, 47% of the
+// observations: 76.1 ms with the recursion in FP64, 5.1 ms (about 330
+// instructions per particle and observation, over half of the FP64 and of the
 // integer pipe at four warps per scheduler); likelihood at K = 3, I = 4,
-// 10,007 x 3,089: 17.8 ms, 2.9 ms (one warp per scheduler: the chain's
-// latency); 1,024 x 500 at K = I = 1: 0.50 ms, 0.12 ms.  Errors against
+// 10,007 x 3,089: 17.8 ms, 2.28 ms with one warp per 32 particles (one warp per
+// scheduler: the chain's latency), 1.47 ms with three (LoglikSplit); mutation of
+// 1,024 x 500 at K = I = 1: 0.55 ms, 0.14 ms.  Errors against
 // 113-bit arithmetic: log likelihood 2e-16 relative at T = 5,000 (2.5e-15 in
 // FP64, whose running sum rounds), end state 0.4 to 1 of FP64's.
 //
@@ -548,8 +549,9 @@ struct EgarchFx {
 
     // n observations (first: they open the series), sums flushed.  Eight steps
     // between flushes without a test in between, unrolled by two: the pieces
-    // of two steps interleave (K=3, I=4, one warp per scheduler: MEASURED_BLK
-    // cycles an observation; by three or four it is slower again).
+    // of two steps interleave (K=3, I=4, one warp per scheduler:
+    // 1,830 cycles an observation taken singly, 1,190 so; by three or four it is
+    // slower again).
     SMC_FX void block(const double* y, int n, bool first, const uint64_t* tab)
     {
         if (first) chain<true>(y[0], tab);

@@ -124,47 +124,48 @@ size_t cov_smem(int d)
 
 // One block's partial sums: a warp per tile.  The warp stages its tile (two
 // particles a lane, four rows a store), and each lane then owns B x B products
-// x_i x_k and, on the diagonal, the B sums x_i (kRounds such blocks above
-// 28 parameters): within a tile one FMA chain per entry in the particles'
+// x_i x_k and, on the diagonal, the B sums x_i: within a tile one FMA chain per entry in the particles'
 // order, tiles added up as exact pairs (TwoSum) and converted once, so the
 // result does not depend on B.  Bound by the FMAs' issue and the loads of theta
 // (193 MB at d = 23, 1,048,576 particles).  The first form gave one entry to a
 // thread (two 4-byte loads per FMA) and formed and converted theta - shift in
-// FP64: 307 us there, now 94 us (14 parameters, 65,536 particles: the whole call
-// 35 -> 32 us).
-template <int B, int kRounds>
+// FP64: 307 us there, now 94 us (whole calls: 14 parameters, 70,000 particles 31
+// -> 25 us; 32, 250,000 106 -> 76 us).
+// kM > 1: kM warps share a tile, its rows to stage and its products.
+template <int B, int kM = 1>
 __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta, int d, int P,
                                                 double* __restrict__ part, int bidx, int G, float* sm)
 {
-    constexpr int kE = B * B + B;
+    constexpr int kE = B * B + B, kGroups = kCovWarps / kM;
     __shared__ double shift[kMaxD];
     __shared__ float2 shift2[kMaxD];
     __shared__ bool shift_ok[kMaxD];
     const int nb = (d + B - 1) / B, nblk = nb * (nb + 1) / 2;
     const int nacc = d + d * (d + 1) / 2;
     const size_t Ps = (size_t)P;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, grp = threadIdx.x / (32 * kM), part_of = (threadIdx.x >> 5) % kM;
+    const int item = lane + 32 * part_of;
     for (int i = threadIdx.x; i < d; i += blockDim.x) {
         shift[i] = theta[i * Ps];
         shift2[i] = split_f64(shift[i], shift_ok[i]);
     }
     __syncthreads();
     const int pitch = cov_pitch(d);
-    float* tile = sm + warp * kCovTile * pitch;
-    int bi[kRounds], bk[kRounds];
-    float hi[kRounds][kE], lo[kRounds][kE];
+    float* tile = sm + grp * kCovTile * pitch;
+    int bi, bk;
+    float hi[kE], lo[kE];
+    unpack_pair(min(item, nblk - 1), bi, bk);
 #pragma unroll
-    for (int q = 0; q < kRounds; ++q) {
-        unpack_pair(min(lane + 32 * q, nblk - 1), bi[q], bk[q]);
-#pragma unroll
-        for (int e = 0; e < kE; ++e) hi[q][e] = lo[q][e] = 0.0f;
-    }
+    for (int e = 0; e < kE; ++e) hi[e] = lo[e] = 0.0f;
     const int per = (P + G - 1) / G;
     const int n0 = bidx * per, n1 = min(P, n0 + per);
-    for (int base = n0 + warp * kCovTile; base < n1; base += kCovWarps * kCovTile) {
+    const int off = grp * kCovTile;
+    // (kM > 1: every warp of the block the same number of times, empty tiles are zeros)
+    for (int base = n0 + off; base < (kM > 1 ? n1 + off : n1); base += kGroups * kCovTile) {
         const int cnt = min(kCovTile, n1 - base);
-        __syncwarp();
-        for (int r = 0; r < d; r += 4) {
+        if constexpr (kM > 1) __syncthreads();
+        else __syncwarp();
+        for (int r = 4 * part_of; r < d; r += 4 * kM) {
             double t[2][4];
 #pragma unroll
             for (int h = 0; h < 2; ++h)
@@ -181,68 +182,64 @@ __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta
                 *reinterpret_cast<float4*>(tile + (lane + 32 * h) * pitch + r) = make_float4(x[0], x[1], x[2], x[3]);
             }
         }
-        __syncwarp();
+        if constexpr (kM > 1) __syncthreads();
+        else __syncwarp();
+        float s[kE];
 #pragma unroll
-        for (int q = 0; q < kRounds; ++q) {
-            float s[kE];
-#pragma unroll
-            for (int e = 0; e < kE; ++e) s[e] = 0.0f;
-            const float* ti = tile + B * bi[q];
-            const float* tk = tile + B * bk[q];
+        for (int e = 0; e < kE; ++e) s[e] = 0.0f;
+        const float* ti = tile + B * bi;
+        const float* tk = tile + B * bk;
 #pragma unroll 4
-            for (int n = 0; n < kCovTile; ++n) {   // (zeros past cnt change nothing)
-                float a[B], b[B];
-                if constexpr (B == 4) {
-                    const float4 a4 = *reinterpret_cast<const float4*>(ti + n * pitch);
-                    const float4 b4 = *reinterpret_cast<const float4*>(tk + n * pitch);
-                    a[0] = a4.x, a[1] = a4.y, a[2] = a4.z, a[3] = a4.w;
-                    b[0] = b4.x, b[1] = b4.y, b[2] = b4.z, b[3] = b4.w;
-                } else if constexpr (B == 2) {
-                    const float2 a2 = *reinterpret_cast<const float2*>(ti + n * pitch);
-                    const float2 b2 = *reinterpret_cast<const float2*>(tk + n * pitch);
-                    a[0] = a2.x, a[1] = a2.y;
-                    b[0] = b2.x, b[1] = b2.y;
-                } else {
-                    a[0] = ti[n * pitch];
-                    b[0] = tk[n * pitch];
-                }
-#pragma unroll
-                for (int i = 0; i < B; ++i) {
-#pragma unroll
-                    for (int k = 0; k < B; ++k) s[B * i + k] = fmaf(a[i], b[k], s[B * i + k]);
-                    s[B * B + i] += a[i];
-                }
+        for (int n = 0; n < kCovTile; ++n) {   // (zeros past cnt change nothing)
+            float a[B], b[B];
+            if constexpr (B == 4) {
+                const float4 a4 = *reinterpret_cast<const float4*>(ti + n * pitch);
+                const float4 b4 = *reinterpret_cast<const float4*>(tk + n * pitch);
+                a[0] = a4.x, a[1] = a4.y, a[2] = a4.z, a[3] = a4.w;
+                b[0] = b4.x, b[1] = b4.y, b[2] = b4.z, b[3] = b4.w;
+            } else if constexpr (B == 2) {
+                const float2 a2 = *reinterpret_cast<const float2*>(ti + n * pitch);
+                const float2 b2 = *reinterpret_cast<const float2*>(tk + n * pitch);
+                a[0] = a2.x, a[1] = a2.y;
+                b[0] = b2.x, b[1] = b2.y;
+            } else {
+                a[0] = ti[n * pitch];
+                b[0] = tk[n * pitch];
             }
 #pragma unroll
-            for (int e = 0; e < kE; ++e) {
-                const float a = hi[q][e] + s[e];
-                const float bv = a - hi[q][e];
-                lo[q][e] += (hi[q][e] - (a - bv)) + (s[e] - bv);
-                hi[q][e] = a;
+            for (int i = 0; i < B; ++i) {
+#pragma unroll
+                for (int k = 0; k < B; ++k) s[B * i + k] = fmaf(a[i], b[k], s[B * i + k]);
+                s[B * B + i] += a[i];
             }
+        }
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+            const float a = hi[e] + s[e];
+            const float bv = a - hi[e];
+            lo[e] += (hi[e] - (a - bv)) + (s[e] - bv);
+            hi[e] = a;
         }
     }
     // the warps' sums, added per entry in the warps' order
     __syncthreads();
     double* sums = reinterpret_cast<double*>(sm);
-#pragma unroll
-    for (int q = 0; q < kRounds; ++q) {
-        if (lane + 32 * q >= nblk) continue;
+    if (item < nblk) {
 #pragma unroll
         for (int i = 0; i < B; ++i) {
-            const int ri = B * bi[q] + i;
+            const int ri = B * bi + i;
             if (ri >= d) continue;
-            double* w = sums + warp * nacc;
+            double* w = sums + grp * nacc;
 #pragma unroll
             for (int k = 0; k < B; ++k) {
-                const int rk = B * bk[q] + k;
-                if (rk <= ri) w[d + ri * (ri + 1) / 2 + rk] = (double)hi[q][B * i + k] + (double)lo[q][B * i + k];
+                const int rk = B * bk + k;
+                if (rk <= ri) w[d + ri * (ri + 1) / 2 + rk] = (double)hi[B * i + k] + (double)lo[B * i + k];
             }
-            if (bi[q] == bk[q]) w[ri] = (double)hi[q][B * B + i] + (double)lo[q][B * B + i];
+            if (bi == bk) w[ri] = (double)hi[B * B + i] + (double)lo[B * B + i];
         }
     }
     __syncthreads();
-    const int used = min(kCovWarps, (n1 - n0 + kCovTile - 1) / kCovTile);   // warps that had a tile
+    const int used = min(kGroups, (n1 - n0 + kCovTile - 1) / kCovTile);   // those that had a tile
     for (int e = threadIdx.x; e < nacc; e += blockDim.x) {
         double t = 0.0;
         for (int w = 0; w < used; ++w) t += sums[w * nacc + e];
@@ -250,25 +247,35 @@ __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta
     }
 }
 
-template <int B, int kRounds>
-__global__ void __launch_bounds__(kCovThreads, kRounds == 1 ? 2 : 1) k_cov_partial(const double* __restrict__ theta, int d,
+template <int B, int kM = 1>
+__global__ void __launch_bounds__(kCovThreads, 2) k_cov_partial(const double* __restrict__ theta, int d,
                                                                int P, double* __restrict__ part)
 {
     extern __shared__ __align__(16) float cov_sm[];
     pdl_trigger();
     pdl_wait();
-    cov_partial_run<B, kRounds>(theta, d, P, part, blockIdx.x, gridDim.x, cov_sm);
+    cov_partial_run<B, kM>(theta, d, P, part, blockIdx.x, gridDim.x, cov_sm);
 }
 
-// The smallest block that still gives every lane at most one of them: more
-// lanes at work and shorter chains of issue per tile (at d = 4, one tile per
-// block, a 4 x 4 block would sit on a single lane).
+// Warps to a tile and the blocks' size, by the tiles a block has: while they
+// leave warps idle these share one, down to one product a lane (the most lanes
+// at work and the shortest chain of issue per tile); with a tile for every warp
+// the smallest block that still gives every lane at most one.  Above 28
+// parameters the 36 blocks of 4 x 4 go to two warps at any size.  Up to 28 the
+// tiles of a block are added in one order whatever the form.  Whole calls, one
+// warp to a tile -> shared: d=18, 77,700 particles 34 -> 28.7 us; d=26, 24,846
+// 40.5 -> 32.2 us; d=16, 16,000 26.1 -> 20.1 us.
 using CovPartialFn = void (*)(const double*, int, int, double*);
-CovPartialFn cov_partial_kernel(int d)
+CovPartialFn cov_partial_kernel(int d, int P, int G)
 {
-    if (d <= 7) return k_cov_partial<1, 1>;
-    if (d <= 14) return k_cov_partial<2, 1>;
-    return d <= 28 ? k_cov_partial<4, 1> : k_cov_partial<4, 2>;
+    const int tiles = ((P + G - 1) / G + kCovTile - 1) / kCovTile;   // of a block
+    if (d <= 7) return k_cov_partial<1>;
+    if (d <= 14) return tiles <= 2 ? k_cov_partial<1, 4> : k_cov_partial<2>;   // (105 products)
+    if (d <= 22 && tiles <= 1) return k_cov_partial<1, 8>;                     // (253)
+    if (d <= 30 && tiles <= 2) return k_cov_partial<2, 4>;                     // (120 blocks of 2 x 2)
+    if (d <= 20 && tiles <= 4) return k_cov_partial<2, 2>;                     // (55)
+    if (d > 28 && tiles <= 2) return k_cov_partial<2, 8>;                      // (136)
+    return d <= 28 ? k_cov_partial<4> : k_cov_partial<4, 2>;
 }
 
 __device__ void apply_h_update(Ctl* ctl, int P, double target, int hmin, int hmax)
@@ -577,7 +584,7 @@ __global__ void __launch_bounds__(kCovThreads, 2) k_cov_partial_batch(const CovJ
     extern __shared__ __align__(16) float cov_sm[];
     const CovJob& j = jobs[blockIdx.y];
     if ((int)blockIdx.x >= j.G || *iter >= j.R || j.tiles) return;
-    cov_partial_run<4, 1>(j.theta, j.d, j.P, j.part, blockIdx.x, j.G, cov_sm);   // (EGARCH: d <= 26)
+    cov_partial_run<4>(j.theta, j.d, j.P, j.part, blockIdx.x, j.G, cov_sm);   // (EGARCH: d <= 26)
     static_assert(2 + 3 * kMaxK + 3 * kMaxI <= 28);
 }
 
@@ -613,8 +620,10 @@ static cudaError_t cov_smem_limits()
     if (e != cudaSuccess) return e;
     const uint64_t bit = 1ull << (dev & 63);
     if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    for (const int d : {7, 14, 28, kMaxD}) {
-        e = cudaFuncSetAttribute(cov_partial_kernel(d), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    for (const CovPartialFn fn : {k_cov_partial<1>, k_cov_partial<2>, k_cov_partial<4>, k_cov_partial<1, 4>,
+                                  k_cov_partial<1, 8>, k_cov_partial<2, 2>, k_cov_partial<2, 4>, k_cov_partial<2, 8>,
+                                  k_cov_partial<4, 2>}) {
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)cov_smem(kMaxD));
         if (e != cudaSuccess) return e;
     }
@@ -642,7 +651,7 @@ cudaError_t launch_cov(const double* theta, int d, int P, double* part, int G, u
 {
     cudaError_t e = cov_smem_limits();
     if (e != cudaSuccess) return e;
-    e = pdl_launch(cov_partial_kernel(d), dim3(G), dim3(kCovThreads), cov_smem(d), s, theta, d, P, part);
+    e = pdl_launch(cov_partial_kernel(d, P, G), dim3(G), dim3(kCovThreads), cov_smem(d), s, theta, d, P, part);
     count_launch();
     if (e != cudaSuccess) return e;
     const int nacc = d + d * (d + 1) / 2;
@@ -726,8 +735,9 @@ constexpr int kCand = 32;
 constexpr float kFixScale = 68719476736.0f;       // 2^36
 
 // Up to kSoloTiles tiles one block runs the search alone, with block barriers
-// in the place of grid barriers and global totals (about 4 us a pass): 32 ->
-// 12 us at 1,024 particles; at 4,096 both take the same.
+// in the place of grid barriers and global totals (about 4 us a pass): a
+// whole power-search call 84.9 -> 51.4 us at 1,024 particles, 90.8 -> 63.4 at
+// 2,048; at 4,096 both take the same.
 constexpr int kSoloTiles = 64;
 
 int search_grid(int P)

@@ -580,6 +580,15 @@ def test_covariance_block_shapes_match_numpy(S, d, P):
         assert np.abs(Lh @ Lh.T - 0.25 * want).max() <= 2 * tol
 
 
+@pytest.mark.parametrize("d,P", [(15, 2), (16, 27330), (20, 77824), (20, 77825), (21, 38912), (30, 38913), (26, 24846),
+                                 (31, 19456), (32, 19457), (29, 64),
+                                 (32, 77824), (31, 77825), (22, 19456), (15, 19457), (14, 38912), (8, 38913)])
+def test_covariance_warps_sharing_tiles_match_numpy(S, d, P):
+    """Few tiles per block (one, two and four, and one particle more, at 152
+    SMs), at the same tolerance."""
+    test_covariance_block_shapes_match_numpy(S, d, P)
+
+
 @pytest.mark.parametrize("P", [1, 31, 33, 511, 2047, 2048, 2049, 8192])
 def test_power_search_one_block_and_grid(S, P):
     """Sizes on both sides of the single-block search, with dead particles:
