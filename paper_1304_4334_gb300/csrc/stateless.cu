@@ -68,8 +68,9 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // that returns a number synchronises, so a call after a device-wide wait paid
 // 200 us for mapping its memory again (random walk, K=2, I=2, 65,536 x 5,000:
 // first call after a wait 545 -> 341 us; power search, S phase and covariance
-// at 1,024 particles: 475 -> 250 us; calls in a row cost the same).  What is kept serves every stream and thread (the pool orders
-// reuse between streams itself); smc_release_workspace() gives it back.
+// at 1,024 particles: 475 -> 250 us; calls in a row cost the same).  What is kept
+// serves every stream and thread (the pool orders reuse between streams
+// itself); smc_release_workspace() gives it back.
 constexpr uint64_t kPoolKeep = 512ull << 20;
 constexpr int kMaxPools = 64;
 std::mutex g_pool_mu;
@@ -89,12 +90,16 @@ cudaError_t pool_of_device(cudaMemPool_t* out)
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
         cudaMemPool_t pool = nullptr;
-        e = cudaMemPoolCreate(&pool, &props);
+        // (the first call may be one that a stream capture records)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        e = cudaThreadExchangeStreamCaptureMode(&mode);
         if (e != cudaSuccess) return e;
         uint64_t keep = kPoolKeep;
-        e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        e = cudaMemPoolCreate(&pool, &props);
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (e != cudaSuccess) {
-            cudaMemPoolDestroy(pool);
+            if (pool) cudaMemPoolDestroy(pool);
             return e;
         }
         g_pool[dev] = pool;
