@@ -109,7 +109,7 @@ def mala_ops_per_eval(K, I, gamma):
 NOMINAL_RATES = {"ffma": 128.0, "ffma2": 128.0, "ex2": 32.0, "issue": 4.0}
 
 
-def alu_peak_evals(K, I, gamma, sms, mhz, paired=False, mala=False, rates=None):
+def alu_peak_evals(K, I, gamma, sms, mhz, paired=False, mala=False, rates=None, mix_pairs=False):
     """Evaluations/s bound at the given SM clock from the FP32 pipe, the SFU
     (ex2/lg2) and instruction issue.  `rates` are per SM and clock: lane
     operations of FFMA ("ffma"), of the paired FFMA2 ("ffma2") and of MUFU.EX2
@@ -118,13 +118,16 @@ def alu_peak_evals(K, I, gamma, sms, mhz, paired=False, mala=False, rates=None):
     instruction once), else the measured rates of smc_peaks.  With paired FP32
     instructions (two particles per thread) an FP32 instruction carries two
     lanes' work, so issue counts fp32/2 + mufu per evaluation while the FP32
-    pipe (at the FFMA2 rate) still bounds fp32."""
+    pipe (at the FFMA2 rate) still bounds fp32.  mix_pairs: one particle per
+    thread with the mixture terms of two observations in paired instructions
+    (5 instructions fewer per two observations at I = 2, 3 I - 1 above)."""
     r = dict(NOMINAL_RATES)
     if rates:
         r.update({k: v for k, v in rates.items() if k in r and v})
     fp32, mufu = (mala_ops_per_eval if mala else alu_ops_per_eval)(K, I, gamma)
-    limits = {"issue": 32.0 * r["issue"] / ((fp32 / 2.0 if paired else fp32) + mufu),
-              "fp32": (r["ffma2"] if paired else r["ffma"]) / fp32, "mufu": r["ex2"] / mufu}
+    saved = {1: 0, 2: 5}.get(I, 3 * I - 1) / 2.0 if mix_pairs else 0.0
+    limits = {"issue": 32.0 * r["issue"] / ((fp32 / 2.0 if paired else fp32 - saved) + mufu),
+              "fp32": (r["ffma2"] if paired or mix_pairs else r["ffma"]) / fp32, "mufu": r["ex2"] / mufu}
     pipe = min(limits, key=limits.get)
     return sms * mhz * 1e6 * limits[pipe], pipe
 
@@ -686,12 +689,13 @@ def main():
     traffic = MUTATE_TRAFFIC.get((args.workload, shape[0], shape[1])) if not mala else None
     mhz, src = sm_max_mhz()
     paired = shape[0] == 2
+    pairs = not paired and not mala   # (the FP64 workload has I = 1: nothing to pair)
     # MALA's bound counts its forward, recomputation and reverse sweep per
     # evaluation (mala_ops_per_eval).  The pipe rates per SM and clock are
     # those the microbenchmark measured on this device before the timed region
     # (smc_peaks), at the maximum SM clock; the nominal rates give a second bound.
-    peak, pipe = alu_peak_evals(w.K, w.I, w.gamma, SM_COUNT_GB300, mhz, paired, mala, rates=rates)
-    peak_nom, pipe_nom = alu_peak_evals(w.K, w.I, w.gamma, SM_COUNT_GB300, mhz, paired, mala)
+    peak, pipe = alu_peak_evals(w.K, w.I, w.gamma, SM_COUNT_GB300, mhz, paired, mala, rates=rates, mix_pairs=pairs)
+    peak_nom, pipe_nom = alu_peak_evals(w.K, w.I, w.gamma, SM_COUNT_GB300, mhz, paired, mala, mix_pairs=pairs)
     avg_launch_s = (mut_ms / mut_n) / 1e3 if mut_n else float("nan")
     if args.tempering == "power":
         achieved = w.P * w.T / avg_launch_s if mut_n else float("nan")
@@ -719,7 +723,7 @@ def main():
                              "autotune_ms_per_iteration": shape[2]}}
     if clk.get("sm_mhz"):
         roof["frac_at_median_clock"] = achieved / alu_peak_evals(w.K, w.I, w.gamma, SM_COUNT_GB300, clk["sm_mhz"],
-                                                                 paired, mala, rates=rates)[0]
+                                                                 paired, mala, rates=rates, mix_pairs=pairs)[0]
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu:
