@@ -291,8 +291,11 @@ struct EgarchFx {
         ly = (uint64_t)(ok ? fx_round(lyd * 0x1p55) + fx_round(lye * 0x1p55) : 0) ^ (1ull << 63);
         double cmax = 0.0;
 #pragma unroll
-        for (int k = 0; k < K; ++k) cmax = fmax(cmax, g * (beta[k] + std::fabs(gamma[k])));
-        ok = ok && cmax < 15.8;
+        for (int k = 0; k < K; ++k) {
+            const double c = g * (beta[k] + std::fabs(gamma[k]));
+            ok = ok && c < 15.8;   // (each by itself: a NaN fails it, fmax would drop it)
+            cmax = fmax(cmax, c);
+        }
         cs = cmax < 0.99 ? 0 : (cmax < 3.96 ? 2 : 4);
         const double cunit = cs == 0 ? 0x1p60 : (cs == 2 ? 0x1p58 : 0x1p56);
 #pragma unroll

@@ -152,3 +152,42 @@ def test_fixed_point_recursion_against_long_double(tmp_path):
         assert bad == "0", (K, I, T)
         assert float(fx) <= max(float(dbl), float(mag) * 2.0 ** -52), (K, I, T, fx, dbl, mag)
         assert float(state) <= 100 * 2.0 ** -52, (K, I, T, state)
+
+
+SETUP = r"""
+#include <cstdio>
+#include "HEADER"
+#define __device__
+#include "TABLE"
+using namespace smc;
+// every parameter in turn NaN, inf, -inf: setup() must send the particle to FP64
+template <int K, int I> int test() {
+    int wrong = 0;
+    const double bad[] = {NAN, INFINITY, -INFINITY};
+    for (int j = -1; j < 2 + 3 * K + (I > 1 ? 3 * I : 0); ++j)
+        for (double x : bad) {
+            double v[2 + 3 * K + 3 * I] = {0.0003, -4.6};
+            for (int k = 0; k < K; ++k) v[2 + k] = 0.9, v[2 + K + k] = 0.1, v[2 + 2 * K + k] = -0.05;
+            for (int i = 0; i < I; ++i) v[2 + 3 * K + i] = 1.0 / I, v[2 + 3 * K + I + i] = 0.0, v[2 + 3 * K + 2 * I + i] = 1.0;
+            if (j >= 0) v[j] = x;
+            EgarchFx<K, I> f;
+            f.setup(v[0], v[1], v + 2, v + 2 + K, v + 2 + 2 * K, v + 2 + 3 * K, v + 2 + 3 * K + I,
+                    v + 2 + 3 * K + 2 * I, 0, 1.0 / log(2.0));
+            if ((f.bad != 0u) != (j >= 0)) ++wrong, printf("K=%d I=%d parameter %d value %g: bad %u\n", K, I, j, x, f.bad);
+        }
+    return wrong;
+}
+int main() { return test<1, 1>() + test<2, 2>() + test<3, 4>() + test<4, 3>() ? 1 : 0; }
+"""
+
+
+def test_setup_refuses_every_parameter_that_is_not_finite(tmp_path):
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("no host C++ compiler")
+    src = tmp_path / "setup.cpp"
+    src.write_text(SETUP.replace("HEADER", HEADER).replace("TABLE", TABLE))
+    exe = tmp_path / "setup"
+    subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout

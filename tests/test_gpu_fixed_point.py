@@ -168,3 +168,41 @@ def test_likelihood_kernels_of_few_and_many_particles(S, K, I_, T):
     assert sane.sum() > P // 2
     np.testing.assert_allclose(l1[sane], l2[sane], rtol=1e-9)
     np.testing.assert_allclose(s1[sane], s2[sane], rtol=1e-9, atol=1e-12)
+
+
+def _few_and_many(S, K, I_, spec, y, th, grad):
+    """Likelihoods (and gradients) of the same particles from the kernels of a
+    small call and of a large one."""
+    torch = torch_cuda()
+    n = 200 * torch.cuda.get_device_properties(0).multi_processor_count
+    out = []
+    for tt in (th, np.resize(th, (n, spec.d))):
+        ll = torch.empty(len(tt), dtype=torch.float64, device="cuda")
+        st = torch.empty((K + 1, len(tt)), dtype=torch.float64, device="cuda")
+        if grad:
+            g = torch.empty((spec.d, len(tt)), dtype=torch.float64, device="cuda")
+            S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(tt), ll, g, st)
+        else:
+            S.loglik(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(tt), ll, None, st)
+        out.append(host(ll)[:len(th)])
+    return out
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (2, 2), (3, 4)])
+@pytest.mark.parametrize("grad", [False, True])
+def test_parameters_that_are_not_finite(S, K, I_, grad):
+    """Each parameter in turn NaN, inf or -inf: the log likelihood is the
+    oracle's, -inf for every NaN, in every kernel."""
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 100, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    values = [np.nan, np.inf, -np.inf]
+    th = np.repeat(particles(spec.d, truth, K, I_, True, 1, 85), 3 * spec.d, axis=0)
+    for j in range(spec.d):
+        th[3 * j:3 * j + 3, j] = values
+    ll_o = O.loglik(spec, y, th)
+    assert np.all(ll_o[::3] == -np.inf)
+    for ll in _few_and_many(S, K, I_, spec, y, th, grad):
+        assert np.all(ll[::3] == -np.inf), np.flatnonzero(ll[::3] != -np.inf)
+        np.testing.assert_allclose(ll[np.isfinite(ll_o)], ll_o[np.isfinite(ll_o)], rtol=1e-9)
+        assert np.all(ll[~np.isfinite(ll_o)] == -np.inf)
