@@ -110,15 +110,17 @@ __device__ __noinline__ double weights_f64(const EgarchParams<double, K, I>& q, 
         mx = fmax(mx, x[i]);
     }
     uint64_t s = 0;
+    bool nan = false;   // (fmax drops a NaN, fx_exp_q61 takes it for 0)
 #pragma unroll
     for (int i = 0; i < I; ++i) {
+        nan = nan || fx_isnan(x[i]);
         r[i] = fx_exp_q61(mx - x[i], tab);
         s += r[i];
     }
     const uint64_t Y = fx_rcp(s);
 #pragma unroll
     for (int i = 0; i < I; ++i) r[i] = fx_mulhi(r[i], Y);
-    return isnan(eps) ? eps : mx + log((double)s * 0x1p-61);
+    return nan ? (double)NAN : mx + log((double)s * 0x1p-61);
 }
 
 template <int K, int I, int kSeg>

@@ -71,6 +71,8 @@ SMC_FX uint64_t fx_bits(double x)
 #endif
 }
 
+SMC_FX bool fx_isnan(double x) { return (fx_bits(x) << 1) > 0xffe0000000000000ull; }
+
 SMC_FX uint32_t fx_mulhi32(uint32_t a, uint32_t b)
 {
 #if defined(__CUDA_ARCH__)

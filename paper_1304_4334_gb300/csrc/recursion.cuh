@@ -530,7 +530,8 @@ struct EgarchF64 {
 
     // One observation: log p - log s_t, with s_t (I >= 2; units 2^-61) apart.
     // An infinite or NaN shock makes the largest term x_i, and with it the
-    // result, infinite or NaN.
+    // result, infinite or NaN; a single term that is NaN (a component whose
+    // sigma_i is zero) makes the result NaN.
     template <bool kFirst>
     __device__ __forceinline__ double terms(double y, uint64_t& s)
     {
@@ -564,9 +565,14 @@ struct EgarchF64 {
                 x[i] = lo;
             }
             s = 1ull << 61;
+            bool nan = false;   // (fx_exp_q61 takes one for 0; x[0]'s own stays in m)
 #pragma unroll
-            for (int i = 1; i < I; ++i) s += fx_exp_q61(m - x[i], tab);
-            return m - lh;
+            for (int i = 1; i < I; ++i) {
+                const double w = m - x[i];
+                nan = nan || fx_isnan(w);
+                s += fx_exp_q61(w, tab);
+            }
+            return nan ? (double)NAN : m - lh;
         }
     }
 

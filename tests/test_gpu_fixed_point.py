@@ -206,3 +206,24 @@ def test_parameters_that_are_not_finite(S, K, I_, grad):
         assert np.all(ll[::3] == -np.inf), np.flatnonzero(ll[::3] != -np.inf)
         np.testing.assert_allclose(ll[np.isfinite(ll_o)], ll_o[np.isfinite(ll_o)], rtol=1e-9)
         assert np.all(ll[~np.isfinite(ll_o)] == -np.inf)
+
+
+@pytest.mark.parametrize("K,I_", [(1, 2), (2, 2), (3, 4)])
+@pytest.mark.parametrize("grad", [False, True])
+def test_mixture_parameters_past_the_exponentials_range(S, K, I_, grad):
+    """Each mixture parameter in turn at +-400 and +-800, where its exponential
+    or the component's standard deviation under- or overflows: a component with
+    sigma_i = 0 has a density that is NaN, and so -inf, whichever its place."""
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 100, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    values = [-800.0, -400.0, 400.0, 800.0]
+    th = np.repeat(particles(spec.d, truth, K, I_, True, 1, 87), 4 * 3 * I_, axis=0)
+    for j in range(3 * I_):
+        th[4 * j:4 * j + 4, spec.d - 3 * I_ + j] = values
+    ll_o = O.loglik(spec, y, th)
+    sane = ll_o > -1e7
+    assert np.all(ll_o[4 * 2 * I_::4] == -np.inf)      # sigma_i = exp(-800)
+    for ll in _few_and_many(S, K, I_, spec, y, th, grad):
+        np.testing.assert_allclose(ll[sane], ll_o[sane], rtol=1e-9)
+        assert np.all(ll[~sane] < -1e6), np.flatnonzero(~(ll < -1e6) & ~sane)
