@@ -6,50 +6,51 @@
 #include "loglik_split.cuh"
 #include "phase.cuh"
 
-#include <type_traits>
-
 namespace smc {
 
 inline int mutate_grid(int P, int threads = kMutThreads) { return (P + threads - 1) / threads; }
 
-// The kernel variant for P particles (one per thread): the policy's Wide form,
-// where it has one, while the particles leave the SMs room for it.
-template <class Pol, class = void>
-struct KernelPick {
-    static void (*mutate(int))(MutateArgs) { return k_mutate<Pol>; }
-    static void (*loglik(int))(LoglikArgs) { return k_loglik<Pol>; }
-};
+// The kernel for P particles (one per thread): the policy's form for few
+// particles (Few) up to the warps per SM that the policy gives.
 template <class Pol>
-struct KernelPick<Pol, std::enable_if_t<!std::is_same_v<typename Pol::Wide, Pol> && (Pol::kNi > 1)>> {
-    static bool wide(int P) { return P <= kWideWarpsPerSm * 32 * device_sm_count(); }
-    static void (*mutate(int P))(MutateArgs) { return wide(P) ? k_mutate<typename Pol::Wide> : k_mutate<Pol>; }
-    static void (*loglik(int P))(LoglikArgs) { return wide(P) ? k_loglik<typename Pol::Wide> : k_loglik<Pol>; }
+struct KernelPick {
+    static bool few(int P, int warps) { return P <= warps * 32 * device_sm_count(); }
+    template <bool kIndep>
+    static void (*mutate(int P))(MutateArgs)
+    {
+        constexpr int w = kIndep ? Pol::kFewIndep : Pol::kFewMutate;
+        if constexpr (w > 0)
+            if (few(P, w)) return k_mutate<typename Pol::Few, kIndep>;
+        return k_mutate<Pol, kIndep>;
+    }
+    static void (*loglik(int P))(LoglikArgs)
+    {
+        if constexpr (Pol::kFewLoglik > 0)
+            if (few(P, Pol::kFewLoglik)) return k_loglik<typename Pol::Few>;
+        return k_loglik<Pol>;
+    }
 };
+
+template <template <int, int> class Pol, int K, bool kIndep>
+void (*mutate_kernel(int I, int P))(MutateArgs)
+{
+    switch (I) {
+    case 1: return KernelPick<Pol<K, 1>>::template mutate<kIndep>(P);
+    case 2: return KernelPick<Pol<K, 2>>::template mutate<kIndep>(P);
+    case 3: return KernelPick<Pol<K, 3>>::template mutate<kIndep>(P);
+    case 4: return KernelPick<Pol<K, 4>>::template mutate<kIndep>(P);
+    }
+    return nullptr;
+}
 
 // One particle per thread; threads = a multiple of 32 up to kMutMaxThreads (the caller checks).
 template <template <int, int> class Pol, int K>
 cudaError_t launch_mutate_k(const MutateArgs& a, int threads, cudaStream_t s)
 {
     const int g = mutate_grid(a.P, threads);
-    if (a.qmean) {   // independent sampler
-        switch (a.m.I) {
-        case 1: k_mutate<Pol<K, 1>, true><<<g, threads, 0, s>>>(a); break;
-        case 2: k_mutate<Pol<K, 2>, true><<<g, threads, 0, s>>>(a); break;
-        case 3: k_mutate<Pol<K, 3>, true><<<g, threads, 0, s>>>(a); break;
-        case 4: k_mutate<Pol<K, 4>, true><<<g, threads, 0, s>>>(a); break;
-        default: return cudaErrorInvalidValue;
-        }
-        return cudaGetLastError();
-    }
-    void (*k)(MutateArgs) = nullptr;
-    switch (a.m.I) {
-    case 1: k = KernelPick<Pol<K, 1>>::mutate(a.P); break;
-    case 2: k = KernelPick<Pol<K, 2>>::mutate(a.P); break;
-    case 3: k = KernelPick<Pol<K, 3>>::mutate(a.P); break;
-    case 4: k = KernelPick<Pol<K, 4>>::mutate(a.P); break;
-    default: return cudaErrorInvalidValue;
-    }
-    if (a.dependent) return pdl_launch(k, g, threads, 0, s, a);
+    const auto k = a.qmean ? mutate_kernel<Pol, K, true>(a.m.I, a.P) : mutate_kernel<Pol, K, false>(a.m.I, a.P);
+    if (!k) return cudaErrorInvalidValue;
+    if (a.dependent && !a.qmean) return pdl_launch(k, g, threads, 0, s, a);
     k<<<g, threads, 0, s>>>(a);
     return cudaGetLastError();
 }

@@ -132,7 +132,7 @@ __device__ __forceinline__ void pit_setup_egarch(const ModelDev& m, const double
     }
 }
 
-template <int K, int I, bool kDelta>
+template <int K, int I, bool kDelta, bool kPair>
 struct PolicyEgarchF32T {
     using Real = float;
     using Obs = float;
@@ -140,13 +140,13 @@ struct PolicyEgarchF32T {
     using Model = EgarchF32<K, I, kDelta>;
     static constexpr int kNs = K + 1;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;   // Table 1
-    static constexpr int kBound = I == 1 ? 256 : kMutMaxThreads, kMinBlocks = 0, kLoglikBlocks = 0;
+    static constexpr int kBound = kPair ? kMutMaxThreads : 256, kMinBlocks = 0, kLoglikBlocks = 0;
     static constexpr bool kExpTab = false;
     __device__ static void setup(Model& mdl, const ModelDev& m, const Real* full, const uint64_t* = nullptr)
     {
         mdl.setup(full, m.gamma, m.eps0_zero);
     }
-    __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f32(mdl, pipe, T); }
+    __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f32<kPair>(mdl, pipe, T); }
     __device__ static void state_out(const Model& mdl, double* st) { mdl.state_out(st); }
     __device__ static void load_state(Model& mdl, const double* st) { mdl.load_state(st); }
     __device__ static double logdens(Model& mdl, const Obs* obs, int s, int)
@@ -172,15 +172,44 @@ struct PolicyEgarchF32T {
 // The FP32 recursion of the M phase (alpha v as one FMA) and, for the kernels
 // that see raw prior draws (the stand-alone likelihood and the data-tempering
 // C phase), the form that carries 1 - alpha (EgarchF32's kDelta).
+//
+// Few: the form for few particles, up to kFewMutate, kFewIndep (independent
+// sampler) or kFewLoglik warps per SM (0: none).  Paired mixture instructions
+// save issue slots where the schedulers are full (EgarchF32::mix2); with one or
+// two warps per scheduler the launch is bound by a warp's own chain, which the
+// pairing makes longer (the first observation's terms wait for the second's
+// shock).  Random walk at T=1500, scalar -> paired, 15,000 and 38,912 particles:
+// K=1,I=2 48.1 -> 51.5, 57.0 -> 59.7 us; K=2,I=3 68.6 -> 73.9, 89.7 -> 92.6;
+// K=2,I=4 68.5 -> 84.1, 98.3 -> 106.4; K=3,I=4 82.8 -> 86.4, 113.0 -> 113.8; from
+// 60,000 on the paired form is ahead (148 -> 138, 165 -> 160, 191 -> 178).  Two
+// models are compiled to a schedule that is ahead at every size (K=2,I=2 56.2 ->
+// 53.5, 66.8 -> 65.5 us; K=4,I=4 99.6 -> 96.0, 132 -> 127), one only later (K=4,I=2
+// 119.5 -> 123.8 us at 50,000, 148.6 -> 146.3 at 60,000).
+constexpr int mutate_scalar_warps(int K, int I)
+{
+    if (I == 1 || (K == I && I % 2 == 0)) return 0;
+    return K == 4 && I == 2 ? 12 : 8;
+}
 template <int K, int I>
-struct PolicyEgarchF32 : PolicyEgarchF32T<K, I, false> {};
+struct PolicyEgarchF32 : PolicyEgarchF32T<K, I, false, (I > 1)> {
+    using Few = PolicyEgarchF32T<K, I, false, false>;
+    static constexpr int kFewMutate = mutate_scalar_warps(K, I), kFewIndep = kFewMutate, kFewLoglik = 0;
+};
+// Paired at I = 2 (K=1 49.2 -> 42.7 us at 2,000 x 1,500, K=2 49.2 -> 45.2, K=4 55.4 ->
+// 57.5: scalar there up to 8 warps per SM).  At I >= 3 the longer chain of the
+// 1 - alpha form leaves the paired mixture exposed with a warp per scheduler
+// (K=2,I=3, 10,007 x 4,000: 116 -> 139 us), and from 30,000 particles both take
+// the same.
 template <int K, int I>
-struct PolicyEgarchF32Delta : PolicyEgarchF32T<K, I, true> {};
+struct PolicyEgarchF32Delta : PolicyEgarchF32T<K, I, true, I == 2> {
+    using Few = PolicyEgarchF32T<K, I, true, false>;
+    static constexpr int kFewMutate = 0, kFewIndep = 0, kFewLoglik = K == 4 && I == 2 ? 8 : 0;
+};
 
 // FP64: the fixed-point recursion for whole series (PolicyEgarchF64Fx: M phase,
 // stand-alone likelihood), the FP64 recursion observation by observation
 // (PolicyEgarchF64: data-tempering C phase).
-// kWide: no register cap.  Two blocks of 224 per SM (128 registers) are faster
+// kWide (the form for few particles): no register cap.  Two blocks of 224 per SM (128 registers) are faster
 // where the particles fill them (65,536 x 2,000: K=3, I=4 4.0 ms against 4.3 ms
 // with 255 registers, K=2, I=3 2.83 against 3.53 ms; K=2, I=2, x 5,000: 5.14
 // against 6.06 ms); with at most 10 warps per SM the kernel is bound by each
@@ -192,7 +221,7 @@ struct PolicyEgarchF64FxT {
     using Obs = double;
     static constexpr int kChunk = kChunkF64;
     using Model = EgarchFxSafe<K, I>;
-    static constexpr int kNs = K + 1, kNi = I;
+    static constexpr int kNs = K + 1;
     static constexpr int kMaxFree = I == 1 ? 2 + 3 * K : 2 + 3 * K + 3 * I;
     static constexpr int kBound = kMutMaxThreads, kMinBlocks = kWide ? 0 : 2;   // (0: no minimum)
     static constexpr int kLoglikBlocks = kWide ? 1 : 4;
@@ -207,9 +236,9 @@ struct PolicyEgarchF64FxT {
 
 template <int K, int I>
 struct PolicyEgarchF64Fx : PolicyEgarchF64FxT<K, I> {
-    using Wide = PolicyEgarchF64FxT<K, I, true>;
+    using Few = PolicyEgarchF64FxT<K, I, true>;
+    static constexpr int kFewMutate = I > 1 ? 10 : 0, kFewIndep = 0, kFewLoglik = kFewMutate;
 };
-constexpr int kWideWarpsPerSm = 10;
 
 template <int K, int I>
 struct PolicyEgarchF64 {

@@ -383,14 +383,12 @@ struct EgarchF32 {
         }
     }
 
-    // (The 1 - alpha form with I >= 3 stays scalar: with a warp per scheduler
-    // its longer chain leaves the paired mixture exposed, K=2, I=3, 10,007
-    // particles x 4,000: 139 us against 116 us, and from 30,000 particles both
-    // take the same.)
-    template <bool kFirst>
+    // kPair: the mixture terms of two observations in paired instructions
+    // (bitwise the scalar ones; the kernels' policies say which).
+    template <bool kFirst, bool kPair>
     __device__ __forceinline__ void step2(float y0, float y1, const MixPair& q)
     {
-        if constexpr (kDelta && I >= 3) {
+        if constexpr (!kPair) {
             step<kFirst>(y0);
             step<false>(y1);
             return;
@@ -830,7 +828,7 @@ constexpr int kChunkF64 = 512;    // elements per staged chunk (4 KB)
 // through `pipe`.  Every thread of the block must call it (it contains block
 // barriers); `active` selects whose result matters.  Returns false on a
 // staging timeout.
-template <int K, int I, bool kDelta>
+template <bool kPair, int K, int I, bool kDelta>
 __device__ __forceinline__ bool run_egarch_f32(EgarchF32<K, I, kDelta>& mdl, ObsPipe<float, kChunkF32>& pipe,
                                                int T)
 {
@@ -847,20 +845,20 @@ __device__ __forceinline__ bool run_egarch_f32(EgarchF32<K, I, kDelta>& mdl, Obs
             const float4* y4 = reinterpret_cast<const float4*>(yb + 32 * u);
             if (c == 0 && u == 0) {
                 float4 q = y4[0];
-                mdl.template step2<true>(q.x, q.y, mp);
-                mdl.template step2<false>(q.z, q.w, mp);
+                mdl.template step2<true, kPair>(q.x, q.y, mp);
+                mdl.template step2<false, kPair>(q.z, q.w, mp);
 #pragma unroll
                 for (int j = 1; j < 8; ++j) {
                     q = y4[j];
-                    mdl.template step2<false>(q.x, q.y, mp);
-                    mdl.template step2<false>(q.z, q.w, mp);
+                    mdl.template step2<false, kPair>(q.x, q.y, mp);
+                    mdl.template step2<false, kPair>(q.z, q.w, mp);
                 }
             } else {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float4 q = y4[j];
-                    mdl.template step2<false>(q.x, q.y, mp);
-                    mdl.template step2<false>(q.z, q.w, mp);
+                    mdl.template step2<false, kPair>(q.x, q.y, mp);
+                    mdl.template step2<false, kPair>(q.z, q.w, mp);
                 }
             }
             mdl.flush();

@@ -604,3 +604,78 @@ def test_power_search_one_block_and_grid(S, P):
     assert abs(dphi - d_o) <= 1e-4 * d_o + 1e-12, (dphi, d_o)
     w = np.exp(dphi * (ll - ll.max()))
     np.testing.assert_allclose(rss, w.sum() ** 2 / (P * (w ** 2).sum()), rtol=1e-11)
+
+
+# Warps per SM at which a call's kernel or launch shape changes (one particle
+# or two per thread; forms for few particles; register caps).
+FORM_EDGES = [4, 8, 10, 12, 21, 40, 54, 160]
+
+
+@pytest.mark.parametrize("precision,K,I_", [("fp32", 1, 1), ("fp32", 2, 1), ("fp32", 3, 1), ("fp32", 1, 2),
+                                            ("fp32", 2, 2), ("fp32", 4, 2), ("fp32", 2, 3), ("fp32", 3, 4),
+                                            ("fp32", 4, 4), ("fp64", 1, 1), ("fp64", 2, 2), ("fp64", 3, 4)])
+@pytest.mark.parametrize("sampler", ["rw", "indep"])
+def test_mutation_forms_are_bitwise_alike(S, precision, K, I_, sampler):
+    """The first particles of calls on both sides of every size at which the
+    kernel or its shape changes are the same bits: the forms differ in how
+    instructions are paired, registers capped and particles spread, not in what
+    they compute."""
+    torch = torch_cuda()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    prec = S.FP64 if precision == "fp64" else S.FP32
+    truth = egarch_truth(K, I_)
+    T, n = 65, 77
+    y = I.simulate_egarch(truth, T, seed=91)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    th = particles(spec.d, truth, K, I_, True, n, 93)
+    m = S.model_egarch(K, I_, True)
+    obs = dev(y, torch.float64 if prec == S.FP64 else torch.float32)
+    # (0.05: the cloud's own spread, at which the independent sampler accepts)
+    L = dev(np.diag(np.full(spec.d, 0.02 if sampler == "rw" else 0.05)))
+    want = None
+    for P in [n] + [32 * sms * w + more for w in FORM_EDGES for more in (0, 1)]:
+        if prec == S.FP64 and P > 32 * sms * 22:
+            continue
+        x = soa(th).repeat(1, -(-P // n))[:, :P].contiguous()
+        ll, lp = (torch.empty(P, dtype=torch.float64, device="cuda") for _ in range(2))
+        st = torch.empty((K + 1, P), dtype=torch.float64, device="cuda")
+        S.loglik(m, prec, obs, x[:, :n].contiguous(), ll[:n], lp[:n], st0 := st[:, :n].contiguous())
+        for t in (ll, lp):
+            t[:] = t[:n].repeat(-(-P // n))[:P]
+        st = st0.repeat(1, -(-P // n))[:, :P].contiguous()
+        if sampler == "rw":
+            S.mutate_rw(m, prec, obs, x, ll, lp, st, L, 0.5, 9, 2, 3)
+        else:
+            S.mutate_indep(m, prec, obs, x, ll, lp, st, dev(th.mean(axis=0)), L, 0.5, 9, 2, 3)
+        got = [host(x[:, :n]), host(ll[:n]), host(lp[:n]), host(st[:, :n])]
+        if want is None:
+            want = got
+            assert 0 < np.any(got[0].T != th, axis=1).sum() < n
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b), P
+
+
+@pytest.mark.parametrize("precision,K,I_", [("fp32", 2, 2), ("fp32", 4, 2), ("fp64", 2, 2), ("fp64", 3, 4)])
+def test_likelihood_forms_are_bitwise_alike(S, precision, K, I_):
+    """As above for the stand-alone likelihood; in FP64 above the sizes that
+    several warps per 32 particles take, whose last bits differ."""
+    torch = torch_cuda()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    prec = S.FP64 if precision == "fp64" else S.FP32
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 65, seed=95)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    n = 77
+    th = particles(spec.d, truth, K, I_, True, n, 97)
+    obs = dev(y, torch.float64 if prec == S.FP64 else torch.float32)
+    want = None
+    for w in [5, 8, 10, 12]:
+        for P in (32 * sms * w, 32 * sms * w + 1):
+            x = soa(th).repeat(1, -(-P // n))[:, :P].contiguous()
+            ll, lp = (torch.empty(P, dtype=torch.float64, device="cuda") for _ in range(2))
+            st = torch.empty((K + 1, P), dtype=torch.float64, device="cuda")
+            S.loglik(S.model_egarch(K, I_, True), prec, obs, x, ll, lp, st)
+            got = [host(ll[:n]), host(lp[:n]), host(st[:, :n])]
+            want = want or got
+            for a, b in zip(got, want):
+                assert np.array_equal(a, b), P
