@@ -67,23 +67,41 @@ static int balanced_threads(int P, int ppt)
     return kMutMaxThreads;
 }
 
+// Warps on the fullest SM when `warps` warps are launched `per_block` at a time.
+static int fullest_sm(int warps, int per_block)
+{
+    const int blocks = (warps + per_block - 1) / per_block, sms = device_sm_count();
+    return (blocks + sms - 1) / sms * per_block;
+}
+
 // Blocks of up to 224 threads, sized to the SM count, while more than four warps
-// per SM are there and at most three such blocks per SM hold them (the SMs are
-// then evenly loaded: K=2, I=2, 65,536 x 2,000 in FP32 0.125 ms against
-// 0.128 ms in 128-thread blocks, in FP64 2.18 against 2.24 ms; 98,304: 0.178
-// against 0.182 ms), 128 beyond (131,072: 0.206 against 0.213 ms).  Two
-// particles per thread only at I = 1, where there is no mixture to pair over
-// observations, and from 40 warps per SM (K=1, 262,144 x 2,000: 0.170 against
-// 0.187 ms; 196,608: equal; K=3, I=4, 524,288: 1.41 ms against 1.29 ms with one
-// particle per thread).
+// per SM are there, at most three such blocks per SM hold them and the fullest
+// SM gets fewer warps than with 128-thread blocks (K=2, I=2, 65,536 x 2,000 in
+// FP32 0.125 ms against 0.128 ms, in FP64 2.18 against 2.24 ms; 98,304: 0.178
+// against 0.182 ms), 128 otherwise: beyond (131,072: 0.206 against 0.213 ms),
+// and where the balanced blocks only regroup as many warps, since blocks of six
+// load the four schedulers unevenly (50,000 x 1,500, 12 warps per SM as 3 x 4 and
+// as 2 x 6: K=4, I=1 94.6 and 97.9 us, K=4, I=2 119.6 and 125.4).
+//
+// Two particles per thread only at I = 1, where there is no mixture to pair over
+// observations, and where they are ahead at every size measured: K=1 from 45
+// warps per SM (x 1,000, one -> two particles per thread: 230,000 particles 1.05
+// of the speed, 450,000 1.08, 900,000 1.09; 200,000 0.98), K=2 from 54 (270,000
+// 1.03, 450,000 and 900,000 1.04; 200,000 0.96).  At K=3, 4 the last wave decides
+// (400,000 0.985 and 1.00, 780,000 0.97 and 0.99, 1,000,000 1.05 and 1.06); K=3,
+// I=4, 524,288 x 2,000: 1.29 -> 1.41 ms.
 void mutate_default_shape(const ModelDev& m, int precision, bool random_walk, int P, int* ppt, int* threads)
 {
     const int warps = (P + 31) / 32, sms = device_sm_count();
     *ppt = 1;
     *threads = kMutThreads;
     if (m.kind == SMC_LINREG) return;
-    if (warps > 4 * sms && warps <= 3 * sms * (kMutMaxThreads / 32)) *threads = balanced_threads(P, 1);
-    else if (m.I == 1 && precision == SMC_FP32 && random_walk && warps >= 40 * sms) *ppt = 2;
+    if (warps > 4 * sms && warps <= 3 * sms * (kMutMaxThreads / 32)) {
+        const int t = balanced_threads(P, 1);
+        if (fullest_sm(warps, t / 32) < fullest_sm(warps, kMutThreads / 32)) *threads = t;
+    } else if (m.I == 1 && precision == SMC_FP32 && random_walk) {
+        if (m.K <= 2 && warps >= (m.K == 1 ? 45 : 54) * sms) *ppt = 2;
+    }
 }
 
 cudaError_t launch_mutate_x2(const MutateArgs& a, int threads, cudaStream_t s)

@@ -183,12 +183,14 @@ struct PolicyEgarchF32T {
 // K=2,I=4 68.5 -> 84.1, 98.3 -> 106.4; K=3,I=4 82.8 -> 86.4, 113.0 -> 113.8; from
 // 60,000 on the paired form is ahead (148 -> 138, 165 -> 160, 191 -> 178).  Two
 // models are compiled to a schedule that is ahead at every size (K=2,I=2 56.2 ->
-// 53.5, 66.8 -> 65.5 us; K=4,I=4 99.6 -> 96.0, 132 -> 127), one only later (K=4,I=2
-// 119.5 -> 123.8 us at 50,000, 148.6 -> 146.3 at 60,000).
+// 53.5, 66.8 -> 65.5 us; K=4,I=4 99.6 -> 96.0, 132 -> 127), two only later (K=2,I=4
+// 1.005 of the scalar form's time at 50,000; K=4,I=2 1.01 at 70,000 and 90,000,
+// 235 -> 236 us at 120,000, 361 -> 355 at 200,000).
 constexpr int mutate_scalar_warps(int K, int I)
 {
     if (I == 1 || (K == I && I % 2 == 0)) return 0;
-    return K == 4 && I == 2 ? 12 : 8;
+    if (I == 2 && K == 4) return 26;
+    return I == 4 && K == 2 ? 12 : 8;
 }
 template <int K, int I>
 struct PolicyEgarchF32 : PolicyEgarchF32T<K, I, false, (I > 1)> {

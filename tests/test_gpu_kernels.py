@@ -608,7 +608,7 @@ def test_power_search_one_block_and_grid(S, P):
 
 # Warps per SM at which a call's kernel or launch shape changes (one particle
 # or two per thread; forms for few particles; register caps).
-FORM_EDGES = [4, 8, 10, 12, 21, 40, 54, 160]
+FORM_EDGES = [4, 8, 10, 12, 21, 26, 45, 54]
 
 
 @pytest.mark.parametrize("precision,K,I_", [("fp32", 1, 1), ("fp32", 2, 1), ("fp32", 3, 1), ("fp32", 1, 2),
