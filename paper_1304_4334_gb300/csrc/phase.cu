@@ -96,19 +96,32 @@ __device__ __forceinline__ void unpack_pair(int e, int& i, int& k)
     k = e - ii * (ii + 1) / 2;
 }
 
-// theta - shift rounded to FP32, without FP64 instructions: the difference of
-// the FP32 high parts is exact as a pair (TwoSum), the low parts' difference
-// joins its error term (the FP64 difference's rounding, but for ties within
-// 2^-23 of an FP32 unit).
-__device__ __forceinline__ float diff_to_f32(double th, double shift, float2 sh, bool sok)
+// theta - shift in FP32, without FP64 instructions where the FP32 parts carry it:
+// the difference of the high parts is exact as a pair (TwoSum), the low parts'
+// difference joins its error term.  The parts hold 48 of FP64's 53 bits, so the
+// result is within 2^-47 of the larger operand; where it is at least `small`,
+// 2^-16 |shift|, that is 2^-7 of FP32's unit beside the half unit of its own
+// rounding.  A smaller one (a cloud that is tight for its distance from zero) is
+// formed in FP64: the whole call at 1,048,576 x 23 takes 113 us at a spread of
+// 0.5, 122 at 1e-3, 157 at 1e-6 and below (322 with every difference in FP64
+// and one entry to a thread).
+__device__ __noinline__ float small_diff_to_f32(double th, double shift)
+{
+    // particle 0 itself and its copies: no FP64 instruction
+    const long long b = __double_as_longlong(th);
+    if (b == __double_as_longlong(shift) && (((unsigned long long)b >> 52) & 0x7ffu) != 0x7ffu) return 0.0f;
+    return __double2float_rn(th - shift);
+}
+
+__device__ __forceinline__ float diff_to_f32(double th, double shift, float2 sh, bool sok, float small)
 {
     bool ok;
     const float2 t = split_f64(th, ok);
-    if (!(ok && sok)) return diff_f64_to_f32(th, shift);
     const float s = t.x - sh.x;
     const float bv = s - t.x;
     const float e = (t.x - (s - bv)) + (-sh.x - bv);
-    return s + (e + (t.y - sh.y));
+    const float x = s + (e + (t.y - sh.y));
+    return ok && sok && fabsf(x) >= small ? x : small_diff_to_f32(th, shift);
 }
 
 // Shared memory of the partial sums: per warp a tile [64][pitch] of shifted
@@ -140,6 +153,7 @@ __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta
     __shared__ double shift[kMaxD];
     __shared__ float2 shift2[kMaxD];
     __shared__ bool shift_ok[kMaxD];
+    __shared__ float shift_small[kMaxD];
     const int nb = (d + B - 1) / B, nblk = nb * (nb + 1) / 2;
     const int nacc = d + d * (d + 1) / 2;
     const size_t Ps = (size_t)P;
@@ -148,6 +162,7 @@ __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta
     for (int i = threadIdx.x; i < d; i += blockDim.x) {
         shift[i] = theta[i * Ps];
         shift2[i] = split_f64(shift[i], shift_ok[i]);
+        shift_small[i] = fabsf(shift2[i].x) * 0x1p-16f;
     }
     __syncthreads();
     const int pitch = cov_pitch(d);
@@ -178,7 +193,7 @@ __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
                     x[u] = r + u < d && lane + 32 * h < cnt
-                               ? diff_to_f32(t[h][u], shift[r + u], shift2[r + u], shift_ok[r + u]) : 0.0f;
+                               ? diff_to_f32(t[h][u], shift[r + u], shift2[r + u], shift_ok[r + u], shift_small[r + u]) : 0.0f;
                 *reinterpret_cast<float4*>(tile + (lane + 32 * h) * pitch + r) = make_float4(x[0], x[1], x[2], x[3]);
             }
         }

@@ -679,3 +679,21 @@ def test_likelihood_forms_are_bitwise_alike(S, precision, K, I_):
             want = want or got
             for a, b in zip(got, want):
                 assert np.array_equal(a, b), P
+
+
+@pytest.mark.parametrize("d,P", [(1, 1000), (8, 70000), (23, 20000), (32, 4096)])
+@pytest.mark.parametrize("centre", [1.0, -3.7])
+@pytest.mark.parametrize("spread", [1e-4, 1e-6, 1e-12, 1e-14])
+def test_covariance_of_a_tight_cloud(S, d, P, centre, spread):
+    """A cloud far narrower than its distance from zero, on both sides of a power
+    of two or within one: theta minus particle 0 is exact in FP64, so V is as
+    accurate as for any other cloud (64 x 2^-24 of its largest entry)."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(d + P)
+    th = centre * (1.0 + spread * rng.normal(size=(P, d)))
+    mean, cov, L = (torch.empty(s, dtype=torch.float64, device="cuda") for s in ((d,), (d, d), (d, d)))
+    S.cov_chol(soa(th), 5, mean, cov, L)
+    want = np.cov((th - th[0]).T).reshape(d, d)
+    assert np.abs(host(cov) - want).max() <= 64 * 2.0 ** -24 * np.abs(want).max()
+    sd = np.sqrt(np.diag(want).max())
+    np.testing.assert_allclose(host(mean), th[0] + (th - th[0]).mean(axis=0), rtol=2.0 ** -51, atol=64 * 2.0 ** -24 * sd)
