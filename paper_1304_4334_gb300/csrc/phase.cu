@@ -73,7 +73,7 @@ __device__ __forceinline__ float2 split_f64(double d, bool& ok)
 // combination does not cancel: V = [S2 - S1 S1'/P] / (P - 1) on shifted data.
 // Within a tile of 64 particles the shifted values and their products are
 // summed in FP32 (the FP64 pipe of this part is 1/64 of its FP32 rate); tiles
-// and blocks are combined in FP64.  V only scales the random-walk proposal, so
+// are combined as FP32 pairs within a warp, in FP64 across warps and blocks.  V only scales the random-walk proposal, so
 // its ~1e-6 relative accuracy leaves the Metropolis kernel exact.
 constexpr int kCovThreads = 256;
 constexpr int kCovTile = 64;
@@ -135,11 +135,45 @@ size_t cov_smem(int d)
     return tiles > sums ? tiles : sums;
 }
 
+// The same sums with the tiles' added in FP64 one by one, for a block in which
+// the running FP32 sum is not finite (values past 1e18 of each other, infinities,
+// NaNs).  Every thread of the block calls it.
+__device__ __noinline__ void cov_partial_f64(const double* __restrict__ theta, int d, int P, double* part, int bidx,
+                                             int G, const double* shift, float* sm)
+{
+    constexpr int kPitch = kCovTile + 1;
+    const int nacc = d + d * (d + 1) / 2;
+    const int per = (P + G - 1) / G;
+    const int n0 = bidx * per, n1 = min(P, n0 + per);
+    for (int e0 = 0; e0 < nacc; e0 += kCovThreads) {
+        const int e = e0 + (int)threadIdx.x;
+        int i = 0, k = 0;
+        if (e >= d && e < nacc) unpack_pair(e - d, i, k);
+        double acc = 0.0;
+        for (int base = n0; base < n1; base += kCovTile) {
+            __syncthreads();
+            for (int x = threadIdx.x; x < d * kCovTile; x += kCovThreads) {
+                const int j = x / kCovTile, n = x % kCovTile;
+                sm[j * kPitch + n] = base + n < n1 ? __double2float_rn(theta[(size_t)j * P + base + n] - shift[j]) : 0.0f;
+            }
+            __syncthreads();
+            if (e >= nacc) continue;
+            float s = 0.0f;
+            for (int n = 0; n < kCovTile; ++n)
+                s = e < d ? s + sm[e * kPitch + n] : fmaf(sm[i * kPitch + n], sm[k * kPitch + n], s);
+            acc += (double)s;
+        }
+        if (e < nacc) part[(size_t)bidx * nacc + e] = acc;
+    }
+}
+
 // One block's partial sums: a warp per tile.  The warp stages its tile (two
 // particles a lane, four rows a store), and each lane then owns B x B products
 // x_i x_k and, on the diagonal, the B sums x_i: within a tile one FMA chain per entry in the particles'
-// order, tiles added up as exact pairs (TwoSum) and converted once, so the
-// result does not depend on B.  Bound by the FMAs' issue and the loads of theta
+// order.  A warp adds its tiles' sums up as FP32 pairs (TwoSum, Knuth: the error term is exact,
+// its running sum rounds, so n tiles leave at most n^2 2^-49 of the sum of magnitudes, 2^-43 for
+// the 7 tiles of 1,048,576 particles, against 2^-24 in each tile's own sum) and converts them
+// once; warps and blocks are added in FP64.  Bound by the FMAs' issue and the loads of theta
 // (193 MB at d = 23, 1,048,576 particles).  The first form gave one entry to a
 // thread (two 4-byte loads per FMA) and formed and converted theta - shift in
 // FP64: 307 us there, now 94 us (whole calls: 14 parameters, 70,000 particles 31
@@ -236,8 +270,14 @@ __device__ __forceinline__ void cov_partial_run(const double* __restrict__ theta
             hi[e] = a;
         }
     }
+    bool finite = true;
+#pragma unroll
+    for (int e = 0; e < kE; ++e) finite = finite && fabsf(hi[e]) < INFINITY;
+    if (__syncthreads_or(!finite)) {
+        cov_partial_f64(theta, d, P, part, bidx, G, shift, sm);
+        return;
+    }
     // the warps' sums, added per entry in the warps' order
-    __syncthreads();
     double* sums = reinterpret_cast<double*>(sm);
     if (item < nblk) {
 #pragma unroll

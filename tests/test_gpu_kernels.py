@@ -697,3 +697,36 @@ def test_covariance_of_a_tight_cloud(S, d, P, centre, spread):
     assert np.abs(host(cov) - want).max() <= 64 * 2.0 ** -24 * np.abs(want).max()
     sd = np.sqrt(np.diag(want).max())
     np.testing.assert_allclose(host(mean), th[0] + (th - th[0]).mean(axis=0), rtol=2.0 ** -51, atol=64 * 2.0 ** -24 * sd)
+
+
+@pytest.mark.parametrize("d", [1, 8, 14, 20, 28, 32])
+@pytest.mark.parametrize("P", [40000, 1 << 20])
+def test_covariance_of_a_cloud_past_the_fp32_range(S, d, P):
+    """Products of 3e18 or so: each tile's sums are FP32 numbers, the totals over
+    a block's tiles are not.  V is finite and as accurate as for any cloud."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(d)
+    th = 8e17 * rng.normal(size=(P, d)) + 1.0
+    th[0] = 0.5     # (the shift)
+    mean, cov, L = (torch.empty(s, dtype=torch.float64, device="cuda") for s in ((d,), (d, d), (d, d)))
+    S.cov_chol(soa(th), 5, mean, cov, L)
+    want = np.cov(th.T).reshape(d, d)
+    assert np.abs(host(cov) - want).max() <= 64 * 2.0 ** -24 * np.abs(want).max()
+
+
+def test_covariance_with_a_value_that_is_not_finite(S):
+    """One particle's parameter NaN or infinite: its row and column of V are not
+    finite, the other entries are those of the cloud."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(5)
+    th = rng.normal(size=(30000, 5)) + 1.0
+    for bad in (np.nan, np.inf, -np.inf):
+        x = th.copy()
+        x[12345, 2] = bad
+        mean, cov, L = (torch.empty(s, dtype=torch.float64, device="cuda") for s in ((5,), (5, 5), (5, 5)))
+        S.cov_chol(soa(x), 5, mean, cov, L)
+        c = host(cov)
+        want = np.cov(th.T)
+        keep = [0, 1, 3, 4]
+        assert not np.isfinite(c[2]).any() and not np.isfinite(c[:, 2]).any()
+        assert np.abs(c - want)[np.ix_(keep, keep)].max() <= 64 * 2.0 ** -24 * np.abs(want).max()
