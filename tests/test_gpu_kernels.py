@@ -730,3 +730,14 @@ def test_covariance_with_a_value_that_is_not_finite(S):
         keep = [0, 1, 3, 4]
         assert not np.isfinite(c[2]).any() and not np.isfinite(c[:, 2]).any()
         assert np.abs(c - want)[np.ix_(keep, keep)].max() <= 64 * 2.0 ** -24 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("d", [15, 20, 21, 28, 30, 31])
+@pytest.mark.parametrize("tiles", [1, 2, 3, 4, 5])
+def test_covariance_forms_by_tiles_per_block(S, d, tiles):
+    """The largest particle count with so many tiles in a block and the next, on
+    this device's SMs (two blocks of 64-particle tiles each)."""
+    torch = torch_cuda()
+    P = 2 * torch.cuda.get_device_properties(0).multi_processor_count * 64 * tiles
+    for n in (P, P + 1):
+        test_covariance_block_shapes_match_numpy(S, d, n)
