@@ -7,9 +7,8 @@
 //     fixed-point recursion (EgarchFx; the FP64 recursion takes particles out
 //     of its ranges);
 //   - the component weights r_i come from integer exponentials and an integer
-//     reciprocal of their sum;
-//   - the sums over t keep r_i (exact integers), r_i eps and r_i eps^2 per
-//     component, from which d log p_i, d mu_i and d a_i follow once at the end
+//     reciprocal of their sum, assembled as FP64 numbers by integer instructions;
+//   - the sums over t keep r_i, r_i eps and r_i eps^2 per component, from which d log p_i, d mu_i and d a_i follow once at the end
 //     (4 FP64 instructions per component and observation instead of 11).
 // About 40 FP64 instructions per particle and observation at K = 2, I = 2
 // against 230 with FP64 exponentials and division.
@@ -96,37 +95,34 @@ __device__ __forceinline__ void natural_to_theta_f64(const EgarchParams<double, 
     }
 }
 
-// r_i (2^-59) with the terms x_i formed in FP64 (any parameters and shock);
-// returns log sum_i exp(x_i).
+// r_i with the terms x_i formed in FP64 (any parameters and shock); returns
+// log sum_i exp(x_i).  A term that is NaN makes all of them NaN.
 template <int K, int I>
 __device__ __noinline__ double weights_f64(const EgarchParams<double, K, I>& q, double eps, const uint64_t* tab,
-                                           uint64_t* r)
+                                           double* r)
 {
-    double x[I], mx = -INFINITY;
+    double x[I], mx = -INFINITY, s = 0.0;
 #pragma unroll
     for (int i = 0; i < I; ++i) {
         const double z = (eps - q.mu[i]) / q.sig[i];
         x[i] = log(q.p[i]) - log(q.sig[i]) - 0.5 * z * z;
         mx = fmax(mx, x[i]);
     }
-    uint64_t s = 0;
-    bool nan = false;   // (fmax drops a NaN, fx_exp_q61 takes it for 0)
 #pragma unroll
     for (int i = 0; i < I; ++i) {
-        nan = nan || fx_isnan(x[i]);
-        r[i] = fx_exp_q61(mx - x[i], tab);
+        r[i] = fx_exp_neg(mx - x[i], tab);
         s += r[i];
     }
-    const uint64_t Y = fx_rcp(s);
+    const double is = 1.0 / s;
 #pragma unroll
-    for (int i = 0; i < I; ++i) r[i] = fx_mulhi(r[i], Y);
-    return nan ? (double)NAN : mx + log((double)s * 0x1p-61);
+    for (int i = 0; i < I; ++i) r[i] *= is;
+    return mx + log(s);
 }
 
 template <int K, int I, int kSeg>
 struct AdjointF64 {
     EgarchFxSafe<K, I> mdl;
-    double a2[I], m2[I];         // a_i^2, mu_i a_i^2, times 2^-59 (the units of r_i)
+    double a2[I], m2[I];         // a_i^2, mu_i a_i^2
 
     __device__ __forceinline__ void setup(const double* th, int has_gamma, int eps0_zero, const uint64_t* tab)
     {
@@ -134,7 +130,7 @@ struct AdjointF64 {
 #pragma unroll
         for (int i = 0; i < I; ++i) {
             const double a = 1.0 / mdl.q.sig[i];
-            a2[i] = a * a * 0x1p-59;
+            a2[i] = a * a;
             m2[i] = mdl.q.mu[i] * a2[i];
         }
     }
@@ -198,15 +194,13 @@ struct AdjointF64 {
     {
         constexpr int NS = 2 + 3 * K;      // mu, log sigma, alpha, beta, gamma
         constexpr int W = K + 2;
-        double gs[NS], s1[I], s2[I], vb[K];
-        uint64_t s0[I];
+        double gs[NS], s0[I], s1[I], s2[I], vb[K];
         for (int i = 0; i < NS + 3 * I; ++i) gn[i] = 0.0;
 #pragma unroll
         for (int i = 0; i < NS; ++i) gs[i] = 0.0;
 #pragma unroll
         for (int i = 0; i < I; ++i) {
-            s1[i] = s2[i] = 0.0;
-            s0[i] = 0;
+            s0[i] = s1[i] = s2[i] = 0.0;
         }
 #pragma unroll
         for (int k = 0; k < K; ++k) vb[k] = 0.0;
@@ -224,14 +218,13 @@ struct AdjointF64 {
         auto back = [&](double eps, double inv, const double* vp, double ep, bool has_prev) {
             double eb = -eps;
             if constexpr (I >= 2) {
-                uint64_t r[I];
+                double r[I];
                 if (!(fixed && fx.weights(eps * 0x1p53, r, mdl.tab))) weights_f64(mdl.q, eps, mdl.tab, r);
                 eb = 0.0;
 #pragma unroll
                 for (int i = 0; i < I; ++i) {
-                    const double ri = (double)(int64_t)r[i];
-                    const double re = ri * eps;
-                    eb = fma(-re, a2[i], fma(ri, m2[i], eb));
+                    const double re = r[i] * eps;
+                    eb = fma(-re, a2[i], fma(r[i], m2[i], eb));
                     s0[i] += r[i];
                     s1[i] += re;
                     s2[i] = fma(re, eps, s2[i]);
@@ -296,14 +289,6 @@ struct AdjointF64 {
                 back(b[K * stride], b[(K + 1) * stride], vp, bq[K * stride], true);
             }
             back(buf[K * stride], buf[(K + 1) * stride], vprev, eprev, t0 > 0);
-            if constexpr (I >= 2) {            // (r_i <= 2^59: the sum of 16 is at most 2^63)
-                static_assert(kSeg <= 16);
-#pragma unroll
-                for (int i = 0; i < I; ++i) {
-                    gn[NS + i] += (double)s0[i] * 0x1p-59;
-                    s0[i] = 0;
-                }
-            }
             if ((sg & 7) == 0) {
 #pragma unroll
                 for (int i = 0; i < NS; ++i) {
@@ -312,9 +297,10 @@ struct AdjointF64 {
                 }
 #pragma unroll
                 for (int i = 0; i < I; ++i) {
+                    gn[NS + i] += s0[i];
                     gn[NS + I + i] += s1[i];
                     gn[NS + 2 * I + i] += s2[i];
-                    s1[i] = s2[i] = 0.0;
+                    s0[i] = s1[i] = s2[i] = 0.0;
                 }
             }
         }
@@ -322,7 +308,7 @@ struct AdjointF64 {
         if constexpr (I >= 2) {
 #pragma unroll
             for (int i = 0; i < I; ++i) {
-                const double r0 = gn[NS + i], r1 = gn[NS + I + i] * 0x1p-59, r2 = gn[NS + 2 * I + i] * 0x1p-59;
+                const double r0 = gn[NS + i], r1 = gn[NS + I + i], r2 = gn[NS + 2 * I + i];
                 const double a = 1.0 / q.sig[i], mu = q.mu[i];
                 gn[NS + I + i] = a * a * (r1 - mu * r0);
                 gn[NS + 2 * I + i] = q.sig[i] * r0 - a * (r2 - mu * (2.0 * r1 - mu * r0));
@@ -603,7 +589,7 @@ struct GradSplit {
                     uint32_t over;
                     fx.mix_terms(e, sm.tab, over);
                     if (over != 0u || !fixed) {
-                        uint64_t r8[I];
+                        double r8[I];
                         fx.pm = pm;
                         fx.pe = pe;
                         fx.sc = sc;
@@ -628,15 +614,13 @@ struct GradSplit {
                   nf * (kLn2 * fx.c0);
         }
         // backward: dl/deps and the component sums
-        double a2[I], m2[I], s1[I], s2[I], g[3 * I];
-        uint64_t s0[I];
+        double a2[I], m2[I], s0[I], s1[I], s2[I], g[3 * I];
 #pragma unroll
         for (int i = 0; i < I; ++i) {
             const double ai = 1.0 / q.sig[i];
-            a2[i] = ai * ai * 0x1p-165;    // (r_i 2^59, eps 2^53, dl/deps 2^-53)
-            m2[i] = q.mu[i] * (ai * ai) * 0x1p-112;
-            s1[i] = s2[i] = 0.0;
-            s0[i] = 0;
+            a2[i] = ai * ai * 0x1p-106;    // (eps 2^53, dl/deps 2^-53)
+            m2[i] = q.mu[i] * (ai * ai) * 0x1p-53;
+            s0[i] = s1[i] = s2[i] = 0.0;
             g[i] = g[I + i] = g[2 * I + i] = 0.0;
         }
         meet();                            // (step 0 is warp 0's alone)
@@ -648,31 +632,26 @@ struct GradSplit {
 #pragma unroll 2
                 for (int r = n - 1; r >= 0; --r) {
                     const double es = b[r][K][lane];
-                    uint64_t ri[I];
+                    double ri[I];
                     if (!(fixed && fx.weights(es, ri, sm.tab))) weights_f64(q, es * 0x1p-53, sm.tab, ri);
                     double d = 0.0;
 #pragma unroll
                     for (int i = 0; i < I; ++i) {
-                        const double rd = (double)(int64_t)ri[i];
-                        const double re = rd * es;
-                        d = fma(-re, a2[i], fma(rd, m2[i], d));
+                        const double re = ri[i] * es;
+                        d = fma(-re, a2[i], fma(ri[i], m2[i], d));
                         s0[i] += ri[i];
                         s1[i] += re;
                         s2[i] = fma(re, es, s2[i]);
                     }
                     dl[r * 32] = d;
                 }
-#pragma unroll
-                for (int i = 0; i < I; ++i) {
-                    g[i] += (double)s0[i] * 0x1p-59;   // (16 r_i of at most 2^59)
-                    s0[i] = 0;
-                }
                 if ((sg & 7) == 0) {
 #pragma unroll
                     for (int i = 0; i < I; ++i) {
+                        g[i] += s0[i];
                         g[I + i] += s1[i];
                         g[2 * I + i] += s2[i];
-                        s1[i] = s2[i] = 0.0;
+                        s0[i] = s1[i] = s2[i] = 0.0;
                     }
                 }
             }
@@ -680,7 +659,7 @@ struct GradSplit {
         }
 #pragma unroll
         for (int i = 0; i < I; ++i) {
-            const double r0 = g[i], r1 = g[I + i] * 0x1p-112, r2 = g[2 * I + i] * 0x1p-112 * 0x1p-53;
+            const double r0 = g[i], r1 = g[I + i] * 0x1p-53, r2 = g[2 * I + i] * 0x1p-106;
             const double ai = 1.0 / q.sig[i], mu = q.mu[i];
             sm.comb[i][lane] = r0;
             sm.comb[I + i][lane] = ai * ai * (r1 - mu * r0);

@@ -450,10 +450,12 @@ struct EgarchFx {
         return (int64_t)((mag ^ nm64) - nm64);
     }
 
-    // Posterior weights r_i of the components (order of setup's arguments;
-    // units 2^-59) for the shock ed (units 2^-53); false where a d_i is out of range.
-    // 1 / s by two Newton steps on integers from the FP32 reciprocal.
-    SMC_FX bool weights(double ed, uint64_t* r, const uint64_t* tab) const
+    // Posterior weights r_i of the components (order of setup's arguments) for
+    // the shock ed (units 2^-53); false where a d_i is out of range.  Each is
+    // 2^-(m - d_i) / s with its own exponent, so a rare component's weight has
+    // as many bits as the others' (0 below 2^-128 of the largest): 1 / s by two
+    // Newton steps on integers from the FP32 reciprocal, no FP64 instruction.
+    SMC_FX bool weights(double ed, double* r, const uint64_t* tab) const
     {
         int64_t D[I], cur = 0;
         uint32_t over = 0;
@@ -465,27 +467,37 @@ struct EgarchFx {
             over |= o;
             cur = D[i] > cur ? D[i] : cur;
         }
-        uint64_t w[I], s = 0;
+        uint64_t w[I], s = 0;                // 2^-(m - d_i) = w 2^(-63 - n)
+        int n[I];
         if (I == 2) {   // one of the two is 1
             const uint64_t Y = (uint64_t)(2 * cur - D[1]);
-            const uint64_t e = fx_shr(fx_exp2neg(Y, tab), (int)(uint32_t)(Y >> 55) + 2);
-            w[0] = cur > 0 ? e : 1ull << 61;
-            w[1] = cur > 0 ? 1ull << 61 : e;
-            s = w[0] + w[1];
+            const uint64_t e = fx_exp2neg(Y, tab);
+            const int ne = (int)(uint32_t)(Y >> 55);
+            w[0] = cur > 0 ? e : 1ull << 63;
+            w[1] = cur > 0 ? 1ull << 63 : e;
+            n[0] = cur > 0 ? ne : 0;
+            n[1] = cur > 0 ? 0 : ne;
+            s = (1ull << 61) + fx_shr(e, ne + 2);
         } else {
 #pragma unroll
             for (int i = 0; i < I; ++i) {
                 const uint64_t Y = (uint64_t)(cur - D[i]);
-                w[i] = fx_shr(fx_exp2neg(Y, tab), (int)(uint32_t)(Y >> 55) + 2);
-                s += w[i];
+                w[i] = fx_exp2neg(Y, tab);
+                n[i] = (int)(uint32_t)(Y >> 55);
+                s += fx_shr(w[i], n[i] + 2);
             }
         }
         const uint64_t Y = fx_rcp(s);
 #pragma unroll
-        for (int i = 0; i < I; ++i) r[i] = fx_mulhi(w[i], Y);
+        for (int i = 0; i < I; ++i) {
+            const uint64_t R = fx_mulhi(w[i], Y);   // in [2^58, 2^61]: r_i = R 2^(-61 - n)
+            const int z = fx_clz64(R) - 1;
+            r[i] = fx_pack(R << z, n[i] + z - 2);
+            if (n[i] > 127) r[i] = 0.0;             // (term() gives -128 below it)
+        }
 #pragma unroll
         for (int i = 1; i < I; ++i) {
-            const uint64_t r0 = r[0], ri = r[i];
+            const double r0 = r[0], ri = r[i];
             r[0] = i == ref ? ri : r0;
             r[i] = i == ref ? r0 : ri;
         }

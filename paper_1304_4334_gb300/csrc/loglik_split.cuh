@@ -67,7 +67,7 @@ struct LoglikSplit {
                 fx.pm = pm;
                 fx.pe = pe;
                 fx.sc = sc;
-                uint64_t ri[I];
+                double ri[I];
                 sum += fixed ? relative(fx, e) : weights_f64(q, e * 0x1p-53, tab, ri);
             }
         }

@@ -191,3 +191,58 @@ def test_setup_refuses_every_parameter_that_is_not_finite(tmp_path):
     subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+WEIGHTS = r"""
+#include <cstdio>
+#include <random>
+#include "HEADER"
+#define __device__
+#include "TABLE"
+using namespace smc;
+typedef long double R;
+// largest |r / exact - 1| / ((1 + |d|) 2^-50) over components, d its log2 distance from the largest
+template <int I> double test(double spread) {
+    std::mt19937_64 g(I);
+    std::normal_distribution<double> N;
+    const double z1[1] = {0.9}, z2[1] = {0.1}, z3[1] = {0.0};
+    double worst = 0;
+    for (int rep = 0; rep < 20000; ++rep) {
+        double p[I], m[I], s[I], r[I];
+        for (int i = 0; i < I; ++i) p[i] = exp(spread * N(g)), m[i] = 0.5 * N(g), s[i] = exp(0.5 * N(g));
+        EgarchFx<1, I> f;
+        f.setup(0, -4.6, z1, z2, z3, p, m, s, 0, 1.0 / log(2.0));
+        const double e = 2 * N(g);
+        if (f.bad || !f.weights(e * 0x1p53, r, g_exp2_neg256)) continue;
+        R x[I], mx = -1e30L, sum = 0;
+        for (int i = 0; i < I; ++i) {
+            const R z = ((R)e - m[i]) / s[i];
+            x[i] = std::log((R)p[i]) - std::log((R)s[i]) - z * z / 2;
+            mx = x[i] > mx ? x[i] : mx;
+        }
+        for (int i = 0; i < I; ++i) sum += std::exp(x[i] - mx);
+        for (int i = 0; i < I; ++i) {
+            const R d = (mx - x[i]) / std::log((R)2);
+            if (d > 120) continue;
+            worst = fmax(worst, (double)(fabsl(r[i] / (std::exp(x[i] - mx) / sum) - 1) / ((1 + d) * 0x1p-50L)));
+        }
+    }
+    return worst;
+}
+int main() { printf("%g %g %g %g\n", test<2>(1), test<2>(12), test<3>(12), test<4>(12)); }
+"""
+
+
+def test_component_weights_against_long_double(tmp_path):
+    """Every weight relative to itself: d_i is a quadratic in FP64 whose terms are
+    up to a few times its own size (setup's rounding, two FMAs: 2^-50 of 1 + |d_i|,
+    in log2 units, covers them), whatever the weight's size."""
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("no host C++ compiler")
+    src = tmp_path / "weights.cpp"
+    src.write_text(WEIGHTS.replace("HEADER", HEADER).replace("TABLE", TABLE))
+    exe = tmp_path / "weights"
+    subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
+    worst = [float(v) for v in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()]
+    assert max(worst) < 8.0, worst

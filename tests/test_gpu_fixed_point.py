@@ -227,3 +227,50 @@ def test_mixture_parameters_past_the_exponentials_range(S, K, I_, grad):
     for ll in _few_and_many(S, K, I_, spec, y, th, grad):
         np.testing.assert_allclose(ll[sane], ll_o[sane], rtol=1e-9)
         assert np.all(ll[~sane] < -1e6), np.flatnonzero(~(ll < -1e6) & ~sane)
+
+
+def _gradient64(th, y, K, I_):
+    """The gradient by torch in FP64, with p_i = 2 / (1 + exp(-2 theta_i)) free of
+    cancellation (the oracle's 1 + tanh(theta_i) loses a small p_i's digits)."""
+    torch = torch_cuda()
+    t = torch.tensor(th.T.copy(), requires_grad=True)
+    j = 2 + 3 * K
+    al, be, ga = torch.tanh(t[2:2 + K]), torch.exp(t[2 + K:2 + 2 * K]), t[2 + 2 * K:j]
+    p = 2.0 / (1.0 + torch.exp(-2.0 * t[j:j + I_]))
+    p = p / p.sum(0)
+    mu, s = t[j + I_:j + 2 * I_], torch.exp(t[j + 2 * I_:])
+    mu = mu - (p * mu).sum(0)
+    c = 1.0 / torch.sqrt((p * (mu * mu + s * s)).sum(0))
+    lp, m, a = torch.log(p) - torch.log(c * s), c * mu, 1.0 / (c * s)
+    v, ll = torch.zeros_like(al), 0.0
+    for n, yt in enumerate(y):
+        if n:
+            v = al * v + be * (e.abs() - np.sqrt(2.0 / np.pi)) + ga * e
+        lh = t[1] + 0.5 * v.sum(0)
+        e = (float(yt) - t[0] / 1000.0) * torch.exp(-lh)
+        z = (e - m) * a
+        ll = ll + torch.logsumexp(lp - 0.5 * z * z, 0) - lh
+    (g,) = torch.autograd.grad(ll.sum(), t)
+    return g.numpy().T
+
+
+@pytest.mark.parametrize("K,I_", [(1, 2), (2, 3), (4, 4)])
+@pytest.mark.parametrize("theta_p", [-6.0, -12.0, -15.0])
+def test_gradient_of_a_rare_component(S, K, I_, theta_p):
+    """A last component of probability about 6e-6, 4e-11, 1e-13: its parameters'
+    gradients are as small, and as accurate for their size (1e-9; FP64 leaves
+    1e-12) as the others', in both gradient kernels."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 130, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    th = particles(spec.d, truth, K, I_, True, 40, 89)
+    th[:, spec.d - 2 * I_ - 1] = theta_p
+    want = _gradient64(th, y, K, I_)
+    last = [spec.d - 2 * I_ - 1, spec.d - I_ - 1, spec.d - 1]
+    for n in (40, 200 * torch.cuda.get_device_properties(0).multi_processor_count):
+        x = np.resize(th, (n, spec.d))
+        ll = torch.empty(n, dtype=torch.float64, device="cuda")
+        g = torch.empty((spec.d, n), dtype=torch.float64, device="cuda")
+        S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(x), ll, g)
+        np.testing.assert_allclose(host(g)[last, :40].T, want[:, last], rtol=1e-9)
