@@ -154,7 +154,7 @@ struct AdjointF64 {
             mdl.close(fx, y + t0, t0, n, T);
         }
         if (!mdl.out) mdl.fx.restore(mdl.saved);
-        mdl.state_out(st);
+        mdl.state_out(st, y + T - 1);
         return mdl.finish(T);
     }
 
@@ -266,8 +266,8 @@ struct AdjointF64 {
             fx.bad = 0;
             auto keep = [&](int r) {
                 double s[K + 1];
-                fx.state_out(s, kLn2);
-                put(buf + (size_t)r * W * stride, stride, s, s[K], fx.inv_h());
+                fx.state_out(s, kLn2);   // (its shock is not used)
+                put(buf + (size_t)r * W * stride, stride, s, fx.eps_scaled(0), fx.inv_h_scaled(0));
             };
             if (t0 == 0) fx.template chain<true>(y[0], mdl.tab);
             else fx.template chain<false>(y[t0], mdl.tab);
@@ -338,7 +338,7 @@ struct GradSplit {
     static constexpr int kSeg = 16, W = K + 2;
     static constexpr double kVu = 0x1p55 * 0.5 / kLn2;   // V_k units of v_k
     struct Smem {
-        double slab[3][kSeg][W][32];       // V_1..V_K, eps, 1/h
+        double slab[3][kSeg][W][32];       // V_1..V_K, eps, 2^53 / h
         double x[2][kSeg][32];             // forward: shocks; backward: dl/deps 2^-53
         double comb[3 * I + 2][32];        // warp 1's results
         uint64_t tab[256];
@@ -365,7 +365,7 @@ struct GradSplit {
             if (v) {
 #pragma unroll
                 for (int k = 0; k < K; ++k) v[(size_t)r * es_stride + 32 * k] = w.v[k] * kVu;
-                inv[(size_t)r * es_stride] = fx_exp_neg(lsy + 0.5 * vs, w.tab);
+                inv[(size_t)r * es_stride] = fx_exp_neg(lsy + 0.5 * vs, w.tab) * 0x1p53;
             }
         }
         return sum;
@@ -432,6 +432,7 @@ struct GradSplit {
                 if (fx.bad == 0u && !out) {
                     sx += fx.sx;
                     fx.state_out(st, kLn2);
+                    st[K] = fx.eps_scaled(0);
                 } else {
                     if (!out) w.load_state(st);
                     lh64 += segment_f64(w, q.log_sigma_y, y, t0, n, es, 32, nullptr, nullptr);
@@ -502,8 +503,8 @@ struct GradSplit {
                 auto put = [&](int r) {
 #pragma unroll
                     for (int k = 0; k < K; ++k) b[r][k][lane] = (double)fx.V[k];
-                    b[r][K][lane] = (double)fx.shock();
-                    b[r][K + 1][lane] = fx.inv_h();
+                    b[r][K][lane] = fx.eps_scaled(53);
+                    b[r][K + 1][lane] = fx.inv_h_scaled(53);
                 };
                 if (t0 == 0) fx.template chain<true>(y[0], sm.tab);
                 else fx.template chain<false>(y[t0], sm.tab);
@@ -547,7 +548,6 @@ struct GradSplit {
             }
             meet();
         }
-        gn[0] *= 0x1p53;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             gn[2 + k] *= 0.5 / kVu;

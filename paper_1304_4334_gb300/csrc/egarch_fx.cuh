@@ -275,6 +275,7 @@ struct EgarchFx {
     double c0, m0, a0;                   // component 0: log2(p / sigma), mu, 1 / sigma
     int ref;                             // its place in the caller's order
     uint64_t M, X;                       // 1 / h_t = M 2^(-63 - n), n = (X >> 55) - 256
+    double dy;                           // y_t - mu_Y
     uint32_t bad;
 
     // Natural parameters (EgarchParams) in; eps0_zero as in EgarchF64.
@@ -415,10 +416,10 @@ struct EgarchFx {
         }
         sx += X;
         const uint64_t T = tab[(uint32_t)(X >> 47) & 255u], q = fx_exp2neg_q(X);
-        M = T - (fx_mulhi(T, q) >> 8);   // (only where inv_h() is used)
+        M = T - (fx_mulhi(T, q) >> 8);   // (kept only where inv_h_scaled() is used)
         // |eps| = |y - mu| 2^-X: the 53-bit significand times M, shifted; the
         // shift passes 63 for a zero return
-        const double dy = y - mu;
+        dy = y - mu;                     // (kept only where eps_scaled() is used)
         const uint64_t b = fx_bits(dy);
         const int ed = (int)(uint32_t)(b >> 52) & 0x7ff;
         const uint64_t p0 = fx_mulhi((b << 11) | 0x8000000000000000ull, T);   // beside the polynomial
@@ -504,8 +505,19 @@ struct EgarchFx {
         return over == 0u;
     }
 
-    // 1 / h_t of the last chain().
-    SMC_FX double inv_h() const { return fx_pack(M, (int)(uint32_t)(X >> 55) - 256); }
+    // 2^e / h_t and 2^e eps_t of the last chain(), the shock with all its bits
+    // (shock() holds it in units of 2^-53).
+    SMC_FX double inv_h_scaled(int e) const { return fx_pack(M, (int)(uint32_t)(X >> 55) - 256 - e); }
+    SMC_FX double eps_scaled(int e) const { return dy * inv_h_scaled(e); }
+
+    // The shock of an observation y whose volatility V is, as FP64 has it.
+    SMC_FX double shock_of(double y, const uint64_t* tab) const
+    {
+        uint64_t x = ly;
+#pragma unroll
+        for (int k = 0; k < K; ++k) x += (uint64_t)V[k];
+        return (y - mu) * fx_pack(fx_exp2neg(x, tab), (int)(uint32_t)(x >> 55) - 256);
+    }
 
     // eps_t of the last chain() (units 2^-53).
     SMC_FX int64_t shock() const
@@ -672,6 +684,8 @@ struct EgarchFx {
                (double)T * (ln2 * c0 - 0.5 * log2pi);
     }
 
+    // The shock is the recursion's own, in units of 2^-53: what the next
+    // observation takes up.  A caller's end state takes shock_of().
     SMC_FX void state_out(double* st, double ln2) const
     {
 #pragma unroll

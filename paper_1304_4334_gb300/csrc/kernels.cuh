@@ -147,7 +147,7 @@ struct PolicyEgarchF32T {
         mdl.setup(full, m.gamma, m.eps0_zero);
     }
     __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f32<kPair>(mdl, pipe, T); }
-    __device__ static void state_out(const Model& mdl, double* st) { mdl.state_out(st); }
+    __device__ static void state_out(const Model& mdl, double* st, const Obs* = nullptr) { mdl.state_out(st); }
     __device__ static void load_state(Model& mdl, const double* st) { mdl.load_state(st); }
     __device__ static double logdens(Model& mdl, const Obs* obs, int s, int)
     {
@@ -233,7 +233,7 @@ struct PolicyEgarchF64FxT {
         mdl.setup(full, m.gamma, m.eps0_zero, tab);
     }
     __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int) { return run_egarch_f64(mdl, pipe, T); }
-    __device__ static void state_out(const Model& mdl, double* st) { mdl.state_out(st); }
+    __device__ static void state_out(const Model& mdl, double* st, const Obs* y_last) { mdl.state_out(st, y_last); }
 };
 
 template <int K, int I>
@@ -282,7 +282,7 @@ struct PolicyLinreg {
         mdl.setup(full, m.p, m.sigma);
     }
     __device__ static bool run(Model& mdl, ObsPipe<Obs, kChunk>& pipe, int T, int W) { return run_linreg(mdl, pipe, T, W); }
-    __device__ static void state_out(const Model&, double*) {}
+    __device__ static void state_out(const Model&, double*, const Obs* = nullptr) {}
     __device__ static void load_state(Model&, const double*) {}
     __device__ static double logdens(Model& mdl, const Obs* obs, int s, int W)
     {
@@ -424,7 +424,7 @@ __device__ __forceinline__ void mutate_tile(const MutateArgs& a, uint64_t iter, 
             a.lp[p] = lp_new;
             if (a.state) {
                 double st[kMaxState];
-                Pol::state_out(mdl, st);
+                Pol::state_out(mdl, st, (const Obs*)a.obs + (size_t)(a.T - 1) * a.W);
                 for (int k = 0; k < Pol::kNs; ++k) a.state[k * P + p] = st[k];
             }
         }
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kMutThreads, Pol::kLoglikBlocks) k_loglik(Logl
         if (a.lp) a.lp[p] = log_prior(a.m, th);
         if (a.state) {
             double st[kMaxState];
-            Pol::state_out(mdl, st);
+            Pol::state_out(mdl, st, (const Obs*)a.obs + (size_t)(a.T - 1) * a.W);
             for (int k = 0; k < Pol::kNs; ++k) a.state[k * P + p] = st[k];
         }
     }

@@ -188,8 +188,12 @@ struct LoglikSplit {
             meet();
         }
         meet();                            // nseg segments of the other warps
-        if (out) w.state_out(st);
-        else fx.state_out(st, kLn2);
+        if (out) {
+            w.state_out(st);
+        } else {
+            fx.state_out(st, kLn2);
+            st[K] = fx.shock_of(y[T - 1], sm.tab);
+        }
         meet();                            // their results
         unsigned __int128 scw = 0;
         double lm = 0.0;

@@ -728,10 +728,15 @@ struct EgarchFxSafe {
         return acc64 + (fixed ? fx.finish(T - n64, kLn2, kLog2Pi) : 0.0);
     }
 
-    __device__ __forceinline__ void state_out(double* st) const
+    // y_last: the observation that the state is at (null: the shock in units of 2^-53).
+    __device__ __forceinline__ void state_out(double* st, const double* y_last) const
     {
-        if (out) m.state_out(st);
-        else fx.state_out(st, kLn2);
+        if (out) {
+            m.state_out(st);
+            return;
+        }
+        fx.state_out(st, kLn2);
+        if (y_last) st[K] = fx.shock_of(*y_last, tab);
     }
 };
 

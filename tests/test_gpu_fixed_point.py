@@ -274,3 +274,75 @@ def test_gradient_of_a_rare_component(S, K, I_, theta_p):
         g = torch.empty((spec.d, n), dtype=torch.float64, device="cuda")
         S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(x), ll, g)
         np.testing.assert_allclose(host(g)[last, :40].T, want[:, last], rtol=1e-9)
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (2, 2), (3, 4)])
+@pytest.mark.parametrize("grad", [False, True])
+def test_end_state_of_a_tiny_shock(S, K, I_, grad):
+    """A last return within 2^-40 of the mean leaves a shock of 1e-14 or so, which
+    the recursion itself carries in units of 2^-53: the state given out is the
+    shock as FP64 has it."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 45, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    th = particles(spec.d, truth, K, I_, True, 70, 101)
+    th[:, 0] = th[0, 0]
+    y[-1] = th[0, 0] / 1000.0 * (1.0 + 2.0 ** -40)
+    ll_o, st_o = O.loglik(spec, y, th, with_state=True)
+    assert np.all(np.abs(st_o[:, K]) < 1e-12) and np.all(st_o[:, K] != 0.0)
+    for n in (70, 200 * torch.cuda.get_device_properties(0).multi_processor_count):
+        x = np.resize(th, (n, spec.d))
+        ll = torch.empty(n, dtype=torch.float64, device="cuda")
+        st = torch.empty((K + 1, n), dtype=torch.float64, device="cuda")
+        if grad:
+            g = torch.empty((spec.d, n), dtype=torch.float64, device="cuda")
+            S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(x), ll, g, st)
+        else:
+            S.loglik(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(x), ll, None, st)
+        np.testing.assert_allclose(host(st)[K, :70], st_o[:, K], rtol=1e-9)
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (2, 3)])
+def test_mutation_leaves_the_likelihoods_state(S, K, I_):
+    """The state of accepted proposals, tiny last shock included, is the one that
+    the likelihood gives at the new parameters, to the bit."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 45, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    P = 150 * torch.cuda.get_device_properties(0).multi_processor_count
+    th = particles(spec.d, truth, K, I_, True, P, 103)
+    th[:, 0] = th[0, 0]
+    y[-1] = th[0, 0] / 1000.0 * (1.0 - 2.0 ** -40)
+    L = np.diag(np.full(spec.d, 0.02))
+    L[0, 0] = 0.0
+    m, x, obs = S.model_egarch(K, I_, True), soa(th), dev(y)
+    ll, lp = (torch.empty(P, dtype=torch.float64, device="cuda") for _ in range(2))
+    st = torch.empty((K + 1, P), dtype=torch.float64, device="cuda")
+    S.loglik(m, S.FP64, obs, x, ll, lp, st)
+    assert 0 < S.mutate_rw(m, S.FP64, obs, x, ll, lp, st, dev(L), 0.5, 9, 2, 3) < P
+    ll2, lp2, st2 = torch.empty_like(ll), torch.empty_like(lp), torch.empty_like(st)
+    S.loglik(m, S.FP64, obs, x, ll2, lp2, st2)
+    assert torch.equal(ll, ll2) and torch.equal(st, st2) and bool((st[K] != 0).all())
+
+
+@pytest.mark.parametrize("K,I_", [(1, 1), (1, 2), (3, 4)])
+@pytest.mark.parametrize("side", [-1.0, 1.0])
+def test_gradient_at_a_shock_below_the_fixed_point_unit(S, K, I_, side):
+    """A return one rounding off the mean: the shock (5e-18) is not zero, and the
+    derivative of |eps| there has its sign."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 45, seed=71)
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    th = particles(spec.d, truth, K, I_, True, 40, 105)
+    th[:, 0] = th[0, 0]
+    y[20] = np.nextafter(th[0, 0] / 1000.0, side)
+    ll_o, g_o = O.loglik_grad(spec, y, th)
+    for n in (40, 200 * torch.cuda.get_device_properties(0).multi_processor_count):
+        ll = torch.empty(n, dtype=torch.float64, device="cuda")
+        g = torch.empty((spec.d, n), dtype=torch.float64, device="cuda")
+        S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(np.resize(th, (n, spec.d))), ll, g)
+        err = np.abs(host(g)[:, :40].T - g_o).max(axis=1) / np.abs(g_o).max(axis=1)
+        assert err.max() <= 1e-7, err.max()
