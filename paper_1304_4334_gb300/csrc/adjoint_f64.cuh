@@ -215,11 +215,12 @@ struct AdjointF64 {
         }
         const bool fixed = mdl.fixed;
         EgarchFx<K, I> fx = mdl.fx;
+        fx.natural_shocks();
         auto back = [&](double eps, double inv, const double* vp, double ep, bool has_prev) {
             double eb = -eps;
             if constexpr (I >= 2) {
                 double r[I];
-                if (!(fixed && fx.weights(eps * 0x1p53, r, mdl.tab))) weights_f64(mdl.q, eps, mdl.tab, r);
+                if (!(fixed && fx.weights(eps, r, mdl.tab))) weights_f64(mdl.q, eps, mdl.tab, r);
                 eb = 0.0;
 #pragma unroll
                 for (int i = 0; i < I; ++i) {
@@ -267,7 +268,7 @@ struct AdjointF64 {
             auto keep = [&](int r) {
                 double s[K + 1];
                 fx.state_out(s, kLn2);   // (its shock is not used)
-                put(buf + (size_t)r * W * stride, stride, s, fx.eps_scaled(0), fx.inv_h_scaled(0));
+                put(buf + (size_t)r * W * stride, stride, s, fx.eps(), fx.inv_h());
             };
             if (t0 == 0) fx.template chain<true>(y[0], mdl.tab);
             else fx.template chain<false>(y[t0], mdl.tab);
@@ -326,8 +327,8 @@ struct AdjointF64 {
 // Forward: warp 0 leaves each segment's shocks, warp 1 takes their mixture
 // densities.  Backward, at step j: warp 0 recomputes segment n-1-j and runs the
 // carry over segment n+1-j, warp 1 forms dl/deps and the component sums of
-// segment n-j.  Shocks are kept in units of 2^-53 and V_k in 2^-55, and the
-// sums scaled once at the end.
+// segment n-j.  V_k is kept in units of 2^-55 and its sums scaled once at the
+// end; sums of eps^2 are in eps's own units, so they overflow where FP64's do.
 // Measured at T=600, up to one block (of 32 particles) per SM, one warp ->
 // two: K=1,I=2 1,298 -> 703 us, K=2,I=2 1,441 -> 823 us, K=3,I=4 2,604 ->
 // 1,347 us, K=4,I=4 2,884 -> 1,364 us; with all the blocks an SM's shared
@@ -338,8 +339,8 @@ struct GradSplit {
     static constexpr int kSeg = 16, W = K + 2;
     static constexpr double kVu = 0x1p55 * 0.5 / kLn2;   // V_k units of v_k
     struct Smem {
-        double slab[3][kSeg][W][32];       // V_1..V_K, eps, 2^53 / h
-        double x[2][kSeg][32];             // forward: shocks; backward: dl/deps 2^-53
+        double slab[3][kSeg][W][32];       // V_1..V_K, eps, 1/h
+        double x[2][kSeg][32];             // forward: shocks (2^-53); backward: dl/deps
         double comb[3 * I + 2][32];        // warp 1's results
         uint64_t tab[256];
     };
@@ -347,10 +348,10 @@ struct GradSplit {
     // Both warps, each from its own place in the code.
     __device__ __forceinline__ static void meet() { asm volatile("barrier.sync 1, 64;" ::: "memory"); }
 
-    // A segment of warp 0 in FP64: shocks out (and V, 1/h for the recomputation),
-    // log h summed; w carries the state.
+    // A segment of warp 0 in FP64: shocks out, times `unit` (and V, 1/h for the
+    // recomputation), log h summed; w carries the state.
     __device__ __noinline__ static double segment_f64(EgarchF64<K, I>& w, double lsy, const double* __restrict__ y,
-                                                      int t0, int n, double* es, int es_stride, double* v, double* inv)
+                                                      int t0, int n, double unit, double* es, int es_stride, double* v, double* inv)
     {
         double sum = 0.0;
         for (int r = 0; r < n; ++r) {
@@ -361,11 +362,11 @@ struct GradSplit {
 #pragma unroll
             for (int k = 1; k < K; ++k) vs += w.v[k];
             sum += lsy + 0.5 * vs;
-            es[(size_t)r * es_stride] = w.eps * 0x1p53;
+            es[(size_t)r * es_stride] = w.eps * unit;
             if (v) {
 #pragma unroll
                 for (int k = 0; k < K; ++k) v[(size_t)r * es_stride + 32 * k] = w.v[k] * kVu;
-                inv[(size_t)r * es_stride] = fx_exp_neg(lsy + 0.5 * vs, w.tab) * 0x1p53;
+                inv[(size_t)r * es_stride] = fx_exp_neg(lsy + 0.5 * vs, w.tab);
             }
         }
         return sum;
@@ -432,10 +433,10 @@ struct GradSplit {
                 if (fx.bad == 0u && !out) {
                     sx += fx.sx;
                     fx.state_out(st, kLn2);
-                    st[K] = fx.eps_scaled(0);
+                    st[K] = fx.eps();
                 } else {
                     if (!out) w.load_state(st);
-                    lh64 += segment_f64(w, q.log_sigma_y, y, t0, n, es, 32, nullptr, nullptr);
+                    lh64 += segment_f64(w, q.log_sigma_y, y, t0, n, 0x1p53, es, 32, nullptr, nullptr);
                     n64 += n;
                     out = !(fixed && fx.enter(w.v, w.eps));
                     w.state_out(st);
@@ -456,18 +457,18 @@ struct GradSplit {
         for (int k = 0; k < K; ++k) {
             vb[k] = 0.0;                   // 2 dL/dv_k,t+1
             al[k] = q.alpha[k];
-            ga[k] = q.gamma[k] * 0x1p-54;
-            bp[k] = (q.beta[k] + q.gamma[k]) * 0x1p-54;
-            bm[k] = (q.gamma[k] - q.beta[k]) * 0x1p-54;
+            ga[k] = 0.5 * q.gamma[k];
+            bp[k] = 0.5 * (q.beta[k] + q.gamma[k]);
+            bm[k] = 0.5 * (q.gamma[k] - q.beta[k]);
         }
         auto carry = [&](double dle, double es, double inv, const double* vp, double ep, bool has_prev) {
-            double eb = dle;               // dL/deps 2^-53
+            double eb = dle;               // dL/deps
 #pragma unroll
             for (int k = 0; k < K; ++k) eb = fma(vb[k], es > 0.0 ? bp[k] : (es < 0.0 ? bm[k] : ga[k]), eb);
             const double sb = fma(-eb, es, -1.0);
             gs[0] = fma(-eb, inv, gs[0]);
             gs[1] += sb;
-            const double ae = fabs(ep) - kSqrt2OverPi * 0x1p53;
+            const double ae = fabs(ep) - kSqrt2OverPi;
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 vb[k] = fma(al[k], vb[k], sb);
@@ -476,7 +477,7 @@ struct GradSplit {
                     gs[2 + K + k] = fma(vb[k], ae, gs[2 + K + k]);
                     gs[2 + 2 * K + k] = fma(vb[k], ep, gs[2 + 2 * K + k]);
                 } else if (a.m.eps0_zero) {
-                    gs[2 + K + k] = fma(vb[k], -kSqrt2OverPi * 0x1p53, gs[2 + K + k]);
+                    gs[2 + K + k] = fma(vb[k], -kSqrt2OverPi, gs[2 + K + k]);
                 }
             }
         };
@@ -503,8 +504,8 @@ struct GradSplit {
                 auto put = [&](int r) {
 #pragma unroll
                     for (int k = 0; k < K; ++k) b[r][k][lane] = (double)fx.V[k];
-                    b[r][K][lane] = fx.eps_scaled(53);
-                    b[r][K + 1][lane] = fx.inv_h_scaled(53);
+                    b[r][K][lane] = fx.eps();
+                    b[r][K + 1][lane] = fx.inv_h();
                 };
                 if (t0 == 0) fx.template chain<true>(y[0], sm.tab);
                 else fx.template chain<false>(y[t0], sm.tab);
@@ -519,7 +520,7 @@ struct GradSplit {
 #pragma unroll
                     for (int k = 0; k < K; ++k) w.v[k] = v0[k];
                     w.eps = e0;
-                    segment_f64(w, q.log_sigma_y, y, t0, n, &b[0][K][lane], W * 32, &b[0][0][lane], &b[0][K + 1][lane]);
+                    segment_f64(w, q.log_sigma_y, y, t0, n, 1.0, &b[0][K][lane], W * 32, &b[0][0][lane], &b[0][K + 1][lane]);
                 }
             }
             if (j >= 2) {                  // carry over segment nseg + 1 - j
@@ -537,7 +538,7 @@ struct GradSplit {
                 entering(sg, v0, e0);
 #pragma unroll
                 for (int k = 0; k < K; ++k) v0[k] *= kVu;
-                carry(dl[0], b[0][K][lane], b[0][K + 1][lane], v0, e0 * 0x1p53, t0 > 0);
+                carry(dl[0], b[0][K][lane], b[0][K + 1][lane], v0, e0, t0 > 0);
                 if ((sg & 7) == 0) {
 #pragma unroll
                     for (int i = 0; i < NS; ++i) {
@@ -551,8 +552,8 @@ struct GradSplit {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             gn[2 + k] *= 0.5 / kVu;
-            gn[2 + K + k] *= 0x1p-54;
-            gn[2 + 2 * K + k] *= 0x1p-54;
+            gn[2 + K + k] *= 0.5;
+            gn[2 + 2 * K + k] *= 0.5;
         }
         meet();                            // warp 1's results
 #pragma unroll
@@ -588,7 +589,9 @@ struct GradSplit {
                     const int pe = fx.pe;
                     uint32_t over;
                     fx.mix_terms(e, sm.tab, over);
-                    if (over != 0u || !fixed) {
+                    // (a shock past fixed point's range has its square taken in its own units)
+                    const bool far = (fx_bits(e) << 1) >= (uint64_t)(1023 + 60) << 53;
+                    if (over != 0u || !fixed || far) {
                         double r8[I];
                         fx.pm = pm;
                         fx.pe = pe;
@@ -614,12 +617,13 @@ struct GradSplit {
                   nf * (kLn2 * fx.c0);
         }
         // backward: dl/deps and the component sums
+        fx.natural_shocks();
         double a2[I], m2[I], s0[I], s1[I], s2[I], g[3 * I];
 #pragma unroll
         for (int i = 0; i < I; ++i) {
             const double ai = 1.0 / q.sig[i];
-            a2[i] = ai * ai * 0x1p-106;    // (eps 2^53, dl/deps 2^-53)
-            m2[i] = q.mu[i] * (ai * ai) * 0x1p-53;
+            a2[i] = ai * ai;
+            m2[i] = q.mu[i] * (ai * ai);
             s0[i] = s1[i] = s2[i] = 0.0;
             g[i] = g[I + i] = g[2 * I + i] = 0.0;
         }
@@ -633,7 +637,7 @@ struct GradSplit {
                 for (int r = n - 1; r >= 0; --r) {
                     const double es = b[r][K][lane];
                     double ri[I];
-                    if (!(fixed && fx.weights(es, ri, sm.tab))) weights_f64(q, es * 0x1p-53, sm.tab, ri);
+                    if (!(fixed && fx.weights(es, ri, sm.tab))) weights_f64(q, es, sm.tab, ri);
                     double d = 0.0;
 #pragma unroll
                     for (int i = 0; i < I; ++i) {
@@ -659,7 +663,7 @@ struct GradSplit {
         }
 #pragma unroll
         for (int i = 0; i < I; ++i) {
-            const double r0 = g[i], r1 = g[I + i] * 0x1p-53, r2 = g[2 * I + i] * 0x1p-106;
+            const double r0 = g[i], r1 = g[I + i], r2 = g[2 * I + i];
             const double ai = 1.0 / q.sig[i], mu = q.mu[i];
             sm.comb[i][lane] = r0;
             sm.comb[I + i][lane] = ai * ai * (r1 - mu * r0);

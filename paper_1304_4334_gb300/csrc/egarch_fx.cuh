@@ -416,10 +416,10 @@ struct EgarchFx {
         }
         sx += X;
         const uint64_t T = tab[(uint32_t)(X >> 47) & 255u], q = fx_exp2neg_q(X);
-        M = T - (fx_mulhi(T, q) >> 8);   // (kept only where inv_h_scaled() is used)
+        M = T - (fx_mulhi(T, q) >> 8);   // (kept only where inv_h() is used)
         // |eps| = |y - mu| 2^-X: the 53-bit significand times M, shifted; the
         // shift passes 63 for a zero return
-        dy = y - mu;                     // (kept only where eps_scaled() is used)
+        dy = y - mu;                     // (kept only where eps() is used)
         const uint64_t b = fx_bits(dy);
         const int ed = (int)(uint32_t)(b >> 52) & 0x7ff;
         const uint64_t p0 = fx_mulhi((b << 11) | 0x8000000000000000ull, T);   // beside the polynomial
@@ -505,10 +505,21 @@ struct EgarchFx {
         return over == 0u;
     }
 
-    // 2^e / h_t and 2^e eps_t of the last chain(), the shock with all its bits
-    // (shock() holds it in units of 2^-53).
-    SMC_FX double inv_h_scaled(int e) const { return fx_pack(M, (int)(uint32_t)(X >> 55) - 256 - e); }
-    SMC_FX double eps_scaled(int e) const { return dy * inv_h_scaled(e); }
+    // From here on weights() takes eps itself in the place of eps 2^53 (and
+    // mix_terms() must not be called).
+    SMC_FX void natural_shocks()
+    {
+#pragma unroll
+        for (int i = 0; i < kM; ++i) {
+            A[i] *= 0x1p106;
+            B[i] *= 0x1p53;
+        }
+    }
+
+    // 1 / h_t and eps_t of the last chain(), the shock with all its bits (shock()
+    // holds it in units of 2^-53).
+    SMC_FX double inv_h() const { return fx_pack(M, (int)(uint32_t)(X >> 55) - 256); }
+    SMC_FX double eps() const { return dy * inv_h(); }
 
     // The shock of an observation y whose volatility V is, as FP64 has it.
     SMC_FX double shock_of(double y, const uint64_t* tab) const

@@ -177,7 +177,7 @@ struct LoglikSplit {
                     fx.state_out(st, kLn2);
                     w.load_state(st);
                 }
-                lh64 += GradSplit<K, I>::segment_f64(w, q.log_sigma_y, y, t0, n, es, 32, nullptr, nullptr);
+                lh64 += GradSplit<K, I>::segment_f64(w, q.log_sigma_y, y, t0, n, 0x1p53, es, 32, nullptr, nullptr);
                 for (int r = 0; r < n; ++r) {
                     const double z = es[r * 32] * 0x1p-53 - fx.m0;
                     q64 = fma(z, z, q64);

@@ -346,3 +346,24 @@ def test_gradient_at_a_shock_below_the_fixed_point_unit(S, K, I_, side):
         S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(np.resize(th, (n, spec.d))), ll, g)
         err = np.abs(host(g)[:, :40].T - g_o).max(axis=1) / np.abs(g_o).max(axis=1)
         assert err.max() <= 1e-7, err.max()
+
+
+@pytest.mark.parametrize("K,I_", [(1, 2), (2, 3)])
+def test_gradient_of_an_enormous_shock(S, K, I_):
+    """A return of 1e140: l is about -1e283, finite, and so is its gradient, in
+    both gradient kernels (nothing is scaled on the way)."""
+    torch = torch_cuda()
+    truth = egarch_truth(K, I_)
+    y = I.simulate_egarch(truth, 40, seed=71)
+    y[-1] = 1e140
+    spec = O.ModelSpec(K=K, I=I_, gamma=True)
+    th = particles(spec.d, truth, K, I_, True, 40, 107)
+    ll_o, g_o = O.loglik_grad(spec, y, th)
+    assert np.isfinite(ll_o).all() and np.isfinite(g_o).all()
+    for n in (40, 200 * torch.cuda.get_device_properties(0).multi_processor_count):
+        ll = torch.empty(n, dtype=torch.float64, device="cuda")
+        g = torch.empty((spec.d, n), dtype=torch.float64, device="cuda")
+        S.loglik_grad(S.model_egarch(K, I_, True), S.FP64, dev(y), soa(np.resize(th, (n, spec.d))), ll, g)
+        np.testing.assert_allclose(host(ll)[:40], ll_o, rtol=1e-9)
+        err = np.abs(host(g)[:, :40].T - g_o).max(axis=1) / np.abs(g_o).max(axis=1)
+        assert err.max() <= 1e-7, err.max()
