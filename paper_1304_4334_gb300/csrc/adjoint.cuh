@@ -30,6 +30,14 @@
 
 namespace smc {
 
+// Observations per checkpoint segment of the EGARCH adjoint (the reverse
+// sweep's shared-memory slab holds one segment per thread); the checkpoint
+// buffers are sized from the same value.  (16 in FP32 as well, for more
+// resident blocks, was measured and not kept: 5.81 against 5.90 ms per launch
+// at K=2, I=2, T=5000, 262,144 particles, for twice the checkpoint memory.)
+template <typename Real>
+constexpr int mala_seg() { return sizeof(Real) == 4 ? 32 : 16; }
+
 template <typename Real>
 __device__ __forceinline__ Real nexp(Real x)
 {

@@ -336,7 +336,7 @@ struct AdjointF64 {
 // second wave would take what the split gains (k_loglik_grad then).
 template <int K, int I>
 struct GradSplit {
-    static constexpr int kSeg = 16, W = K + 2;
+    static constexpr int kSeg = mala_seg<double>(), W = K + 2;   // (the caller's checkpoint block is sized from it)
     static constexpr double kVu = 0x1p55 * 0.5 / kLn2;   // V_k units of v_k
     struct Smem {
         double slab[3][kSeg][W][32];       // V_1..V_K, eps, 1/h
