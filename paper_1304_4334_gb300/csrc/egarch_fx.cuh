@@ -203,10 +203,10 @@ SMC_FX uint64_t fx_rcp(uint64_t s)
     return Y;
 }
 
-// e^-x in FP64 without FP64 instructions for |x| < 700: within a unit in the
-// last place for |x| < 128, within 2^-51 beyond, where x itself, a rounded
-// FP64 sum, is known to 2^-46 at best; the library's exponential where the
-// result leaves the normal range, and its limits past that.
+// e^-x in FP64 without FP64 instructions for |x| < 700, within a unit in the
+// last place (from 128 on x log2(e) has more than 64 bits: its full product is
+// taken, log2(e)'s own rounding is 2^-54 of the exponent at most); the library's
+// exponential where the result leaves the normal range, and its limits past that.
 SMC_FX double fx_exp_neg(double x, const uint64_t* tab)
 {
     const uint64_t sg = (uint64_t)((int64_t)fx_bits(x) >> 63);
@@ -217,11 +217,12 @@ SMC_FX double fx_exp_neg(double x, const uint64_t* tab)
         X = (X ^ sg) - sg;
         n = (int)((int64_t)X >> 55);
     } else if (std::fabs(x) < 700.0) {
-        const uint64_t b = fx_bits(x);                // units of 2^-53, then 2^-52
-        X = fx_mulhi(((b << 11) | 0x8000000000000000ull) >> (1033 - ((int)(b >> 52) & 0x7ff)), kFxLog2e);
-        X = (X ^ sg) - sg;
-        n = (int)((int64_t)X >> 52);
-        X <<= 3;
+        const uint64_t b = fx_bits(x);                // |x| = m 2^(e - 1023 - 63), e from 1030 to 1032
+        const uint64_t m = (b << 11) | 0x8000000000000000ull;
+        const unsigned __int128 w = ((unsigned __int128)m * kFxLog2e) >> (1094 - ((int)(b >> 52) & 0x7ff));
+        const __int128 v = sg ? -(__int128)w : (__int128)w;   // units of 2^-55
+        n = (int)(v >> 55);
+        X = (uint64_t)v;
     } else if (std::fabs(x) < 1024.0) {
         return fx_exp_library(-x);
     } else {

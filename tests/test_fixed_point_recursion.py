@@ -246,3 +246,39 @@ def test_component_weights_against_long_double(tmp_path):
     subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
     worst = [float(v) for v in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()]
     assert max(worst) < 8.0, worst
+
+
+EXP = r"""
+#include <cstdio>
+#include <random>
+#include "HEADER"
+#define __device__
+#include "TABLE"
+using namespace smc;
+int main() {
+    std::mt19937_64 g(2);
+    double u = 0;
+    for (int i = 0; i < 1000000; ++i) {
+        const double x = (i & 1 ? -1 : 1) * (128.0 + 572.0 * (double)(g() >> 11) * 0x1p-53);
+        u = fmax(u, (double)fabsl(fx_exp_neg(x, g_exp2_neg256) / expl(-(long double)x) - 1));
+    }
+    for (double x : {128.0, 255.999999999999, 256.0, 511.999999999999, 512.0, 699.999999999999})
+        for (double s : {-1.0, 1.0})
+            u = fmax(u, (double)fabsl(fx_exp_neg(s * x, g_exp2_neg256) / expl(-(long double)(s * x)) - 1));
+    printf("%.17g\n", u);
+}
+"""
+
+
+def test_exponential_from_128_to_700(tmp_path):
+    """Rounding of the result (2^-53), of log2(e) (2^-64 of up to 1010: 2^-54) and
+    of the product (2^-55), the last two times ln 2: below 2^-52."""
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("no host C++ compiler")
+    src = tmp_path / "exp.cpp"
+    src.write_text(EXP.replace("HEADER", HEADER).replace("TABLE", TABLE))
+    exe = tmp_path / "exp"
+    subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
+    u = float(subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout)
+    assert u < 2.0 ** -52, u
