@@ -1401,9 +1401,10 @@ __global__ void __launch_bounds__(kSelThreads) k_select(SelectArgs a)
             a.lw[j] = lwj;
             a.a[j] += lwj;
             if (a.a_score) a.a_score[j] += lwj;   // log score: cycles after the burn-in
-            a.gstat[3 * j + 0] = lmax;
-            a.gstat[3 * j + 1] = s1;
-            a.gstat[3 * j + 2] = s2;
+            double* g = a.gstat + 3 * (size_t)j;
+            g[0] = lmax;
+            g[1] = s1;
+            g[2] = s2;
         }
         if (a.stats_only) return;
         wmax = lmax == -INFINITY ? 0.0 : 1.0;

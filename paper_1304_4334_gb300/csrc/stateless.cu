@@ -439,13 +439,13 @@ smc_status smc_resample_logw(const double* logw, int J, int N, int resampler, ui
     if (!logw || !idx || J < 1 || N < 1 || N > SMC_MAX_N || resampler < 0 || resampler > 3) return SMC_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
     // a [J] and the error word (cleared together), lw [J], gstat [3 J]
-    const size_t n_buf = (size_t)(5 * J + 1) * sizeof(double);
+    const size_t Js = (size_t)J, n_buf = (5 * Js + 1) * sizeof(double);
     Scratch w(s);
     w.add(n_buf);
     CK(w.get());
     double* buf = w.take<double>(n_buf);
-    int* err = reinterpret_cast<int*>(buf + J);
-    CK(cudaMemsetAsync(buf, 0, (size_t)(J + 1) * sizeof(double), s));
+    int* err = reinterpret_cast<int*>(buf + Js);
+    CK(cudaMemsetAsync(buf, 0, (Js + 1) * sizeof(double), s));
     SelectArgs sa;
     std::memset(&sa, 0, sizeof sa);
     sa.mode = 1;
@@ -456,15 +456,15 @@ smc_status smc_resample_logw(const double* logw, int J, int N, int resampler, ui
     sa.seed = seed;
     sa.cycle = cycle;
     sa.a = buf;
-    sa.lw = buf + J + 1;
-    sa.gstat = buf + 2 * J + 1;
+    sa.lw = buf + Js + 1;
+    sa.gstat = buf + 2 * Js + 1;
     sa.idx = idx;
     sa.err = err;
     cudaError_t e = launch_select(sa, s);
     int h = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, err, sizeof h, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && lwbar)
-        e = cudaMemcpyAsync(lwbar, buf + J + 1, (size_t)J * sizeof(double), cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(lwbar, buf + Js + 1, Js * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return SMC_ECUDA;
     if (h & kErrDegenerate) return SMC_EDEGENERATE;

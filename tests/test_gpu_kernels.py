@@ -741,3 +741,19 @@ def test_covariance_forms_by_tiles_per_block(S, d, tiles):
     P = 2 * torch.cuda.get_device_properties(0).multi_processor_count * 64 * tiles
     for n in (P, P + 1):
         test_covariance_block_shapes_match_numpy(S, d, n)
+
+
+def test_resample_of_very_many_groups(S):
+    """429,496,730 groups of one particle: five values of scratch per group are
+    more than 2^31 of them (17 GB)."""
+    import ctypes as C
+    torch = torch_cuda()
+    J = 429496730
+    lw = torch.zeros(J, dtype=torch.float64, device="cuda")
+    idx = torch.full((J,), -1, dtype=torch.int32, device="cuda")
+    st = S.lib().smc_resample_logw(C.c_void_p(lw.data_ptr()), J, 1, S.RESIDUAL, 1, 1, C.c_void_p(idx.data_ptr()), None,
+                                   C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == S.OK and int(idx.min()) == 0 and int(idx.max()) == 0
+    del lw, idx
+    torch.cuda.empty_cache()
+    S.release_workspace()
