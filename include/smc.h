@@ -394,7 +394,9 @@ void smc_batch_free(smc_batch* b);
  * and custom drivers).  All enqueue on `stream`; temporaries they need are
  * allocated stream-ordered from the library's memory pool of the current device
  * and released to it before return.  The pool keeps up to 512 MiB for the next
- * call; smc_release_workspace gives the unused part back to the device.
+ * call, memory that other allocators of the process (torch's, say) do not see as
+ * free; smc_release_workspace gives the unused part back to the device.  No call
+ * may follow a cudaDeviceReset.
  * ------------------------------------------------------------------------- */
 smc_status smc_release_workspace(void);
 
@@ -403,7 +405,11 @@ smc_status smc_release_workspace(void);
  * SMC_FP32, double[T] for EGARCH with SMC_FP64, or double[T][W] records
  * [x_1..x_p, y, 0...] with W = smc_linreg_width(p) for LINREG; 16-byte
  * aligned.  theta: device [d][P].  Outputs (device, nullable except ll):
- * ll[P], lp[P] (log prior), state[K+1][P] (v_kT, eps_T). */
+ * ll[P], lp[P] (log prior), state[K+1][P] (v_kT, eps_T).  With SMC_FP64 and
+ * I >= 2 the kernel depends on P, and with it the last bits of a particle's ll
+ * (of its state too after values that leave the fixed-point ranges): in a call
+ * of another size the same particle may differ by rounding.  Runs do not (one
+ * kernel at every size). */
 smc_status smc_loglik(const smc_model* m, int precision, const void* obs, int T,
                       const double* theta, int P, double* ll, double* lp, double* state,
                       void* stream);
@@ -425,7 +431,9 @@ smc_status smc_mutate_rw(const smc_model* m, int precision, const void* obs, int
  * EGARCH recursion of Section 5.1 with checkpoints of the state every 32 (FP32)
  * or 16 (FP64) observations; for LINREG the closed form sum_t (y_t - x_t'b) x_t
  * / sigma^2.  Layouts as smc_loglik; grad: device [d][P].  Checkpoint scratch
- * is allocated stream-ordered (about (K+1) T P / 32 values). */
+ * is allocated stream-ordered (about (K+1) T P / 32 values in FP32, / 16 in
+ * FP64).  With SMC_FP64 and I >= 2 the last bits of a particle's ll and grad
+ * depend on P, as for smc_loglik. */
 smc_status smc_loglik_grad(const smc_model* m, int precision, const void* obs, int T,
                            const double* theta, int P, double* ll, double* grad, double* state,
                            void* stream);

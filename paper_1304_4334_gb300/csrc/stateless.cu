@@ -70,7 +70,10 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // first call after a wait 545 -> 341 us; power search, S phase and covariance
 // at 1,024 particles: 475 -> 250 us; calls in a row cost the same).  What is kept
 // serves every stream and thread (the pool orders reuse between streams
-// itself); smc_release_workspace() gives it back.
+// itself); smc_release_workspace() gives it back, and the driver takes it for an
+// allocation of this process that would fail otherwise.  The handle lives as long
+// as the process: after cudaDeviceReset it is stale, so no stateless call may
+// follow one.
 constexpr uint64_t kPoolKeep = 512ull << 20;
 constexpr int kMaxPools = 64;
 std::mutex g_pool_mu;
