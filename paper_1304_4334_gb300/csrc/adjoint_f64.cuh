@@ -444,7 +444,7 @@ struct GradSplit {
             }
             meet();
         }
-        const double logh = lh64 + kLn2 * EgarchFx<K, I>::to_double((__int128)sx - ((__int128)(T - n64) << 63)) * 0x1p-55;
+        const double logh = lh64 + kLn2 * fx_to_double((__int128)sx - ((__int128)(T - n64) << 63), -55);
         if (active && a.state)
 #pragma unroll
             for (int k = 0; k <= K; ++k) a.state[k * P + p] = st[k];
@@ -612,7 +612,7 @@ struct GradSplit {
         double lm = lm64;
         if (fixed) {
             const double nf = (double)(T - n64);
-            lm += kLn2 * (EgarchFx<K, I>::to_double((__int128)scw) * 0x1p-55 + (double)fx.pe + log2((double)fx.pm * 0x1p-62)) -
+            lm += kLn2 * (fx_to_double((__int128)scw, -55) + (double)fx.pe + log2((double)fx.pm * 0x1p-62)) -
                   0.5 * (fx.a0 * fx.a0) * (e2 * 0x1p-106 - 2.0 * fx.m0 * (e1 * 0x1p-53) + nf * (fx.m0 * fx.m0)) +
                   nf * (kLn2 * fx.c0);
         }

@@ -132,15 +132,6 @@ SMC_FX uint64_t fx_exp2neg(uint64_t X, const uint64_t* tab)
     return T - (fx_mulhi(T, fx_exp2neg_q(X)) >> 8);
 }
 
-SMC_FX int64_t fx_round(double x)   // nearest integer (|x| < 2^62)
-{
-#if defined(__CUDA_ARCH__)
-    return __double2ll_rn(x);
-#else
-    return (int64_t)std::nearbyint(x);
-#endif
-}
-
 // |x| in units of 2^-56 for |x| < 128 (truncated); false beyond, and for inf, NaN.
 SMC_FX bool fx_fixed56(double x, uint64_t& X)
 {
@@ -231,6 +222,35 @@ SMC_FX double fx_exp_neg(double x, const uint64_t* tab)
     return fx_pack(fx_exp2neg(X, tab), n);            // e^-x = M 2^(-63 - n)
 }
 
+// |x| < c (c > 0); false for a NaN.  On the integer pipe: a comparison holds the
+// FP64 pipe like any other FP64 instruction.
+SMC_FX bool fx_below(double x, double c) { return (fx_bits(x) << 1) < (fx_bits(c) << 1); }
+
+// Nearest integer to x 2^s (ties away from zero) for |x| 2^s < 2^62, from the
+// bits of x: a product and a conversion on the FP64 pipe take 128 cycles per
+// warp, and a setup has 2 + 3 K of them.
+SMC_FX int64_t fx_scaled(double x, int s)
+{
+    const uint64_t b = fx_bits(x);
+    const int sh = 1085 - s - ((int)(b >> 52) & 0x7ff);   // |x| 2^s = m 2^-(sh + 1)
+    const uint64_t r = (fx_shr((b << 11) | 0x8000000000000000ull, sh > 0 ? sh : 0) + 1ull) >> 1;
+    const uint64_t sg = (uint64_t)((int64_t)b >> 63);
+    return (int64_t)((r ^ sg) - sg);
+}
+
+// v 2^e in FP64 (rounded once, normal range; zero for zero), likewise.
+SMC_FX double fx_to_double(__int128 v, int e)
+{
+    const uint64_t sg = (uint64_t)(v >> 127);
+    const unsigned __int128 m = sg ? -(unsigned __int128)v : (unsigned __int128)v;
+    const uint64_t hi = (uint64_t)(m >> 64), lo = (uint64_t)m;
+    if ((hi | lo) == 0ull) return 0.0;
+    const int z = hi ? fx_clz64(hi) : 64 + fx_clz64(lo);
+    const uint64_t t = hi ? (hi << z) | fx_shr(lo, 64 - z) : lo << (z - 64);   // m = t 2^(64 - z), bit 63 set
+    const double d = fx_pack(t >> 1, z - 128 - e);
+    return sg ? -d : d;
+}
+
 // Product of the mixture sums s (units 2^-61, in [1, 4]): pm 2^(pe - 62) with
 // pm kept in [2^62, 2^63).
 SMC_FX void fx_product(uint64_t& pm, int& pe, uint64_t s)
@@ -290,27 +310,27 @@ struct EgarchFx {
         // (the product's rounding error and log2(e)'s own go in separately: a
         // constant error of log2 h_t scales every shock)
         const double lyd = log_sigma_y * log2e;
-        ok = ok && std::fabs(lyd) < fmin(40.0, 255.0 - K * kVmax) && std::fabs(mu_y) < 1e30;
+        ok = ok && fx_below(lyd, 40.0 < 255.0 - K * kVmax ? 40.0 : 255.0 - K * kVmax) && fx_below(mu_y, 1e30);
         const double lye = fma(log_sigma_y, log2e, -lyd) + log_sigma_y * kFxLog2eLo;
-        ly = (uint64_t)(ok ? fx_round(lyd * 0x1p55) + fx_round(lye * 0x1p55) : 0) ^ (1ull << 63);
-        double cmax = 0.0;
+        ly = (uint64_t)(ok ? fx_scaled(lyd, 55) + fx_scaled(lye, 55) : 0) ^ (1ull << 63);
+        bool c0ok = true, c2ok = true;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const double c = g * (beta[k] + std::fabs(gamma[k]));
-            ok = ok && c < 15.8;   // (each by itself: a NaN fails it, fmax would drop it)
-            cmax = fmax(cmax, c);
+            ok = ok && fx_below(c, 15.8);   // (each by itself: a NaN fails it)
+            c0ok = c0ok && fx_below(c, 0.99);
+            c2ok = c2ok && fx_below(c, 3.96);
         }
-        cs = cmax < 0.99 ? 0 : (cmax < 3.96 ? 2 : 4);
-        const double cunit = cs == 0 ? 0x1p60 : (cs == 2 ? 0x1p58 : 0x1p56);
+        cs = c0ok ? 0 : (c2ok ? 2 : 4);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            ok = ok && std::fabs(alpha[k]) <= 1.0 && beta[k] >= 0.0;
-            int64_t as = fx_round(ok ? alpha[k] * 0x1p60 : 0.0) + (1ll << 60);
+            ok = ok && fx_below(alpha[k], 1.0 + 0x1p-52) && !(fx_bits(beta[k]) >> 63);
+            int64_t as = fx_scaled(ok ? alpha[k] : 0.0, 60) + (1ll << 60);
             as = as < (1ll << 61) ? as : (1ll << 61) - 1;   // alpha = 1 to FP64 precision
             ah[k] = (int32_t)(as >> 30);
             al[k] = (int32_t)as & 0x3fffffff;
-            const int64_t bi = fx_round(ok ? beta[k] * g * cunit : 0.0);
-            const int64_t gi = fx_round(ok ? gamma[k] * g * cunit : 0.0);
+            const int64_t bi = fx_scaled(ok ? beta[k] * g : 0.0, 60 - cs);
+            const int64_t gi = fx_scaled(ok ? gamma[k] * g : 0.0, 60 - cs);
             const int64_t cpi = bi + gi, cmi = bi - gi;
             cph[k] = (int32_t)(cpi >> 29);
             cpl[k] = (int32_t)cpi & 0x1fffffff;
@@ -666,8 +686,8 @@ struct EgarchFx {
         for (int k = 0; k < K; ++k) ok = ok && std::fabs(v[k] * g) < kVmax - 1.0;
         if (!ok) return false;
 #pragma unroll
-        for (int k = 0; k < K; ++k) V[k] = fx_round(v[k] * g * 0x1p55);
-        E = (uint64_t)fx_round(std::fabs(eps) * 0x1p53);
+        for (int k = 0; k < K; ++k) V[k] = fx_scaled(v[k] * g, 55);
+        E = (uint64_t)fx_scaled(std::fabs(eps), 53);
         set_limbs(E << cs);
         neg = eps < 0.0 ? -1 : 0;
         return true;
@@ -679,18 +699,13 @@ struct EgarchFx {
         el = (int32_t)((uint32_t)Es & 0x1fffffffu);
     }
 
-    SMC_FX static double to_double(__int128 v)
-    {
-        return (double)(int64_t)(v >> 64) * 0x1p64 + (double)(uint64_t)v;
-    }
-
     // log p(y_1:T | theta) after the last flush.
     SMC_FX double finish(int T, double ln2, double log2pi) const
     {
-        const double sle = to_double((__int128)(scw - sx) + ((__int128)T << 63)) * 0x1p-55;
-        const double s2d = to_double((__int128)s2) * 0x1p-86;
+        const double sle = fx_to_double((__int128)(scw - sx) + ((__int128)T << 63), -55);
+        const double s2d = fx_to_double((__int128)s2, -86);
         if (I == 1) return ln2 * sle - 0.5 * s2d - 0.5 * log2pi * (double)T;
-        const double s1e = to_double(s1w) * 0x1p-53;
+        const double s1e = fx_to_double(s1w, -53);
         const double q = s2d - 2.0 * m0 * s1e + (double)T * (m0 * m0);
         return ln2 * (sle + (double)pe + log2((double)pm * 0x1p-62)) - 0.5 * (a0 * a0) * q +
                (double)T * (ln2 * c0 - 0.5 * log2pi);
@@ -702,7 +717,7 @@ struct EgarchFx {
     {
 #pragma unroll
         for (int k = 0; k < K; ++k) st[k] = (double)V[k] * (2.0 * ln2 * 0x1p-55);
-        st[K] = (neg ? -1.0 : 1.0) * ((double)E * 0x1p-53);
+        st[K] = (double)shock() * 0x1p-53;
     }
 };
 

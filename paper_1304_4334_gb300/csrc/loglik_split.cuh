@@ -202,12 +202,11 @@ struct LoglikSplit {
             scw += ((unsigned __int128)sm.hi[m][lane] << 64) + sm.lo[m][lane];
             lm += sm.lm[m][lane];
         }
-        using Fx = EgarchFx<K, I>;
-        const double sle = Fx::to_double((__int128)(scw - sx) + ((__int128)(T - n64) << 63)) * 0x1p-55;
+        const double sle = fx_to_double((__int128)(scw - sx) + ((__int128)(T - n64) << 63), -55);
         double ll = kLn2 * sle + lm - lh64 - 0.5 * kLog2Pi * (double)T;
         if (fixed) {
             const double nf = (double)(T - n64);
-            const double qd = Fx::to_double((__int128)s2) * 0x1p-86 - 2.0 * fx.m0 * (Fx::to_double(s1) * 0x1p-53) +
+            const double qd = fx_to_double((__int128)s2, -86) - 2.0 * fx.m0 * fx_to_double(s1, -53) +
                               nf * (fx.m0 * fx.m0) + q64;
             ll += (double)T * (kLn2 * fx.c0) - 0.5 * (fx.a0 * fx.a0) * qd;
         }
