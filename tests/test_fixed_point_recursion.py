@@ -282,3 +282,74 @@ def test_exponential_from_128_to_700(tmp_path):
     subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
     u = float(subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout)
     assert u < 2.0 ** -52, u
+
+
+BLOCK = "#include <algorithm>\n" + SRC[:SRC.index("template <int K, int I> void test(")] + r"""
+// Blocks of any length with the state taken out and up again in between; beta of
+// any size (the coefficients' three scales, cs = 0, 2, 4).
+template <int K, int I> void test(int T, double beta, int cs) {
+    std::mt19937_64 g(1000 * K + 10 * I + cs);
+    std::normal_distribution<double> N;
+    std::vector<double> fx, dbl, mags;
+    int used = 0, wrong = 0;
+    for (int p = 0; p < 4000; ++p) {
+        std::vector<double> y(T);
+        for (auto& x : y) x = 0.0003 + 0.01 * N(g);
+        Par q;
+        q.mu = 0.0003;
+        q.lsy = log(0.01);
+        for (int k = 0; k < K; ++k) q.al[k] = 0.3 + 0.1 * N(g), q.be[k] = beta * exp(0.05 * N(g)), q.ga[k] = 0.05 * N(g);
+        double v = 0;
+        for (int i = 0; i < I; ++i) q.p[i] = 1.0 / I, q.m[i] = 0, q.s[i] = exp(0.3 * i), v += q.p[i] * q.s[i] * q.s[i];
+        for (int i = 0; i < I; ++i) q.s[i] /= sqrt(v);
+        EgarchFx<K, I> f;
+        f.setup(q.mu, q.lsy, q.al, q.be, q.ga, q.p, q.m, q.s, 0, 1.0 / log(2.0));
+        wrong += f.cs != cs;
+        for (int t = 0, n = 1; t < T; t += n, n = 1 + (5 * n) % 33) {
+            n = n < T - t ? n : T - t;
+            f.block(&y[t], n, t == 0, g_exp2_neg256);
+            double st[K + 1];
+            f.state_out(st, log(2.0));
+            if (!f.bad && !f.enter(st, st[K])) f.bad = 1;
+        }
+        if (f.bad) continue;                 // (left the ranges: not this test's)
+        R sq[K + 1], mag;
+        double sd[K + 1], magd;
+        const R lq = plain<R, K, I>(q, y, sq, &mag);
+        const R ed = plain<double, K, I>(q, y, sd, &magd) - lq, e = f.finish(T, log(2.0), log(2 * M_PI)) - lq;
+        fx.push_back((double)fabsl(e)), dbl.push_back((double)fabsl(ed)), mags.push_back((double)mag), ++used;
+    }
+    for (auto* x : {&fx, &dbl, &mags}) std::sort(x->begin(), x->end());
+    for (double at : {0.5, 0.9}) {
+        const int n = (int)(at * used);
+        printf("%d %d %d %.17g %.17g %.17g %d %d\n", K, I, cs, fx[n], dbl[n], mags[n], used, wrong);
+    }
+}
+int main() {
+    test<1, 1>(90, 0.1, 0);
+    test<2, 3>(90, 0.5, 0);
+    test<1, 2>(90, 1.8, 2);
+    test<2, 2>(60, 1.7, 2);
+    test<1, 1>(12, 7.0, 4);
+    test<1, 3>(12, 7.0, 4);
+}
+"""
+
+
+def test_blocks_and_large_coefficients_against_long_double(tmp_path):
+    """As the first test, through block() and enter(): at the median particle and at
+    the 90% one (a recursion with beta = 7 amplifies any rounding, so that one
+    particle can make up a mean square) no larger an error than the recursion in
+    double, or 2^-52 of the magnitudes summed."""
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("no host C++ compiler")
+    src = tmp_path / "block.cpp"
+    src.write_text(BLOCK.replace("HEADER", HEADER).replace("TABLE", TABLE))
+    exe = tmp_path / "block"
+    subprocess.run([gxx, "-O1", "-std=gnu++17", "-o", str(exe), str(src)], check=True)
+    rows = [x.split() for x in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split("\n") if x]
+    assert len(rows) == 12
+    for K, I, cs, fx, dbl, mag, used, wrong in rows:
+        assert int(used) >= 500 and wrong == "0", (K, I, cs, used, wrong)
+        assert float(fx) <= max(float(dbl), float(mag) * 2.0 ** -52), (K, I, cs, fx, dbl, mag)
