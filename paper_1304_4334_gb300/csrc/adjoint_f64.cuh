@@ -14,7 +14,7 @@
 // against 230 with FP64 exponentials and division.
 // Measured (value and gradient, K = 2, I = 2, 2,049 particles x 1,037
 // observations, a warp per scheduler at most): 7.9 ms in FP64 throughout, 2.42
-// ms in AdjointF64, 1.35 ms in GradSplit.
+// ms in AdjointF64, 1.33 ms in GradSplit.
 #pragma once
 
 #include "adjoint.cuh"

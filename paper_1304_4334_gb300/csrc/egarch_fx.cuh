@@ -12,8 +12,8 @@
 //     integer and fraction parts index 2^-X = 2^-n 2^(-j/256) 2^-r directly,
 //     r < 2^-8 by a degree-5 polynomial (2^-60 relative);
 //   - mixture terms relative to component 0, the one with the largest sigma:
-//     d_i = x_i - x_0 is a quadratic in eps (two FP64 FMAs, the only FP64 work
-//     left besides y_t - mu_Y and the conversion of eps), brought to fixed
+//     d_i = x_i - x_0 is a quadratic in eps (two FP64 FMAs; y_t - mu_Y and the
+//     conversion of eps are the other FP64 work of an observation), brought to fixed
 //     point; m = max(0, d_i), s_t = sum_i 2^(d_i - m) in [1, I], and one
 //     logarithm of the running product of the s_t for the whole series;
 //   - sums of log2 h_t, m, eps_t and eps_t^2 are exact integer sums; x_0's
@@ -28,12 +28,13 @@
 // with all of FP64's bits.
 //
 // Measured, random-walk iteration at K = 2, I = 2, 65,536 particles x 5,000
-// observations: 76.1 ms with the recursion in FP64, 5.1 ms (about 330
-// instructions per particle and observation, over half of the FP64 and of the
-// integer pipe at four warps per scheduler); likelihood at K = 3, I = 4,
-// 10,007 x 3,089: 17.8 ms, 2.28 ms with one warp per 32 particles (one warp per
-// scheduler: the chain's latency), 1.47 ms with three (LoglikSplit); mutation of
-// 1,024 x 500 at K = I = 1: 0.55 ms, 0.14 ms.  Errors against
+// observations: 76.1 ms with the recursion in FP64, 5.06 ms (about 300
+// instructions per particle and observation; x 500: the FP64 pipe 54% busy, the
+// integer multiplier 44%, issue 41%, and a warp waits longest for its own
+// dependent instructions, at 3.4 warps per scheduler); likelihood at K = 3,
+// I = 4, 10,007 x 3,089: 17.8 ms, 2.28 ms with one warp per 32 particles (one
+// warp per scheduler: the chain's latency), 1.47 ms with three (LoglikSplit);
+// mutation of 1,024 x 500 at K = I = 1: 0.55 ms, 0.14 ms.  Errors against
 // 113-bit arithmetic: log likelihood 2e-16 relative at T = 5,000 (2.5e-15 in
 // FP64, whose running sum rounds), end state 0.4 to 1 of FP64's.
 //

@@ -176,7 +176,7 @@ __device__ __noinline__ void cov_partial_f64(const double* __restrict__ theta, i
 // once; warps and blocks are added in FP64.  Bound by the FMAs' issue and the loads of theta
 // (193 MB at d = 23, 1,048,576 particles).  The first form gave one entry to a
 // thread (two 4-byte loads per FMA) and formed and converted theta - shift in
-// FP64: 307 us there, now 94 us (whole calls: 14 parameters, 70,000 particles 31
+// FP64: 307 us there, now 93 us (whole calls: 14 parameters, 70,000 particles 31
 // -> 25 us; 32, 250,000 106 -> 76 us).
 // kM > 1: kM warps share a tile, its rows to stage and its products.
 template <int B, int kM = 1>
