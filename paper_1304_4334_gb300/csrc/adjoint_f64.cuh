@@ -8,7 +8,9 @@
 //     of its ranges);
 //   - the component weights r_i come from integer exponentials and an integer
 //     reciprocal of their sum, assembled as FP64 numbers by integer instructions;
-//   - the sums over t keep r_i, r_i eps and r_i eps^2 per component, from which d log p_i, d mu_i and d a_i follow once at the end
+//   - the sums over t keep r_i, r_i z and r_i z^2 per component, z = eps - mu_i
+//     (about mu_i, and taken together every segment, so that no two large sums
+//     are left to cancel at the end), from which d log p_i, d mu_i and d a_i follow once at the end
 //     (4 FP64 instructions per component and observation instead of 11).
 // About 40 FP64 instructions per particle and observation at K = 2, I = 2
 // against 230 with FP64 exponentials and division.
@@ -122,7 +124,7 @@ __device__ __noinline__ double weights_f64(const EgarchParams<double, K, I>& q, 
 template <int K, int I, int kSeg>
 struct AdjointF64 {
     EgarchFxSafe<K, I> mdl;
-    double a2[I], m2[I];         // a_i^2, mu_i a_i^2
+    double a2[I];                // a_i^2
 
     __device__ __forceinline__ void setup(const double* th, int has_gamma, int eps0_zero, const uint64_t* tab)
     {
@@ -131,7 +133,6 @@ struct AdjointF64 {
         for (int i = 0; i < I; ++i) {
             const double a = 1.0 / mdl.q.sig[i];
             a2[i] = a * a;
-            m2[i] = mdl.q.mu[i] * a2[i];
         }
     }
 
@@ -224,11 +225,12 @@ struct AdjointF64 {
                 eb = 0.0;
 #pragma unroll
                 for (int i = 0; i < I; ++i) {
-                    const double re = r[i] * eps;
-                    eb = fma(-re, a2[i], fma(r[i], m2[i], eb));
+                    const double z = eps - q.mu[i];
+                    const double rz = r[i] * z;
+                    eb = fma(-rz, a2[i], eb);
                     s0[i] += r[i];
-                    s1[i] += re;
-                    s2[i] = fma(re, eps, s2[i]);
+                    s1[i] += rz;
+                    s2[i] = fma(rz, z, s2[i]);
                 }
             }
 #pragma unroll
@@ -296,23 +298,23 @@ struct AdjointF64 {
                     gn[i] += gs[i];
                     gs[i] = 0.0;
                 }
+            }
+            if constexpr (I >= 2) {
 #pragma unroll
                 for (int i = 0; i < I; ++i) {
                     gn[NS + i] += s0[i];
                     gn[NS + I + i] += s1[i];
-                    gn[NS + 2 * I + i] += s2[i];
+                    gn[NS + 2 * I + i] += fma(-a2[i], s2[i], s0[i]);
                     s0[i] = s1[i] = s2[i] = 0.0;
                 }
             }
         }
-        // sum r_i, sum r_i eps, sum r_i eps^2 -> d log p_i, d mu_i, d a_i
+        // sum r_i, sum r_i z, sum r_i (1 - a^2 z^2) -> d log p_i, d mu_i, d a_i
         if constexpr (I >= 2) {
 #pragma unroll
             for (int i = 0; i < I; ++i) {
-                const double r0 = gn[NS + i], r1 = gn[NS + I + i], r2 = gn[NS + 2 * I + i];
-                const double a = 1.0 / q.sig[i], mu = q.mu[i];
-                gn[NS + I + i] = a * a * (r1 - mu * r0);
-                gn[NS + 2 * I + i] = q.sig[i] * r0 - a * (r2 - mu * (2.0 * r1 - mu * r0));
+                gn[NS + I + i] *= a2[i];
+                gn[NS + 2 * I + i] *= q.sig[i];
             }
         }
     }
@@ -328,12 +330,13 @@ struct AdjointF64 {
 // densities.  Backward, at step j: warp 0 recomputes segment n-1-j and runs the
 // carry over segment n+1-j, warp 1 forms dl/deps and the component sums of
 // segment n-j.  V_k is kept in units of 2^-55 and its sums scaled once at the
-// end; sums of eps^2 are in eps's own units, so they overflow where FP64's do.
+// end; sums of z^2 are in eps's own units, so they overflow where FP64's do.
 // Measured at T=600, up to one block (of 32 particles) per SM, one warp ->
 // two: K=1,I=2 1,298 -> 703 us, K=2,I=2 1,441 -> 823 us, K=3,I=4 2,604 ->
 // 1,347 us, K=4,I=4 2,884 -> 1,364 us; with all the blocks an SM's shared
-// memory holds 1,358 -> 822, 1,495 -> 976, 2,723 -> 1,645 us.  Beyond that a
-// second wave would take what the split gains (k_loglik_grad then).
+// memory holds 1,358 -> 822, 1,495 -> 976, 2,723 -> 1,645 us.  (With weights and
+// shocks of all bits the two warps take 688, 773, 1,360 and 1,370 us.)  Beyond that
+// a second wave would take what the split gains (k_loglik_grad then).
 template <int K, int I>
 struct GradSplit {
     static constexpr int kSeg = mala_seg<double>(), W = K + 2;   // (the caller's checkpoint block is sized from it)
@@ -618,12 +621,11 @@ struct GradSplit {
         }
         // backward: dl/deps and the component sums
         fx.natural_shocks();
-        double a2[I], m2[I], s0[I], s1[I], s2[I], g[3 * I];
+        double a2[I], s0[I], s1[I], s2[I], g[3 * I];
 #pragma unroll
         for (int i = 0; i < I; ++i) {
             const double ai = 1.0 / q.sig[i];
             a2[i] = ai * ai;
-            m2[i] = q.mu[i] * (ai * ai);
             s0[i] = s1[i] = s2[i] = 0.0;
             g[i] = g[I + i] = g[2 * I + i] = 0.0;
         }
@@ -641,33 +643,30 @@ struct GradSplit {
                     double d = 0.0;
 #pragma unroll
                     for (int i = 0; i < I; ++i) {
-                        const double re = ri[i] * es;
-                        d = fma(-re, a2[i], fma(ri[i], m2[i], d));
+                        const double z = es - q.mu[i];
+                        const double rz = ri[i] * z;
+                        d = fma(-rz, a2[i], d);
                         s0[i] += ri[i];
-                        s1[i] += re;
-                        s2[i] = fma(re, es, s2[i]);
+                        s1[i] += rz;
+                        s2[i] = fma(rz, z, s2[i]);
                     }
                     dl[r * 32] = d;
                 }
-                if ((sg & 7) == 0) {
 #pragma unroll
-                    for (int i = 0; i < I; ++i) {
-                        g[i] += s0[i];
-                        g[I + i] += s1[i];
-                        g[2 * I + i] += s2[i];
-                        s0[i] = s1[i] = s2[i] = 0.0;
-                    }
+                for (int i = 0; i < I; ++i) {
+                    g[i] += s0[i];
+                    g[I + i] += s1[i];
+                    g[2 * I + i] += fma(-a2[i], s2[i], s0[i]);
+                    s0[i] = s1[i] = s2[i] = 0.0;
                 }
             }
             meet();
         }
 #pragma unroll
         for (int i = 0; i < I; ++i) {
-            const double r0 = g[i], r1 = g[I + i], r2 = g[2 * I + i];
-            const double ai = 1.0 / q.sig[i], mu = q.mu[i];
-            sm.comb[i][lane] = r0;
-            sm.comb[I + i][lane] = ai * ai * (r1 - mu * r0);
-            sm.comb[2 * I + i][lane] = q.sig[i] * r0 - ai * (r2 - mu * (2.0 * r1 - mu * r0));
+            sm.comb[i][lane] = g[i];
+            sm.comb[I + i][lane] = a2[i] * g[I + i];
+            sm.comb[2 * I + i][lane] = q.sig[i] * g[2 * I + i];
         }
         sm.comb[3 * I][lane] = lm;
         meet();                            // warp 0 takes them
