@@ -9,9 +9,12 @@
 //   - the component weights r_i come from integer exponentials and an integer
 //     reciprocal of their sum, assembled as FP64 numbers by integer instructions;
 //   - the sums over t keep r_i, r_i z and r_i z^2 per component, z = eps - mu_i
-//     (about mu_i, and taken together every segment, so that no two large sums
-//     are left to cancel at the end), from which d log p_i, d mu_i and d a_i follow once at the end
-//     (4 FP64 instructions per component and observation instead of 11).
+//     (about mu_i, and combined every segment, so that no two large sums are
+//     left to cancel at the end: the gradient's rms error at K = 1, I = 2, T = 150 is
+//     0.96e-15 of its largest entry, 1.39e-15 with sums over the series,
+//     0.98e-15 with FP64 throughout), from which d log p_i, d mu_i and d a_i
+//     follow at the end (5 FP64 instructions per component and observation
+//     instead of 11).
 // About 40 FP64 instructions per particle and observation at K = 2, I = 2
 // against 230 with FP64 exponentials and division.
 // Measured (value and gradient, K = 2, I = 2, 2,049 particles x 1,037
